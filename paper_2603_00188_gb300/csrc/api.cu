@@ -396,16 +396,29 @@ cudaError_t run_score(const Ctx& c, const LayerPtrs& io, Strided<float> a_base) 
   Strided<float2> rp = c.view<float2>(c.plan.rowpart);
   const int ns = score_nsplit(c.p);
   if (use_tensor_cores(c.p)) return launch_score_umma(c.p, io, rp, ns, a_base, c.err, c.st);
-  return launch_score(c.p, io, rp, ns, a_base, c.err, c.st);
+  return launch_score(c.p, io, rp, ns, a_base, c.st);
+}
+
+// TSG's slices of partial row maxima and their count: in rho_part, or, for
+// the fp32 pass, in the dots (up to four slices; only the tensor-core CSS has
+// dots of its own).
+static_assert(kTsgSimtSlices <= 4, "the fp32 slices fit the four arrays of dots");
+size_t rho_slices(const Ctx& c, int* count) {
+  if (use_tensor_cores(c.p)) {
+    *count = c.plan.nchunk;
+    return c.plan.rho_part;
+  }
+  *count = tsg_simt_slices(c.p, c.ft);
+  return c.plan.dots;
 }
 
 cudaError_t run_tsg(const Ctx& c, const LayerPtrs& io, int metric) {
-  Strided<const float> rn = c.view<const float>(c.plan.rn);
-  Strided<float> rp = c.view<float>(c.plan.rho_part);
+  int slices;
+  Strided<float> rp = c.view<float>(rho_slices(c, &slices));
   if (use_tensor_cores(c.p))
     return launch_tsg_umma(c.p, c.ft, io, c.view<const float>(c.plan.rn_cur), c.plan.cur_pad, rp, metric, c.err,
                            c.st);
-  return launch_tsg(c.p, c.ft, io, rn, rp, metric, c.err, c.st);
+  return launch_tsg(c.p, c.ft, io, c.view<const float>(c.plan.rn), rp, metric, c.st);
 }
 
 // The ablation fields of the parameters, for the selection kernel.
@@ -462,12 +475,11 @@ stlite_status compress_batch(const Ctx& c, const stlite_params* params, const La
   SelectArgs a = {};
   a.mode = (tsg ? kSelGate : 0) | kSelTopk;
   for (int l = 0; l < c.p.L; ++l) a.budget[l] = io.budget[l];
-  a.nchunk = c.plan.nchunk;
+  a.rho_part = c.view<const float>(rho_slices(c, &a.nchunk));
   a.tsg_enable = tsg ? 1 : 0;
   a.css_enable = params->css_enable ? 1 : 0;
   a.alpha = params->alpha;
   select_variants(a, params, c.p);
-  a.rho_part = c.view<const float>(c.plan.rho_part);
   a.rn = c.view<const float>(c.plan.rn);
   a.rho = c.view<float>(c.plan.rho);
   a.tau = c.view<float>(c.plan.tau);
@@ -534,9 +546,8 @@ stlite_status stlite_gate_frames(const stlite_shape* shape, const stlite_frames*
   SelectArgs a = {};
   a.mode = kSelGate;
   a.budget[0] = budget;
-  a.nchunk = c.plan.nchunk;
+  a.rho_part = c.view<const float>(rho_slices(c, &a.nchunk));
   a.tsg_enable = 1;
-  a.rho_part = c.view<const float>(c.plan.rho_part);
   a.rn = c.view<const float>(c.plan.rn);
   a.rho = one(rho);
   a.tau = one(tau);

@@ -75,7 +75,7 @@ struct WsPlan {
   size_t tau;        // float [Hkv]
   size_t gate;       // uint8 [Hkv][N]
   size_t score;      // float [Hkv][N]
-  size_t dots;       // float [4][Hkv][N]: E, S, SE, SW neighbour dots (tensor-core CSS)
+  size_t dots;       // float [4][Hkv][N]: E, S, SE, SW neighbour dots (tensor-core CSS); TSG slices (fp32)
   size_t total;      // bytes of one layer's region
   int nsplit;        // largest key-split count of the row-statistics pass
   int nchunk;        // 256-column slices of rho_part
@@ -110,7 +110,7 @@ cudaError_t launch_inv_norms(const Problem& p, const FrameTable& ft, const Layer
 // Window score (Eq. 2): row statistics then column sums.  rowpart holds, per
 // layer, [Hkv][nsplit][R] float2 followed by [Hkv][R] float (row bias).
 cudaError_t launch_score(const Problem& p, const LayerPtrs& io, Strided<float2> rowpart, int nsplit,
-                         Strided<float> a_base, uint32_t* err, cudaStream_t st);
+                         Strided<float> a_base, cudaStream_t st);
 cudaError_t launch_score_umma(const Problem& p, const LayerPtrs& io, Strided<float2> rowpart,
                               int nsplit, Strided<float> a_base, uint32_t* err, cudaStream_t st);
 // Key splits of window-score pass 1 (the partials it writes per query row);
@@ -128,9 +128,11 @@ void launch_row_bias(const Problem& p, int nsplit, Strided<float2> rowpart, cuda
 // metric: kTsgCosine / kTsgDot / kTsgNegL2.  The slices hold max_j of
 // k_i.k_j * rn_j (cosine), k_i.k_j (dot) or 2 k_i.k_j - |k_j|^2 (negative L2);
 // the selection kernel finishes rho with the row's own term.
+// The fp32 pass writes tsg_simt_slices(p, ft) slices of its own widths.
+constexpr int kTsgSimtSlices = 4;
+int tsg_simt_slices(const Problem& p, const FrameTable& ft);
 cudaError_t launch_tsg(const Problem& p, const FrameTable& ft, const LayerPtrs& io,
-                       Strided<const float> rn, Strided<float> rho_part, int metric, uint32_t* err,
-                       cudaStream_t st);
+                       Strided<const float> rn, Strided<float> rho_part, int metric, cudaStream_t st);
 cudaError_t launch_tsg_umma(const Problem& p, const FrameTable& ft, const LayerPtrs& io,
                             Strided<const float> rn_cur, int cur_pad, Strided<float> rho_part, int metric,
                             uint32_t* err, cudaStream_t st);

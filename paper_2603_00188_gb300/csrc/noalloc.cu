@@ -106,6 +106,6 @@ extern "C" stlite_status stlite_score_noalloc(const stlite_shape* s, const void*
   const Strided<float2> parts = strided(rowpart, 0);
   const Strided<float> out = strided(a_base, 0);
   cudaError_t e = p.dtype == kBF16 ? launch_score_umma(p, io, parts, nsplit, out, err, st)
-                                   : launch_score(p, io, parts, nsplit, out, err, st);
+                                   : launch_score(p, io, parts, nsplit, out, st);
   return e == cudaSuccess ? STLITE_OK : STLITE_ECUDA;
 }

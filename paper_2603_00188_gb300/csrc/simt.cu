@@ -443,66 +443,185 @@ cudaError_t launch_fill_text_nan(const Problem& p, const FrameTable& ft, float* 
   return cudaGetLastError();
 }
 
+// ------------------------------------------------ fp32 tile products
+// The fp32 passes below are products of two sets of 128-wide rows, bound by
+// the FMA pipe.  A CTA of 128 threads forms the 64 x 64 dot products of two
+// row sets in shared memory (rows padded to 132 floats, so that a warp's four
+// rows of A or eight of B lie in different banks), eight x four per thread:
+// per four dimensions, twelve 16-byte shared loads feed 64 packed
+// multiply-adds.  67.6 KB let three CTAs share an SM; one's copies hide behind
+// the others' products.  Even and odd dimensions accumulate apart (the two
+// halves of fma.rn.f32x2), each in ascending order, and are added last.
+// The product alone reaches 50 TFLOP/s of the FMA pipe's 76 (8 x 8 per thread:
+// 52, but two CTAs of half the warps; 4 x 8: 48; unpacked fmaf: the same).
+// One layer of 5 frames of 36 x 64 (11,840 keys, 4 heads of 224 query rows),
+// against one dot product per thread with both operands read from shared
+// memory for every multiply-add: TSG 2,036 -> 483 us (45 TFLOP/s), row
+// statistics 389 -> 94, column sums 466 -> 89; 1,152 keys: 201 -> 15, 90 -> 18
+// and 195 -> 29.
+constexpr int kTileRows = 64;
+constexpr int kTileThreads = 128;
+constexpr int kTilePitch = kD + 4;  // floats
+constexpr int kTileFloats = kTileRows * kTilePitch;
+constexpr int kTA = 8, kTB = 4;  // rows of A and B per thread
+constexpr int kTilesPerSm = 3;
+
+// The thread's rows: ty + 8 i of A, tx + 16 j of B.  A warp holds four ty
+// and eight tx; warps 2 and 3 have the other four ty, odd warps the other tx.
+__device__ __forceinline__ int tile_ty() { return ((threadIdx.x >> 3) & 3) + 4 * (threadIdx.x >> 6); }
+__device__ __forceinline__ int tile_tx() { return (threadIdx.x & 7) + 8 * ((threadIdx.x >> 5) & 1); }
+
+// Starts the copy of rows src(0) .. src(nrows - 1) (512 bytes each) into a
+// tile; the rows after them become zero.  A warp copies one row at a time.
+template <class Src>
+__device__ __forceinline__ void tile_load(float* dst, int nrows, Src src) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll 4
+  for (int r = threadIdx.x >> 5; r < kTileRows; r += kTileThreads / 32) {
+    float* d = dst + r * kTilePitch + 4 * lane;
+    if (r < nrows) {
+      const uint32_t da = static_cast<uint32_t>(__cvta_generic_to_shared(d));
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(da), "l"(src(r) + 4 * lane) : "memory");
+    } else {
+      *reinterpret_cast<float4*>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+}
+// Every copy of the CTA has landed (and every thread's use of the tiles
+// before this call is over).
+__device__ __forceinline__ void tile_ready() {
+  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+}
+
+// d[i][j] = A row (ty + 8 i) . B row (tx + 16 j)
+__device__ __forceinline__ void tile_dots(const float* a, const float* b, float (&d)[kTA][kTB]) {
+  const float* ap = a + tile_ty() * kTilePitch;
+  const float* bp = b + tile_tx() * kTilePitch;
+  unsigned long long acc[kTA][kTB];
+#pragma unroll
+  for (int i = 0; i < kTA; ++i)
+#pragma unroll
+    for (int j = 0; j < kTB; ++j) acc[i][j] = 0ull;
+#pragma unroll 4
+  for (int k = 0; k < kD; k += 4) {
+    ulonglong2 y[kTB];
+#pragma unroll
+    for (int j = 0; j < kTB; ++j) y[j] = *reinterpret_cast<const ulonglong2*>(bp + 16 * j * kTilePitch + k);
+#pragma unroll
+    for (int i = 0; i < kTA; ++i) {
+      const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(ap + 8 * i * kTilePitch + k);
+#pragma unroll
+      for (int j = 0; j < kTB; ++j) {
+        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][j]) : "l"(x.x), "l"(y[j].x));
+        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][j]) : "l"(x.y), "l"(y[j].y));
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < kTA; ++i)
+#pragma unroll
+    for (int j = 0; j < kTB; ++j) {
+      float lo, hi;
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[i][j]));
+      d[i][j] = lo + hi;
+    }
+}
+
 // ------------------------------------------------------- row statistics
 // Window score, first pass (fp32): for every query row r of KV head h (r =
-// window row * G + group member) the running maximum m and sum l of
-// 2^(x - m), x = q.k * log2(e)/sqrt(d), over the keys of one split.
-// grid = (split, layer*Hkv + head, row chunk).
-constexpr int kRsRows = 256;   // query rows per block
-constexpr int kRsKeys = 64;    // keys per smem tile
-constexpr int kRsSmem = (kRsRows * (kD + 1) + kRsKeys * kD) * 4;
+// window row * G + group member) the maximum m and sum l of 2^(x - m), x =
+// q.k * log2(e)/sqrt(d), over the keys of one split (whole 64-key tiles, so
+// that the last splits may be empty).  A thread keeps its eight rows' states
+// over the keys it sees; the sixteen threads of a row merge theirs at the
+// end.  grid = (split, layer*Hkv + head, 64 query rows).
+constexpr int kScoreSimtSmem = 2 * kTileFloats * 4;
 
-template <typename T>
-__global__ void __launch_bounds__(kRsRows) k_rowstats_simt(const __grid_constant__ LayerPtrs io, Problem p,
-                                                           int nsplit, Strided<float2> part_all) {
-  extern __shared__ float sm[];
-  float* qs = sm;                       // [kRsRows][kD+1]
-  float* ks = sm + kRsRows * (kD + 1);  // [kRsKeys][kD]
-  const int s = blockIdx.x, l = blockIdx.y / p.hkv, h = blockIdx.y % p.hkv, r0 = blockIdx.z * kRsRows;
-  const T* q = static_cast<const T*>(io.q[l]);
-  const T* k = static_cast<const T*>(io.k[l]);
+// Query row r of KV head h.
+__device__ __forceinline__ const float* q_row(const float* q, const Problem& p, int h, int r) {
+  const int G = p.G(), wr = r / G;
+  return q + ((size_t)wr * p.hq + h * G + (r - wr * G)) * kD;
+}
+
+// (m, l) <- the states (m, l) and (m2, l2) together; l = 0: an empty state.
+__device__ __forceinline__ void merge_state(float& m, float& l, float m2, float l2) {
+  if (l2 == 0.f) return;
+  if (l == 0.f) {
+    m = m2;
+    l = l2;
+    return;
+  }
+  const float mn = fmaxf(m, m2);
+  l = (m == mn ? l : l * exp2f(m - mn)) + (m2 == mn ? l2 : l2 * exp2f(m2 - mn));
+  m = mn;
+}
+
+__global__ void __launch_bounds__(kTileThreads, kTilesPerSm)
+    k_rowstats_simt(const __grid_constant__ LayerPtrs io, Problem p, int nsplit, Strided<float2> part_all) {
+  extern __shared__ float4 tile_smem[];
+  float* qs = reinterpret_cast<float*>(tile_smem);
+  float* ks = qs + kTileFloats;
+  const int s = blockIdx.x, l = blockIdx.y / p.hkv, h = blockIdx.y % p.hkv, r0 = blockIdx.z * kTileRows;
+  const float* q = static_cast<const float*>(io.q[l]);
+  const float* k = static_cast<const float*>(io.k[l]);
   float2* part = part_all.at(l);
-  const int G = p.G(), R = p.R(), tid = threadIdx.x;
+  const int R = p.R(), ty = tile_ty(), tx = tile_tx();
   const float c = kLog2e * rsqrtf((float)kD);
-  for (int e = tid; e < kRsRows * kD; e += blockDim.x) {
-    int row = e / kD, t = e - row * kD, gr = r0 + row;
-    float x = 0.f;
-    if (gr < R) {
-      int wr = gr / G, g = gr - wr * G;
-      x = Elem<T>::load1(q + ((size_t)wr * p.hq + h * G + g) * kD + t);
-    }
-    qs[row * (kD + 1) + t] = x;
+  const int per = ((p.n + nsplit - 1) / nsplit + kTileRows - 1) / kTileRows * kTileRows;
+  const int j0 = min(p.n, s * per), j1 = min(p.n, j0 + per);
+  tile_load(qs, min(kTileRows, R - r0), [&](int r) { return q_row(q, p, h, r0 + r); });
+  float m[kTA], ls[kTA];
+#pragma unroll
+  for (int i = 0; i < kTA; ++i) {
+    m[i] = -CUDART_INF_F;
+    ls[i] = 0.f;
   }
-  int per = (p.n + nsplit - 1) / nsplit;
-  int j0 = s * per, j1 = min(p.n, j0 + per);
-  float m = -CUDART_INF_F, lsum = 0.f;
-  for (int jt = j0; jt < j1; jt += kRsKeys) {
-    __syncthreads();
-    for (int e = tid; e < kRsKeys * kD; e += blockDim.x) {
-      int jj = e / kD, t = e - jj * kD;
-      ks[e] = (jt + jj < j1) ? Elem<T>::load1(k + ((size_t)(jt + jj) * p.hkv + h) * kD + t) : 0.f;
-    }
-    __syncthreads();
-    int nk = min(kRsKeys, j1 - jt);
-    const float* qr = qs + tid * (kD + 1);
-    for (int jj = 0; jj < nk; ++jj) {
-      const float* kr = ks + jj * kD;
-      float d0 = 0.f, d1 = 0.f;
-#pragma unroll 16
-      for (int t = 0; t < kD; t += 2) {
-        d0 = fmaf(qr[t], kr[t], d0);
-        d1 = fmaf(qr[t + 1], kr[t + 1], d1);
+  for (int jt = j0; jt < j1; jt += kTileRows) {
+    const int nk = min(kTileRows, j1 - jt);
+    tile_load(ks, nk, [&](int r) { return k + ((size_t)(jt + r) * p.hkv + h) * kD; });
+    tile_ready();
+    float d[kTA][kTB];
+    tile_dots(qs, ks, d);
+#pragma unroll
+    for (int i = 0; i < kTA; ++i) {
+      float mn = m[i];
+#pragma unroll
+      for (int j = 0; j < kTB; ++j) {
+        d[i][j] = tx + 16 * j < nk ? d[i][j] * c : -CUDART_INF_F;
+        mn = fmaxf(mn, d[i][j]);
       }
-      float x = (d0 + d1) * c;
-      if (x > m) {
-        lsum = lsum * exp2f(m - x) + 1.0f;
-        m = x;
-      } else {
-        lsum += exp2f(x - m);
+      if (mn != -CUDART_INF_F) {  // no key yet otherwise
+        float sum = 0.f;
+#pragma unroll
+        for (int j = 0; j < kTB; ++j) sum += d[i][j] == mn ? 1.f : exp2f(d[i][j] - mn);
+        ls[i] = (m[i] == mn ? ls[i] : ls[i] * exp2f(m[i] - mn)) + sum;
+        m[i] = mn;
       }
     }
+    __syncthreads();  // the key tile is rewritten
   }
-  if (r0 + tid < R) part[((size_t)h * nsplit + s) * R + r0 + tid] = make_float2(m, lsum);
+  // a row's states: eight lanes of each of two warps
+#pragma unroll
+  for (int i = 0; i < kTA; ++i)
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+      const float m2 = __shfl_xor_sync(0xffffffffu, m[i], o), l2 = __shfl_xor_sync(0xffffffffu, ls[i], o);
+      merge_state(m[i], ls[i], m2, l2);
+    }
+  tile_ready();  // also when the split was empty: the query rows' copies end before the CTA does
+  float2* xch = reinterpret_cast<float2*>(ks);
+  if (tx == 8)
+#pragma unroll
+    for (int i = 0; i < kTA; ++i) xch[ty + 8 * i] = make_float2(m[i], ls[i]);
+  __syncthreads();
+  if (tx == 0)
+#pragma unroll
+    for (int i = 0; i < kTA; ++i) {
+      const float2 o = xch[ty + 8 * i];
+      merge_state(m[i], ls[i], o.x, o.y);
+      const int row = r0 + ty + 8 * i;
+      if (row < R) part[((size_t)h * nsplit + s) * R + row] = make_float2(m[i], ls[i]);
+    }
 }
 
 // Merge the splits: bias[h][r] = -m_r - log2(G * l_r), so that
@@ -563,172 +682,186 @@ void launch_row_bias(const Problem& p, int nsplit, Strided<float2> rowpart, cuda
 }
 
 // ---------------------------------------------------------- column sums
-// Window score, second pass (fp32): a[h][j] = sum_r 2^(x_rj + bias_r).  One
-// thread per key; the key tile is kept (padded) in shared memory.
+// Window score, second pass (fp32): a[h][j] = sum_r 2^(x_rj + bias_r).  The
+// key tile stays, the query rows stream; a thread sums its eight keys over
+// the rows it sees, the sixteen threads of a key add theirs at the end.
 // grid = (key tile, layer*Hkv + head).
-constexpr int kCsKeys = 128;
-constexpr int kCsRows = 32;
-constexpr int kCsMaxR = 1024;
-constexpr int kCsSmem = (kCsKeys * (kD + 1) + kCsRows * kD + kCsMaxR) * 4;
-
-template <typename T>
-__global__ void __launch_bounds__(kCsKeys) k_colsum_simt(const __grid_constant__ LayerPtrs io, Problem p,
-                                                         int nsplit, Strided<float2> part_all,
-                                                         Strided<float> a_all) {
-  extern __shared__ float sm[];
-  float* ks = sm;                            // [kCsKeys][kD+1]
-  float* qs = ks + kCsKeys * (kD + 1);       // [kCsRows][kD]
-  float* bs = qs + kCsRows * kD;             // [R]
-  const int l = blockIdx.y / p.hkv, h = blockIdx.y % p.hkv, j0 = blockIdx.x * kCsKeys, tid = threadIdx.x;
-  const T* q = static_cast<const T*>(io.q[l]);
-  const T* k = static_cast<const T*>(io.k[l]);
-  const float* bias = reinterpret_cast<const float*>(part_all.at(l) + (size_t)p.hkv * nsplit * p.R());
-  float* a_base = a_all.at(l);
-  const int G = p.G(), R = p.R();
+__global__ void __launch_bounds__(kTileThreads, kTilesPerSm)
+    k_colsum_simt(const __grid_constant__ LayerPtrs io, Problem p, int nsplit, Strided<float2> part_all,
+                  Strided<float> a_all) {
+  extern __shared__ float4 tile_smem[];
+  float* ks = reinterpret_cast<float*>(tile_smem);
+  float* qs = ks + kTileFloats;
+  const int l = blockIdx.y / p.hkv, h = blockIdx.y % p.hkv, j0 = blockIdx.x * kTileRows;
+  const float* q = static_cast<const float*>(io.q[l]);
+  const float* k = static_cast<const float*>(io.k[l]);
+  const int R = p.R(), ty = tile_ty(), tx = tile_tx();
+  const float* bias = reinterpret_cast<const float*>(part_all.at(l) + (size_t)p.hkv * nsplit * R) + (size_t)h * R;
   const float c = kLog2e * rsqrtf((float)kD);
-  for (int e = tid; e < kCsKeys * kD; e += blockDim.x) {
-    int jj = e / kD, t = e - jj * kD;
-    ks[jj * (kD + 1) + t] =
-        (j0 + jj < p.n) ? Elem<T>::load1(k + ((size_t)(j0 + jj) * p.hkv + h) * kD + t) : 0.f;
-  }
-  for (int r = tid; r < R; r += blockDim.x) bs[r] = bias[(size_t)h * R + r];
-  float acc = 0.f;
-  const float* kr = ks + tid * (kD + 1);
-  for (int rt = 0; rt < R; rt += kCsRows) {
-    __syncthreads();
-    for (int e = tid; e < kCsRows * kD; e += blockDim.x) {
-      int row = e / kD, t = e - row * kD, gr = rt + row;
-      float x = 0.f;
-      if (gr < R) {
-        int wr = gr / G, g = gr - wr * G;
-        x = Elem<T>::load1(q + ((size_t)wr * p.hq + h * G + g) * kD + t);
-      }
-      qs[e] = x;
+  tile_load(ks, min(kTileRows, p.n - j0), [&](int r) { return k + ((size_t)(j0 + r) * p.hkv + h) * kD; });
+  float acc[kTA];
+#pragma unroll
+  for (int i = 0; i < kTA; ++i) acc[i] = 0.f;
+  for (int rt = 0; rt < R; rt += kTileRows) {
+    const int nr = min(kTileRows, R - rt);
+    tile_load(qs, nr, [&](int r) { return q_row(q, p, h, rt + r); });
+    float bs[kTB];
+#pragma unroll
+    for (int j = 0; j < kTB; ++j) bs[j] = tx + 16 * j < nr ? __ldg(bias + rt + tx + 16 * j) : 0.f;
+    tile_ready();
+    float d[kTA][kTB];
+    tile_dots(ks, qs, d);
+#pragma unroll
+    for (int i = 0; i < kTA; ++i) {
+      float sum = 0.f;
+#pragma unroll
+      for (int j = 0; j < kTB; ++j) sum += tx + 16 * j < nr ? exp2f(fmaf(d[i][j], c, bs[j])) : 0.f;
+      acc[i] += sum;
     }
-    __syncthreads();
-    int nr = min(kCsRows, R - rt);
-    for (int row = 0; row < nr; ++row) {
-      const float* qr = qs + row * kD;
-      float d0 = 0.f, d1 = 0.f;
-#pragma unroll 16
-      for (int t = 0; t < kD; t += 2) {
-        d0 = fmaf(kr[t], qr[t], d0);
-        d1 = fmaf(kr[t + 1], qr[t + 1], d1);
-      }
-      acc += exp2f(fmaf(d0 + d1, c, bs[rt + row]));
-    }
+    __syncthreads();  // the query tile is rewritten
   }
-  if (j0 + tid < p.n) a_base[(size_t)h * p.n + j0 + tid] = acc;
+#pragma unroll
+  for (int i = 0; i < kTA; ++i)
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+  if (tx == 8)
+#pragma unroll
+    for (int i = 0; i < kTA; ++i) qs[ty + 8 * i] = acc[i];
+  __syncthreads();
+  if (tx == 0)
+#pragma unroll
+    for (int i = 0; i < kTA; ++i) {
+      const int j = j0 + ty + 8 * i;
+      if (j < p.n) a_all.at(l)[(size_t)h * p.n + j] = acc[i] + qs[ty + 8 * i];
+    }
 }
 
 cudaError_t launch_score(const Problem& p, const LayerPtrs& io, Strided<float2> rowpart, int nsplit,
-                         Strided<float> a_base, uint32_t* err, cudaStream_t st) {
-  (void)err;
-  if (p.R() > kCsMaxR) return cudaErrorNotSupported;
-  cudaFuncSetAttribute(k_rowstats_simt<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsSmem);
-  cudaFuncSetAttribute(k_rowstats_simt<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsSmem);
-  cudaFuncSetAttribute(k_colsum_simt<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCsSmem);
-  cudaFuncSetAttribute(k_colsum_simt<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCsSmem);
-  dim3 g1(nsplit, p.L * p.hkv, (p.R() + kRsRows - 1) / kRsRows);
-  dim3 g2((p.n + kCsKeys - 1) / kCsKeys, p.L * p.hkv);
+                         Strided<float> a_base, cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(k_rowstats_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, kScoreSimtSmem);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_colsum_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, kScoreSimtSmem);
+  if (e != cudaSuccess) return e;
+  dim3 g1(nsplit, p.L * p.hkv, (p.R() + kTileRows - 1) / kTileRows);
+  dim3 g2((p.n + kTileRows - 1) / kTileRows, p.L * p.hkv);
   {
     TimingScope ts("rowstats_simt", st);
-    if (p.dtype == kBF16)
-      k_rowstats_simt<__nv_bfloat16><<<g1, kRsRows, kRsSmem, st>>>(io, p, nsplit, rowpart);
-    else
-      k_rowstats_simt<float><<<g1, kRsRows, kRsSmem, st>>>(io, p, nsplit, rowpart);
+    k_rowstats_simt<<<g1, kTileThreads, kScoreSimtSmem, st>>>(io, p, nsplit, rowpart);
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   {
     TimingScope ts("row_bias", st);
     launch_row_bias(p, nsplit, rowpart, st);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   TimingScope ts("colsum_simt", st);
-  if (p.dtype == kBF16)
-    k_colsum_simt<__nv_bfloat16><<<g2, kCsKeys, kCsSmem, st>>>(io, p, nsplit, rowpart, a_base);
-  else
-    k_colsum_simt<float><<<g2, kCsKeys, kCsSmem, st>>>(io, p, nsplit, rowpart, a_base);
+  k_colsum_simt<<<g2, kTileThreads, kScoreSimtSmem, st>>>(io, p, nsplit, rowpart, a_base);
   return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ TSG
-// fp32 path of Eq. 6: one thread per historical token, current-frame keys
-// streamed through shared memory.  Writes slice 0 of rho_part (the fp32 path
-// has a single slice).  grid = (row tile, layer*Hkv + head).
-constexpr int kTsKeys = 64;
-constexpr int kTsSmem = (kTsgTile * (kD + 1) + kTsKeys * kD + 2 * kTsKeys) * 4;
+// fp32 path of Eq. 6: a tile of 64 historical tokens against the current
+// frame's keys of one column slice, streamed in tiles of 64.  Writes slice
+// blockIdx.z of rho_part.  grid = (half row tile, layer*Hkv + head, slice).
+constexpr int kTsgSimtSmem = (2 * kTileFloats + 2 * kTileRows) * 4;
 
-template <typename T>
-__global__ void __launch_bounds__(kTsgTile) k_tsg_simt(const __grid_constant__ LayerPtrs io,
-                                                       const __grid_constant__ FrameTable ft, int hkv,
-                                                       Strided<const float> rn_all,
-                                                       Strided<float> rho_all, int metric) {
-  extern __shared__ float sm[];
-  float* hs = sm;                              // [128][kD+1]
-  float* cs = hs + kTsgTile * (kD + 1);        // [kTsKeys][kD]
-  float* cr = cs + kTsKeys * kD;               // [kTsKeys] scale of each current key
-  float* co = cr + kTsKeys;                    // [kTsKeys] offset: value = dot * scale + offset
-  const int t = blockIdx.x, l = blockIdx.y / hkv, h = blockIdx.y % hkv, tid = threadIdx.x;
-  const int n = ft.n_tokens;
-  const T* k = static_cast<const T*>(io.k[l]);
-  const float* rn = rn_all.at(l);
-  float* rho_part = rho_all.at(l);
+__global__ void __launch_bounds__(kTileThreads, kTilesPerSm)
+    k_tsg_simt(const __grid_constant__ LayerPtrs io, const __grid_constant__ FrameTable ft, int hkv,
+               Strided<const float> rn_all, Strided<float> rho_all, int slice_cols, int metric) {
+  extern __shared__ float4 tile_smem[];
+  float* hs = reinterpret_cast<float*>(tile_smem);
+  float* cs = hs + kTileFloats;
+  float* cr = cs + kTileFloats;  // [64] scale of each current key
+  float* co = cr + kTileRows;    // [64] offset: value = dot * scale + offset
+  const int t = blockIdx.x >> 1, l = blockIdx.y / hkv, h = blockIdx.y % hkv, tid = threadIdx.x;
+  const int n = ft.n_tokens, ty = tile_ty(), tx = tile_tx();
+  const float* k = static_cast<const float*>(io.k[l]);
+  const float* rn = rn_all.at(l) + (size_t)h * n + ft.cur_off;
   // tile -> historical frame
   int f = 0;
   while (f + 1 < ft.n_frames - 1 && ft.tile0[f + 1] <= t) ++f;
-  int fend = ft.off[f] + ft.gh[f] * ft.gw[f];
-  int i0 = ft.off[f] + (t - ft.tile0[f]) * kTsgTile;
-  for (int e = tid; e < kTsgTile * kD; e += blockDim.x) {
-    int ii = e / kD, c = e - ii * kD;
-    hs[ii * (kD + 1) + c] = (i0 + ii < fend) ? Elem<T>::load1(k + ((size_t)(i0 + ii) * hkv + h) * kD + c) : 0.f;
-  }
-  float best = -CUDART_INF_F;
-  const float* hr = hs + tid * (kD + 1);
-  for (int jt = 0; jt < ft.cur_len; jt += kTsKeys) {
-    __syncthreads();
-    for (int e = tid; e < kTsKeys * kD; e += blockDim.x) {
-      int jj = e / kD, c = e - jj * kD;
-      int j = ft.cur_off + jt + jj;
-      cs[e] = (jt + jj < ft.cur_len) ? Elem<T>::load1(k + ((size_t)j * hkv + h) * kD + c) : 0.f;
-    }
-    for (int jj = tid; jj < kTsKeys; jj += blockDim.x) {
+  const int fend = ft.off[f] + ft.gh[f] * ft.gw[f];
+  const int i0 = ft.off[f] + (t - ft.tile0[f]) * kTsgTile + (blockIdx.x & 1) * kTileRows;
+  if (i0 >= fend) return;  // the frame's last 128-token tile is at most half full
+  auto key_row = [&](int j) { return k + ((size_t)j * hkv + h) * kD; };
+  tile_load(hs, min(kTileRows, fend - i0), [&](int r) { return key_row(i0 + r); });
+  float best[kTA];
+#pragma unroll
+  for (int i = 0; i < kTA; ++i) best[i] = -CUDART_INF_F;
+  const int jend = min(ft.cur_len, (int)(blockIdx.z + 1) * slice_cols);
+  for (int jt = blockIdx.z * slice_cols; jt < jend; jt += kTileRows) {
+    const int nk = min(kTileRows, jend - jt);
+    tile_load(cs, nk, [&](int r) { return key_row(ft.cur_off + jt + r); });
+    if (tid < kTileRows) {
       // cosine: dot * rn_j; dot: dot; negative L2 (without the row's own
-      // -|k_i|^2): 2 dot - |k_j|^2
-      const float r = (jt + jj < ft.cur_len) ? rn[(size_t)h * n + ft.cur_off + jt + jj] : 0.f;
-      cr[jj] = metric == kTsgCosine ? r : (metric == kTsgDot ? 1.f : 2.f);
-      co[jj] = metric == kTsgNegL2 ? -1.f / (r * r) : 0.f;
+      // -|k_i|^2): 2 dot - |k_j|^2; columns past the slice lose every maximum
+      const float r = tid < nk ? rn[jt + tid] : 0.f;
+      cr[tid] = metric == kTsgCosine ? r : (metric == kTsgDot ? 1.f : 2.f);
+      co[tid] = tid >= nk ? -CUDART_INF_F : (metric == kTsgNegL2 ? -1.f / (r * r) : 0.f);
     }
-    __syncthreads();
-    int nk = min(kTsKeys, ft.cur_len - jt);
-    for (int jj = 0; jj < nk; ++jj) {
-      const float* kr = cs + jj * kD;
-      float d0 = 0.f, d1 = 0.f;
-#pragma unroll 16
-      for (int c = 0; c < kD; c += 2) {
-        d0 = fmaf(hr[c], kr[c], d0);
-        d1 = fmaf(hr[c + 1], kr[c + 1], d1);
-      }
-      best = fmaxf(best, fmaf(d0 + d1, cr[jj], co[jj]));
+    tile_ready();
+    float d[kTA][kTB];
+    tile_dots(hs, cs, d);
+#pragma unroll
+    for (int j = 0; j < kTB; ++j) {
+      const float a = cr[tx + 16 * j], b = co[tx + 16 * j];
+#pragma unroll
+      for (int i = 0; i < kTA; ++i) best[i] = fmaxf(best[i], fmaf(d[i][j], a, b));
+    }
+    __syncthreads();  // the column tile is rewritten
+  }
+#pragma unroll
+  for (int i = 0; i < kTA; ++i)
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) best[i] = fmaxf(best[i], __shfl_xor_sync(0xffffffffu, best[i], o));
+  if (tx == 8)
+#pragma unroll
+    for (int i = 0; i < kTA; ++i) cs[ty + 8 * i] = best[i];
+  __syncthreads();
+  float* rho_part = rho_all.at(l) + ((size_t)blockIdx.z * hkv + h) * n;
+  if (tx == 0)
+#pragma unroll
+    for (int i = 0; i < kTA; ++i) {
+      const int tok = i0 + ty + 8 * i;
+      if (tok < fend) rho_part[tok] = fmaxf(best[i], cs[ty + 8 * i]);
+    }
+}
+
+// Column slices of the fp32 TSG pass (1..kTsgSimtSlices): the count whose
+// CTAs, three to an SM, take the least time in whole waves, a wave costing
+// its column tiles plus about one for the row tile's load.  The slices fold
+// by maximum, so the count changes no result.
+int tsg_simt_slices(const Problem& p, const FrameTable& ft) {
+  if (ft.n_frames < 2) return 1;
+  const long long rows = 2LL * ft.tile0[ft.n_frames - 1] * p.L * p.hkv;
+  const int tiles = (ft.cur_len + kTileRows - 1) / kTileRows;
+  const long long slots = 152 * kTilesPerSm;
+  int best = 1;
+  long long best_cost = 0;
+  for (int s = 1; s <= kTsgSimtSlices; ++s) {
+    const int per = (tiles + s - 1) / s;
+    if (s > 1 && (s - 1) * per >= tiles) break;  // an empty slice
+    const long long cost = ((rows * s + slots - 1) / slots) * (per + 1);
+    if (s == 1 || cost < best_cost) {
+      best = s;
+      best_cost = cost;
     }
   }
-  if (i0 + tid < fend) rho_part[(size_t)h * n + i0 + tid] = best;
+  return best;
 }
 
 cudaError_t launch_tsg(const Problem& p, const FrameTable& ft, const LayerPtrs& io, Strided<const float> rn,
-                       Strided<float> rho_part, int metric, uint32_t* err, cudaStream_t st) {
-  (void)err;
-  cudaFuncSetAttribute(k_tsg_simt<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTsSmem);
-  cudaFuncSetAttribute(k_tsg_simt<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTsSmem);
-  int tiles = ft.n_frames >= 2 ? ft.tile0[ft.n_frames - 1] : 0;
+                       Strided<float> rho_part, int metric, cudaStream_t st) {
+  const int tiles = ft.n_frames >= 2 ? ft.tile0[ft.n_frames - 1] : 0;
   if (tiles == 0) return cudaSuccess;
-  dim3 g(tiles, p.L * p.hkv);
+  cudaError_t e = cudaFuncSetAttribute(k_tsg_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, kTsgSimtSmem);
+  if (e != cudaSuccess) return e;
+  const int slices = tsg_simt_slices(p, ft);
+  const int ctiles = (ft.cur_len + kTileRows - 1) / kTileRows;
+  const int slice_cols = (ctiles + slices - 1) / slices * kTileRows;
   TimingScope ts("tsg_simt", st);
-  if (p.dtype == kBF16)
-    k_tsg_simt<__nv_bfloat16><<<g, kTsgTile, kTsSmem, st>>>(io, ft, p.hkv, rn, rho_part, metric);
-  else
-    k_tsg_simt<float><<<g, kTsgTile, kTsSmem, st>>>(io, ft, p.hkv, rn, rho_part, metric);
+  k_tsg_simt<<<dim3(2 * tiles, p.L * p.hkv, slices), kTileThreads, kTsgSimtSmem, st>>>(io, ft, p.hkv, rn, rho_part,
+                                                                                      slice_cols, metric);
   return cudaGetLastError();
 }
 
