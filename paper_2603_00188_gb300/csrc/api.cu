@@ -139,7 +139,7 @@ WsPlan plan_workspace(const Problem& p, const FrameTable& ft) {
   w.a_base = take(hn * 4);
   w.phi = take(hn * 4);
   w.rho = take(hn * 4);
-  w.rho_part = take((size_t)w.nchunk * hn * 4);
+  w.rho_key = take((size_t)w.nchunk * hn * 4);
   w.tau = take((size_t)p.hkv * 4);
   w.gate = take(hn);
   w.score = take(hn * 4);
@@ -352,6 +352,13 @@ Strided<T> one(T* p) {
   return strided(p, 0);
 }
 
+// Where the inverse norms go; tsg: a TSG pass follows (its row maxima start
+// from zero).
+NormsOut norms_out(const Ctx& c, bool tsg) {
+  return {c.view<float>(c.plan.rn), c.view<float>(c.plan.rn_cur),
+          tsg ? c.view<uint32_t>(c.plan.rho_key) : strided<uint32_t>(nullptr, 0), c.plan.cur_pad};
+}
+
 // CSS (Eqs. 4-5) into phi, plus the inverse key norms rn / rn_cur that TSG
 // uses.  bf16 caches whose grids are at most 127 wide take the tensor-core
 // kernel; otherwise the CUDA-core one.
@@ -359,37 +366,35 @@ Strided<T> one(T* p) {
 // size ablation, on the box-sum kernel).
 // defer_phi: the tensor-core CSS leaves Phi to a later run_css_phi and sets
 // *deferred (the other kernels produce Phi themselves).
-cudaError_t run_css(const Ctx& c, const LayerPtrs& io, Strided<float> phi, int size = 3, bool defer_phi = false,
-                    bool* deferred = nullptr) {
-  Strided<float> rn = c.view<float>(c.plan.rn), rc = c.view<float>(c.plan.rn_cur);
+cudaError_t run_css(const Ctx& c, const LayerPtrs& io, Strided<float> phi, bool tsg, int size = 3,
+                    bool defer_phi = false, bool* deferred = nullptr) {
+  const NormsOut norms = norms_out(c, tsg);
   if (deferred) *deferred = false;
-  if (size > 3) return launch_css_box(c.p, c.ft, io, size, phi, rn, rc, c.plan.cur_pad, c.st);
+  if (size > 3) return launch_css_box(c.p, c.ft, io, size, phi, norms, c.st);
   if (use_tensor_cores(c.p) && css_umma_supported(c.ft)) {
     if (defer_phi && deferred) *deferred = true;
     const size_t hn4 = (size_t)c.p.hkv * c.p.n * 4;
     Strided<float> dE = c.view<float>(c.plan.dots), dS = c.view<float>(c.plan.dots + hn4);
     Strided<float> dSE = c.view<float>(c.plan.dots + 2 * hn4), dSW = c.view<float>(c.plan.dots + 3 * hn4);
-    return launch_css_umma(c.p, c.ft, io, phi, rn, rc, c.plan.cur_pad, dE, dS, dSE, dSW, c.err, c.st,
-                           !(defer_phi && deferred));
+    return launch_css_umma(c.p, c.ft, io, phi, norms, dE, dS, dSE, dSW, c.err, c.st, !(defer_phi && deferred));
   }
-  return launch_css(c.p, c.ft, io, phi, rn, rc, c.plan.cur_pad, c.st);
+  return launch_css(c.p, c.ft, io, phi, norms, c.st);
 }
 
 // Phi of a deferred tensor-core CSS (its dots written), on stream st.
 cudaError_t run_css_phi(const Ctx& c, Strided<float> phi, cudaStream_t st) {
   const size_t hn4 = (size_t)c.p.hkv * c.p.n * 4;
-  return launch_css_phi(c.p, c.ft, phi, c.view<float>(c.plan.rn), c.view<float>(c.plan.rn_cur), c.plan.cur_pad,
-                        c.view<float>(c.plan.dots), c.view<float>(c.plan.dots + hn4),
-                        c.view<float>(c.plan.dots + 2 * hn4), c.view<float>(c.plan.dots + 3 * hn4), st);
+  return launch_css_phi(c.p, c.ft, phi, c.view<const float>(c.plan.rn), c.view<float>(c.plan.dots),
+                        c.view<float>(c.plan.dots + hn4), c.view<float>(c.plan.dots + 2 * hn4),
+                        c.view<float>(c.plan.dots + 3 * hn4), st);
 }
 
-// The inverse norms alone: from the CSS kernel when that is the tensor-core
-// one (so that every path sees the same bits), else from the norms kernel
-// (whose arithmetic matches the CUDA-core CSS kernel's).
+// The inverse norms alone, for TSG: from the CSS kernel when that is the
+// tensor-core one (so that every path sees the same bits), else from the
+// norms kernel (whose arithmetic matches the CUDA-core CSS kernel's).
 cudaError_t run_norms(const Ctx& c, const LayerPtrs& io) {
-  if (use_tensor_cores(c.p) && css_umma_supported(c.ft)) return run_css(c, io, c.view<float>(c.plan.phi));
-  return launch_inv_norms(c.p, c.ft, io, c.view<float>(c.plan.rn), c.view<float>(c.plan.rn_cur), c.plan.cur_pad,
-                          c.st);
+  if (use_tensor_cores(c.p) && css_umma_supported(c.ft)) return run_css(c, io, c.view<float>(c.plan.phi), true);
+  return launch_inv_norms(c.p, c.ft, io, norms_out(c, true), c.st);
 }
 
 cudaError_t run_score(const Ctx& c, const LayerPtrs& io, Strided<float> a_base) {
@@ -399,26 +404,12 @@ cudaError_t run_score(const Ctx& c, const LayerPtrs& io, Strided<float> a_base) 
   return launch_score(c.p, io, rp, ns, a_base, c.st);
 }
 
-// TSG's slices of partial row maxima and their count: in rho_part, or, for
-// the fp32 pass, in the dots (up to four slices; only the tensor-core CSS has
-// dots of its own).
-static_assert(kTsgSimtSlices <= 4, "the fp32 slices fit the four arrays of dots");
-size_t rho_slices(const Ctx& c, int* count) {
-  if (use_tensor_cores(c.p)) {
-    *count = c.plan.nchunk;
-    return c.plan.rho_part;
-  }
-  *count = tsg_simt_slices(c.p, c.ft);
-  return c.plan.dots;
-}
-
 cudaError_t run_tsg(const Ctx& c, const LayerPtrs& io, int metric) {
-  int slices;
-  Strided<float> rp = c.view<float>(rho_slices(c, &slices));
+  Strided<uint32_t> rho_key = c.view<uint32_t>(c.plan.rho_key);
   if (use_tensor_cores(c.p))
-    return launch_tsg_umma(c.p, c.ft, io, c.view<const float>(c.plan.rn_cur), c.plan.cur_pad, rp, metric, c.err,
+    return launch_tsg_umma(c.p, c.ft, io, c.view<const float>(c.plan.rn_cur), c.plan.cur_pad, rho_key, metric, c.err,
                            c.st);
-  return launch_tsg(c.p, c.ft, io, c.view<const float>(c.plan.rn), rp, metric, c.st);
+  return launch_tsg(c.p, c.ft, io, c.view<const float>(c.plan.rn), rho_key, metric, c.st);
 }
 
 // The ablation fields of the parameters, for the selection kernel.
@@ -454,7 +445,7 @@ stlite_status compress_batch(const Ctx& c, const stlite_params* params, const La
   // norms pass provides them.
   bool late_phi = false;
   if (e == cudaSuccess && params->css_enable) {
-    e = run_css(c, io, phi, params->css_size, x != nullptr, &late_phi);
+    e = run_css(c, io, phi, tsg, params->css_size, x != nullptr, &late_phi);
     if (e == cudaSuccess && late_phi) e = cudaEventRecord(x->ev[2], c.st);
   } else if (e == cudaSuccess && tsg) {
     e = run_norms(c, io);
@@ -475,7 +466,7 @@ stlite_status compress_batch(const Ctx& c, const stlite_params* params, const La
   SelectArgs a = {};
   a.mode = (tsg ? kSelGate : 0) | kSelTopk;
   for (int l = 0; l < c.p.L; ++l) a.budget[l] = io.budget[l];
-  a.rho_part = c.view<const float>(rho_slices(c, &a.nchunk));
+  a.rho_key = c.view<const uint32_t>(c.plan.rho_key);
   a.tsg_enable = tsg ? 1 : 0;
   a.css_enable = params->css_enable ? 1 : 0;
   a.alpha = params->alpha;
@@ -546,7 +537,7 @@ stlite_status stlite_gate_frames(const stlite_shape* shape, const stlite_frames*
   SelectArgs a = {};
   a.mode = kSelGate;
   a.budget[0] = budget;
-  a.rho_part = c.view<const float>(rho_slices(c, &a.nchunk));
+  a.rho_key = c.view<const uint32_t>(c.plan.rho_key);
   a.tsg_enable = 1;
   a.rn = c.view<const float>(c.plan.rn);
   a.rho = one(rho);
@@ -564,7 +555,7 @@ stlite_status stlite_spatial_saliency(const stlite_shape* shape, const stlite_fr
   if (s != STLITE_OK) return s;
   if (!k || !phi || !aligned16(k) || !aligned16(phi)) return STLITE_EINVAL;
   const LayerPtrs io = single_layer(nullptr, k, nullptr, nullptr, nullptr, nullptr);
-  cudaError_t e = run_css(c, io, one(phi));
+  cudaError_t e = run_css(c, io, one(phi), false);
   if (e == cudaSuccess) e = launch_fill_text_nan(c.p, c.ft, phi, c.st);
   return cuda_status(e);
 }
@@ -578,8 +569,7 @@ stlite_status stlite_spatial_saliency_size(const stlite_shape* shape, const stli
   if (s != STLITE_OK) return s;
   if (!k || !phi || !aligned16(k) || !aligned16(phi)) return STLITE_EINVAL;
   const LayerPtrs io = single_layer(nullptr, k, nullptr, nullptr, nullptr, nullptr);
-  cudaError_t e = launch_css_box(c.p, c.ft, io, size, one(phi), c.view<float>(c.plan.rn),
-                                 c.view<float>(c.plan.rn_cur), c.plan.cur_pad, c.st);
+  cudaError_t e = launch_css_box(c.p, c.ft, io, size, one(phi), norms_out(c, false), c.st);
   if (e == cudaSuccess) e = launch_fill_text_nan(c.p, c.ft, phi, c.st);
   return cuda_status(e);
 }

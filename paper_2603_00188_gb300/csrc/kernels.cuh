@@ -71,14 +71,14 @@ struct WsPlan {
   size_t a_base;     // float [Hkv][N]
   size_t phi;        // float [Hkv][N]
   size_t rho;        // float [Hkv][N]
-  size_t rho_part;   // float [nchunk][Hkv][N]
+  size_t rho_key;    // uint32 [Hkv][N] TSG row maxima as float_key images (room for nchunk such arrays)
   size_t tau;        // float [Hkv]
   size_t gate;       // uint8 [Hkv][N]
   size_t score;      // float [Hkv][N]
-  size_t dots;       // float [4][Hkv][N]: E, S, SE, SW neighbour dots (tensor-core CSS); TSG slices (fp32)
+  size_t dots;       // float [4][Hkv][N]: E, S, SE, SW neighbour dots (tensor-core CSS)
   size_t total;      // bytes of one layer's region
   int nsplit;        // largest key-split count of the row-statistics pass
-  int nchunk;        // 256-column slices of rho_part
+  int nchunk;        // 256-column chunks of the current frame (bf16)
   int cur_pad;       // current-frame length rounded up to 4
 };
 WsPlan plan_workspace(const Problem& p, const FrameTable& ft);
@@ -101,11 +101,18 @@ class TimingScope {
 };
 
 // ---- launchers ----------------------------------------------------------
-// rn[l][h][j] = 1 / max(|k_l[j,h]|, 1e-8) for every token; the current
-// frame's values are also written to rn_cur[l][h][j - cur_off] (row stride
-// cur_pad).
-cudaError_t launch_inv_norms(const Problem& p, const FrameTable& ft, const LayerPtrs& io, Strided<float> rn,
-                             Strided<float> rn_cur, int cur_pad, cudaStream_t st);
+// What a kernel that forms the inverse key norms writes: rn[l][h][j] = 1 /
+// max(|k_l[j,h]|, 1e-8); the current frame's also to rn_cur[l][h][j -
+// cur_off] (row stride cur_pad); and zero to rho_key (null base: not), for a
+// TSG pass that follows.
+struct NormsOut {
+  Strided<float> rn, rn_cur;
+  Strided<uint32_t> rho_key;
+  int cur_pad;
+};
+// For every token.
+cudaError_t launch_inv_norms(const Problem& p, const FrameTable& ft, const LayerPtrs& io, const NormsOut& norms,
+                             cudaStream_t st);
 
 // Window score (Eq. 2): row statistics then column sums.  rowpart holds, per
 // layer, [Hkv][nsplit][R] float2 followed by [Hkv][R] float (row bias).
@@ -122,47 +129,43 @@ int score_nsplit_max(const Problem& p);
 // follows them in rowpart ([Hkv][R] float per layer).
 void launch_row_bias(const Problem& p, int nsplit, Strided<float2> rowpart, cudaStream_t st);
 
-// TSG partial row maxima: rho_part[l][s][h][i] = max over the current-frame
-// columns of 256-column slice s of k_i.k_j * rn_j, for historical visual
-// tokens i (Eq. 6 before the 1/|k_i| factor).
-// metric: kTsgCosine / kTsgDot / kTsgNegL2.  The slices hold max_j of
-// k_i.k_j * rn_j (cosine), k_i.k_j (dot) or 2 k_i.k_j - |k_j|^2 (negative L2);
-// the selection kernel finishes rho with the row's own term.
-// The fp32 pass writes tsg_simt_slices(p, ft) slices of its own widths.
-constexpr int kTsgSimtSlices = 4;
-int tsg_simt_slices(const Problem& p, const FrameTable& ft);
+// TSG row maxima: rho_key[l][h][i] = max over the current frame's columns j
+// of k_i.k_j * rn_j, for historical visual tokens i (Eq. 6 before the 1/|k_i|
+// factor), as the order-preserving image float_key.  The kernels fold each
+// CTA's columns in with an atomic maximum (exact in any order), so every
+// visual token's entry is zero before: the kernel that writes rn zeroes it.
+// metric: kTsgCosine / kTsgDot / kTsgNegL2.  The maximum is over k_i.k_j *
+// rn_j (cosine), k_i.k_j (dot) or 2 k_i.k_j - |k_j|^2 (negative L2); the
+// selection kernel finishes rho with the row's own term.
 cudaError_t launch_tsg(const Problem& p, const FrameTable& ft, const LayerPtrs& io,
-                       Strided<const float> rn, Strided<float> rho_part, int metric, cudaStream_t st);
+                       Strided<const float> rn, Strided<uint32_t> rho_key, int metric, cudaStream_t st);
 cudaError_t launch_tsg_umma(const Problem& p, const FrameTable& ft, const LayerPtrs& io,
-                            Strided<const float> rn_cur, int cur_pad, Strided<float> rho_part, int metric,
+                            Strided<const float> rn_cur, int cur_pad, Strided<uint32_t> rho_key, int metric,
                             uint32_t* err, cudaStream_t st);
 
-// CSS saliency Phi (Eqs. 4-5) of every visual token; also writes the inverse
-// key norms of every visual token to rn (and of the current frame's to
-// rn_cur, as launch_inv_norms).  Text entries are not touched.
-cudaError_t launch_css(const Problem& p, const FrameTable& ft, const LayerPtrs& io,
-                       Strided<float> phi, Strided<float> rn, Strided<float> rn_cur, int cur_pad,
-                       cudaStream_t st);
+// CSS saliency Phi (Eqs. 4-5) of every visual token; also writes the norms'
+// outputs of every visual token.  Text entries are not touched.
+cudaError_t launch_css(const Problem& p, const FrameTable& ft, const LayerPtrs& io, Strided<float> phi,
+                       const NormsOut& norms, cudaStream_t st);
 // Tensor-core CSS (bf16, every grid at most 127 wide): per-token squared-norm
-// and E/S/SE/SW dots on the tensor cores, then Phi; writes rn and rn_cur as
-// launch_css does.  with_phi = false stops after the dots (rn and rn_cur
+// and E/S/SE/SW dots on the tensor cores, then Phi; writes the norms' outputs
+// as launch_css does.  with_phi = false stops after the dots (norms
 // written), for a later launch_css_phi on the same dots.
 bool css_umma_supported(const FrameTable& ft);
 cudaError_t launch_css_umma(const Problem& p, const FrameTable& ft, const LayerPtrs& io, Strided<float> phi,
-                            Strided<float> rn, Strided<float> rn_cur, int cur_pad, Strided<float> dE,
-                            Strided<float> dS, Strided<float> dSE, Strided<float> dSW, uint32_t* err,
-                            cudaStream_t st, bool with_phi = true);
+                            const NormsOut& norms, Strided<float> dE, Strided<float> dS, Strided<float> dSE,
+                            Strided<float> dSW, uint32_t* err, cudaStream_t st, bool with_phi = true);
 // Phi of the CSS dots (the second kernel of launch_css_umma, on its own;
 // the caller orders it after the dots are written).
-cudaError_t launch_css_phi(const Problem& p, const FrameTable& ft, Strided<float> phi, Strided<float> rn,
-                           Strided<float> rn_cur, int cur_pad, Strided<float> dE, Strided<float> dS,
-                           Strided<float> dSE, Strided<float> dSW, cudaStream_t st);
+cudaError_t launch_css_phi(const Problem& p, const FrameTable& ft, Strided<float> phi, Strided<const float> rn,
+                           Strided<float> dE, Strided<float> dS, Strided<float> dSE, Strided<float> dSW,
+                           cudaStream_t st);
 // CSS over the size x size neighbourhood (size 3, 5, 7 or 9; 3 is the
 // method's Moore neighbourhood) on the CUDA cores, through box sums of the
-// normalised keys; any grid width.  Writes phi, rn and rn_cur as launch_css.
+// normalised keys; any grid width.  Writes phi and the norms' outputs as
+// launch_css.
 cudaError_t launch_css_box(const Problem& p, const FrameTable& ft, const LayerPtrs& io, int size,
-                           Strided<float> phi, Strided<float> rn, Strided<float> rn_cur, int cur_pad,
-                           cudaStream_t st);
+                           Strided<float> phi, const NormsOut& norms, cudaStream_t st);
 // phi[h][j] = NaN for every text token j (one layer).
 cudaError_t launch_fill_text_nan(const Problem& p, const FrameTable& ft, float* phi, cudaStream_t st);
 
@@ -177,18 +180,17 @@ constexpr int kTsgCosine = 0, kTsgDot = 1, kTsgNegL2 = 2;
 struct SelectArgs {
   int mode;
   int budget[kMaxLayers];  // per layer
-  int nchunk;
   int tsg_enable;
   int css_enable;
   float alpha;
-  int tsg_metric;      // kTsgCosine / kTsgDot / kTsgNegL2: how rho is finished from the slices
+  int tsg_metric;      // kTsgCosine / kTsgDot / kTsgNegL2: how rho is finished from the row maxima
   int tsg_fixed;       // 1: tau = tsg_fixed_tau instead of the adaptive select (Eq. 7)
   float tsg_fixed_tau;
   int base_uniform;    // 1: A = a_uniform for every token instead of a_base
   float a_uniform;
   int a_norm_max;      // 1: A / max_j A per head before Eq. 9
   int write_stages;    // 1: write rho, gate and score (the staged outputs); 0: only tau and the indices
-  Strided<const float> rho_part;  // [nchunk][Hkv][N]
+  Strided<const uint32_t> rho_key;  // [Hkv][N]
   Strided<const float> rn;        // [Hkv][N]
   Strided<float> rho;             // out [Hkv][N]
   Strided<float> tau;             // out [Hkv]

@@ -1,18 +1,20 @@
 // Selection kernel.  One cluster of CL CTAs per (layer, KV head); CTA c of a
 // cluster owns the contiguous token range [c*chunk, (c+1)*chunk) and keeps
 // its radix keys in shared memory for every pass.
-//   kSelGate: rho_i = |k_i|^-1 * max over slices of rho_part (Eq. 6), tau =
+//   kSelGate: rho_i = |k_i|^-1 * TSG's row maximum (Eq. 6), tau =
 //             the min(B, |pool|)-th smallest rho (Eq. 7), gate = rho <= tau
 //             (Eq. 8).
 //   kSelTopk: S from Eq. 9, then the B-th largest S and an ordered stream
 //             compaction that emits the kept indices in ascending order,
 //             equal scores resolved towards lower indices.
-// Both selections are exact radix selects on the order-preserving uint32
-// images of the fp32 values, 8 bits per pass.  Each pass builds per-warp
-// histograms (warp-aggregated, no cross-warp atomics), sums them per CTA,
-// then every CTA sums the cluster's histograms through distributed shared
-// memory and picks the same digit; one cluster barrier per pass.
+// Both selections are exact selects on the order-preserving uint32 images of
+// the fp32 values (cluster_select below): the cluster's key range, a 1,024-bin
+// histogram of it, and the few keys of the chosen bin gathered into every CTA
+// and resolved there.
 #include <cooperative_groups.h>
+
+#include <algorithm>
+#include <atomic>
 
 #include "kernels.cuh"
 
@@ -24,12 +26,24 @@ constexpr int kSelThreads = 512;  // two per histogram bin in the radix passes
 constexpr int kSelMaxCluster = 8;
 constexpr int kSelMaxChunk = 49152;  // keys per CTA held in shared memory (192 KB)
 
+constexpr int kSelWarps = kSelThreads / 32;
+constexpr int kSelBins = 1024;           // bins of a histogram pass: two per thread
+constexpr int kSelGather = 2 * kSelThreads;  // most keys a chosen bin may hold to be gathered
+static_assert(kSelBins == 2 * kSelThreads, "a thread sums two bins");
+static_assert(kSelMaxChunk < 65536, "a CTA's bins and counts are 16-bit");
+
+// The keys above a pivot (see cluster_select), of a thread, a CTA or the cluster.
+struct SelStats {
+  uint32_t n, mn, mx;  // their count, the smallest and the largest
+};
+
 struct SelShared {
-  uint32_t whist[kSelThreads / 32][256];  // per-warp histograms
-  uint32_t hist[2][256];  // this CTA's histogram, double-buffered by pass parity
-  uint32_t tot[256];      // cluster-wide histogram of the current pass
-  uint32_t dig[2][3];     // (digit, count above it, count in it), double-buffered by pass parity
-  uint32_t bcast[4];
+  uint32_t hist[2][kSelBins / 2];  // bins 2t (low half) and 2t + 1 of this CTA's keys, by pass parity
+  uint32_t cand[kSelGather];       // the cluster's keys of the chosen bin
+  uint32_t fine[3][256];           // histograms of them
+  SelStats stats[2][2];   // of this CTA: per select of the kernel, above the pivot; at and below it
+  uint32_t n_list;        // keys of the CTA in the chosen bin
+  uint32_t dig[4];        // (bin, count above it, count in it, count in it of the CTAs before this one)
   uint32_t warp_tot[32];
   uint32_t counts[2];     // (greater, equal) of this CTA for the compaction
   float warp_max[32];
@@ -37,6 +51,14 @@ struct SelShared {
   int32_t fr_off[kMaxFrames + 1];  // first token of every frame; fr_off[F] = INT_MAX
   int32_t fr_vend[kMaxFrames];     // end of every frame's visual span
 };
+
+// Cluster barrier (a block barrier when the CTA is alone).
+__device__ __forceinline__ void cluster_barrier(cg::cluster_group& cl, int ncta) {
+  if (ncta > 1)
+    cl.sync();
+  else
+    __syncthreads();
+}
 
 // Maximum of v over every thread of the cluster (every CTA must call it).
 __device__ float cluster_max(cg::cluster_group& cl, float v, SelShared& sh) {
@@ -50,7 +72,7 @@ __device__ float cluster_max(cg::cluster_group& cl, float v, SelShared& sh) {
     for (int w = 1; w < nw; ++w) m = fmaxf(m, sh.warp_max[w]);
     sh.cta_max = m;
   }
-  cl.sync();
+  cluster_barrier(cl, (int)cl.num_blocks());
   float m = -CUDART_INF_F;
   for (int r = 0; r < (int)cl.num_blocks(); ++r) m = fmaxf(m, *cl.map_shared_rank(&sh.cta_max, r));
   return m;
@@ -84,109 +106,241 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* w
   return before + x - v;
 }
 
-// k-th largest (1-indexed) key over the whole cluster; key 0 marks an empty
-// slot.  Returns the key T; *need_out = how many keys equal to T belong to
-// the top k.  Per pass: per-warp histograms, one block barrier, the CTA's
-// histogram (two threads per bin), one cluster barrier, the cluster's
-// histogram (two threads per bin, each reading half of the CTAs), one block
-// barrier, the digit found by warp 0, one block barrier.  The CTA histogram
-// and the digit broadcast are double-buffered by pass parity, so that no
-// barrier is needed before the next pass rewrites them: a buffer is
-// rewritten two passes later, after every thread has passed the barriers
-// that follow its last read.  early: the caller needs only the top-k set,
-// not the k-th key itself, so the select may stop once the chosen bin holds
-// exactly the keys still needed (all of them belong to the top k); it then
-// returns the bin's lower bound minus one with *need_out = 0, which selects
-// the same set.  Every CTA of the cluster takes that decision on the same
-// cluster histogram.
-__device__ uint32_t cluster_select_desc(cg::cluster_group& cl, const uint32_t* keys, int len,
-                                        uint32_t k, SelShared& sh, int& pass,
-                                        uint32_t* need_out, bool early) {
-  uint32_t prefix = 0, mask = 0, need = k;
-  const int tid = threadIdx.x, lane = tid & 31, nw = blockDim.x >> 5, wid = tid >> 5;
-  const int ncta = (int)cl.num_blocks();
-  uint32_t* wh = sh.whist[wid];
-  const int bin = tid >> 1, half = tid & 1;  // 512 threads: two per bin
-  for (int shift = 24; shift >= 0; shift -= 8, ++pass) {
-    uint32_t* hb = sh.hist[pass & 1];
-    for (int b = lane; b < 256; b += 32) wh[b] = 0u;
-    __syncwarp();
-    // per-warp histogram: shared atomics on the warp's own copy (lanes of one
-    // warp that hit one bin are combined by the atomic unit)
-    int i = tid;
-    for (; i + 3 * (int)blockDim.x < len; i += 4 * blockDim.x) {
-      uint32_t k4[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) k4[u] = keys[i + u * blockDim.x];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (k4[u] != 0u && (k4[u] & mask) == prefix) atomicAdd(&wh[(k4[u] >> shift) & 255u], 1u);
-    }
-    for (; i < len; i += blockDim.x) {
+__device__ __forceinline__ void stats_init(SelStats& st) { st = {0u, 0xffffffffu, 0u}; }
+__device__ __forceinline__ void stats_add(SelStats& st, uint32_t key, uint32_t pivot) {
+  if (key > pivot) {
+    ++st.n;
+    st.mn = min(st.mn, key);
+    st.mx = max(st.mx, key);
+  }
+}
+__device__ __forceinline__ void stats_reduce(SelStats& st) {  // over the warp
+  st.n = __reduce_add_sync(0xffffffffu, st.n);
+  st.mn = __reduce_min_sync(0xffffffffu, st.mn);
+  st.mx = __reduce_max_sync(0xffffffffu, st.mx);
+}
+// The cluster's statistics from every thread's (`cta` initialised before).
+__device__ __forceinline__ SelStats stats_cluster(cg::cluster_group& cl, int ncta, SelStats st, SelStats* cta) {
+  const int lane = threadIdx.x & 31;
+  stats_reduce(st);
+  if (lane == 0) {
+    atomicAdd(&cta->n, st.n);
+    atomicMin(&cta->mn, st.mn);
+    atomicMax(&cta->mx, st.mx);
+  }
+  cluster_barrier(cl, ncta);
+  stats_init(st);
+  if (lane < ncta) st = *cl.map_shared_rank(cta, lane);
+  stats_reduce(st);
+  return st;
+}
+
+struct Selected {
+  uint32_t T, need;  // the top k: every key > T, and `need` of the keys == T
+};
+
+// The k largest of the cluster's keys.  `mine`: this thread's statistics of
+// the keys above `pivot`, a value that many keys may share (0 for a closed
+// gate's score, or the mark of an empty slot): keys equal to it are counted
+// there instead of piling up in one bin.  set_only: the caller needs the set,
+// not the k-th key itself, so a bin that holds exactly the keys still needed
+// ends the select (T = its lower bound - 1, need = 0).  `sel` numbers the
+// kernel's selects, `pass` its histogram passes.
+//
+// The range [lo, hi] of the keys that can hold the k-th is known after one
+// exchange of the CTAs' statistics; a pass cuts it into 1,024 equal bins,
+// sums them over the cluster (a thread sums two bins, packed 16-bit in the
+// CTAs' copies) and finds the k-th key's bin.  If that bin's keys are few,
+// every CTA sends its own to all the others, and each resolves them alone;
+// else the bin becomes the range of the next pass (at most four: 32 bits).
+// That is three cluster barriers for an ordinary distribution, each of which
+// costs 0.6 us in a cluster of 4 and 1.2 us in one of 16.  Not inlined: the
+// kernel's second select then finds its instructions in the SM's cache, which
+// is worth 3 us of the 9-12 that a cold one takes.
+//
+// What the cluster's other CTAs read or write is reused only after a later
+// barrier that follows every such access: a pass's bins two passes later, the
+// gathered keys in the next select.
+__device__ __noinline__ Selected cluster_select(int ncta, const uint32_t* keys, int len, uint32_t k, uint32_t pivot,
+                                                SelStats mine, SelShared& sh, int sel, int& pass, bool set_only) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int rank = (int)cl.block_rank();
+  sh.hist[pass & 1][tid] = 0u;
+  if (tid == 0) sh.n_list = 0u;
+  SelStats st = stats_cluster(cl, ncta, mine, &sh.stats[sel][0]);  // (the keys are written, too)
+  uint32_t need = k;
+  if (need > st.n) {
+    // the k-th is the pivot or below: its count and the range below it
+    need -= st.n;
+    stats_init(mine);
+    uint32_t n_eq = 0;
+    for (int i = tid; i < len; i += kSelThreads) {
       const uint32_t key = keys[i];
-      if (key != 0u && (key & mask) == prefix) atomicAdd(&wh[(key >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    {
-      uint32_t t = 0;
-      const int w0 = half * (nw >> 1), w1 = w0 + (nw >> 1);
-#pragma unroll 8
-      for (int w = w0; w < w1; ++w) t += sh.whist[w][bin];
-      t += __shfl_xor_sync(0xffffffffu, t, 1);
-      if (half == 0) hb[bin] = t;
-    }
-    cl.sync();
-    {
-      uint32_t t = 0;
-      for (int r0 = half; r0 < ncta; r0 += 8) {  // four remote reads in flight
-        uint32_t v[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) v[r] = r0 + 2 * r < ncta ? cl.map_shared_rank(hb, r0 + 2 * r)[bin] : 0u;
-        t += (v[0] + v[1]) + (v[2] + v[3]);
+      n_eq += key == pivot;
+      if (key < pivot) {
+        mine.mn = min(mine.mn, key);
+        mine.mx = max(mine.mx, key);
       }
-      t += __shfl_xor_sync(0xffffffffu, t, 1);
-      if (half == 0) sh.tot[bin] = t;
+    }
+    mine.n = n_eq;
+    st = stats_cluster(cl, ncta, mine, &sh.stats[sel][1]);
+    if (need <= st.n) return {pivot, need};
+    need -= st.n;
+  }
+  uint32_t lo = st.mn, hi = st.mx;
+  for (int it = 0; it < 4; ++it) {  // a pass leaves at most a 1,024th of the range: four are enough for 32 bits
+    if (lo == hi) break;  // equal keys
+    const uint32_t span = hi - lo;
+    const int shift = max(0, 22 - __clz(span));  // span >> shift < 1,024
+    uint32_t* hist = sh.hist[pass & 1];
+    ++pass;
+    if (it > 0) {
+      hist[tid] = 0u;
+      __syncthreads();
+    }
+    auto count = [&](uint32_t key) {
+      const uint32_t b = (key - lo) >> shift;
+      if (key - lo <= span) atomicAdd(&hist[b >> 1], b & 1u ? 0x10000u : 1u);
+    };
+    for (int i = tid; i < len >> 2; i += kSelThreads) {
+      const uint4 x = reinterpret_cast<const uint4*>(keys)[i];
+      count(x.x);
+      count(x.y);
+      count(x.z);
+      count(x.w);
+    }
+    if (tid < (len & 3)) count(keys[(len & ~3) + tid]);
+    cluster_barrier(cl, ncta);
+    uint32_t c0 = 0, c1 = 0, b0 = 0, b1 = 0;  // counts of the thread's bins; of the CTAs before this one
+    for (int r0 = 0; r0 < ncta; r0 += 8) {    // eight remote reads in flight
+      uint32_t v[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) v[r] = r0 + r < ncta ? cl.map_shared_rank(hist, r0 + r)[tid] : 0u;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        c0 += v[r] & 0xffffu;
+        c1 += v[r] >> 16;
+        if (r0 + r < rank) {
+          b0 += v[r] & 0xffffu;
+          b1 += v[r] >> 16;
+        }
+      }
+    }
+    // keys in the bins above the thread's two: in its warp, then in the warps above
+    uint32_t incl = c0 + c1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_down_sync(0xffffffffu, incl, o);
+      if (lane + o < 32) incl += v;
+    }
+    if (lane == 0) sh.warp_tot[wid] = incl;
+    __syncthreads();
+    const uint32_t over = __reduce_add_sync(0xffffffffu, lane > wid && lane < kSelWarps ? sh.warp_tot[lane] : 0u);
+    const uint32_t above = over + incl - c0 - c1;
+    if (above < need && need <= above + c0 + c1) {
+      const bool up = need <= above + c1;
+      sh.dig[0] = 2 * tid + (up ? 1 : 0);
+      sh.dig[1] = up ? above : above + c1;
+      sh.dig[2] = up ? c1 : c0;
+      sh.dig[3] = up ? b1 : b0;
     }
     __syncthreads();
-    // warp 0: lane L holds bins 8L .. 8L+7; the digit is the bin where the
-    // count of larger keys first reaches need
-    uint32_t* dg = sh.dig[pass & 1];
-    if (tid < 32) {
-      uint32_t c[8], s = 0;
+    const uint32_t in_bin = sh.dig[2], first = sh.dig[3];
+    need -= sh.dig[1];
+    lo += sh.dig[0] << shift;
+    if (shift == 0) break;
+    if (set_only && in_bin == need && lo != 0u) return {lo - 1u, 0u};
+    hi = lo + min(hi - lo, (1u << shift) - 1u);
+    if (in_bin > kSelGather) continue;
+    // list the bin's keys, then send the list to every CTA
+    const uint32_t width = hi - lo;
+    auto list = [&](uint32_t key) {
+      if (key - lo <= width) sh.cand[first + atomicAdd(&sh.n_list, 1u)] = key;
+    };
+    for (int i = tid; i < len >> 2; i += kSelThreads) {
+      const uint4 x = reinterpret_cast<const uint4*>(keys)[i];
+      list(x.x);
+      list(x.y);
+      list(x.z);
+      list(x.w);
+    }
+    if (tid < (len & 3)) list(keys[(len & ~3) + tid]);
+    if (tid < 256) sh.fine[0][tid] = 0u;
+    __syncthreads();
+    if (ncta > 1) {
+      const uint32_t n = sh.n_list;
+      for (uint32_t i = tid; i < n; i += kSelThreads) {
+        const uint32_t key = sh.cand[first + i];
+        for (int r = 0; r < ncta; ++r)
+          if (r != rank) cl.map_shared_rank(sh.cand, r)[first + i] = key;
+      }
+      cl.sync();
+    }
+    if (in_bin <= 32) {
+      // every warp alone, a key per lane: the k-th has `need` keys at or
+      // above it and fewer than that above
+      const uint32_t key = lane < in_bin ? sh.cand[lane] : 0u;
+      uint32_t gt = 0, ge = 0;
+      for (uint32_t x = 0; x < in_bin; ++x) {
+        const uint32_t o = __shfl_sync(0xffffffffu, key, x);
+        gt += o > key;
+        ge += o >= key;
+      }
+      const bool is = lane < in_bin && gt < need && need <= ge;
+      const int src = __ffs(__ballot_sync(0xffffffffu, is)) - 1;
+      lo = __shfl_sync(0xffffffffu, key, src);
+      need -= __shfl_sync(0xffffffffu, gt, src);
+      break;
+    }
+    // 256 equal bins of the range at a time (it is below 2^22), every warp
+    // finding the bin for itself; three histograms in turn, so that the one
+    // zeroed for the next round is not the one read last
+    const uint32_t k0 = tid < in_bin ? sh.cand[tid] : 0u;  // below lo: not counted
+    const uint32_t k1 = tid + kSelThreads < in_bin ? sh.cand[tid + kSelThreads] : 0u;
+    for (int round = 0; round < 3 && lo != hi; ++round) {
+      const uint32_t w = hi - lo;
+      const int s = max(0, 24 - __clz(w));  // w >> s < 256
+      uint32_t* h = sh.fine[round];
+      if (tid < in_bin && k0 - lo <= w) atomicAdd(&h[(k0 - lo) >> s], 1u);
+      if (tid + kSelThreads < in_bin && k1 - lo <= w) atomicAdd(&h[(k1 - lo) >> s], 1u);
+      if (round < 2 && tid < 256) h[256 + tid] = 0u;
+      __syncthreads();
+      uint32_t c[8], sum = 0;
 #pragma unroll
       for (int b = 0; b < 8; ++b) {
-        c[b] = sh.tot[lane * 8 + b];
-        s += c[b];
+        c[b] = h[lane * 8 + b];
+        sum += c[b];
       }
-      uint32_t incl = s;  // sum over lanes >= lane
+      uint32_t in = sum;  // over this lane and the ones above
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        uint32_t v = __shfl_down_sync(0xffffffffu, incl, o);
-        if (lane + o < 32) incl += v;
+        const uint32_t v = __shfl_down_sync(0xffffffffu, in, o);
+        if (lane + o < 32) in += v;
       }
-      uint32_t above = incl - s;
+      uint32_t up = in - sum, bin = 0, cnt = 0, left = 0;
+      const bool here = up < need && need <= in;
 #pragma unroll
       for (int b = 7; b >= 0; --b) {
-        if (above < need && need <= above + c[b]) {
-          dg[0] = (uint32_t)(lane * 8 + b);
-          dg[1] = above;
-          dg[2] = c[b];
+        if (up < need && need <= up + c[b]) {
+          bin = lane * 8 + b;
+          cnt = c[b];
+          left = need - up;
         }
-        above += c[b];
+        up += c[b];
       }
+      const int src = __ffs(__ballot_sync(0xffffffffu, here)) - 1;
+      bin = __shfl_sync(0xffffffffu, bin, src);
+      cnt = __shfl_sync(0xffffffffu, cnt, src);
+      need = __shfl_sync(0xffffffffu, left, src);
+      lo += bin << s;
+      if (s == 0) break;
+      if (set_only && cnt == need && lo != 0u) return {lo - 1u, 0u};
+      hi = lo + min(hi - lo, (1u << s) - 1u);
     }
-    __syncthreads();
-    need -= dg[1];
-    prefix |= dg[0] << shift;
-    mask |= 0xffu << shift;
-    if (early && shift > 0 && dg[2] == need && prefix != 0u) {
-      ++pass;  // the parity sequence of the double buffers goes on
-      *need_out = 0u;
-      return prefix - 1u;
-    }
+    break;
   }
-  *need_out = need;
-  return prefix;
+  return {lo, need};
 }
 
 // Warms L2 with the 128-byte lines of x[j0, j1) (one prefetch per line):
@@ -198,13 +352,6 @@ __device__ __forceinline__ void prefetch_l2(const void* x, size_t elem, int j0, 
   for (size_t o = (lo & ~(size_t)127) + (size_t)threadIdx.x * 128; o < hi; o += (size_t)blockDim.x * 128)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(b + o));
 }
-
-// Inputs of one pool token's rho: the row maxima of the TSG slices (folded
-// into four) and 1/|k_i|.
-struct RhoIn {
-  float s[4];
-  float rn;
-};
 
 // Token kinds of the flat loops.
 constexpr int kTokText = 0;  // not inside any frame's visual span
@@ -287,7 +434,7 @@ __device__ __forceinline__ void for_tokens4(const SelShared& sh, int F, int j0, 
 }
 
 struct RhoIn4 {
-  float4 s[4];
+  uint4 m;
   float4 rn;
 };
 struct ScoreIn4 {
@@ -315,6 +462,7 @@ __global__ void __launch_bounds__(kSelThreads, 4) k_select(Problem p, const __gr
     sh.fr_off[f] = f < F ? ft.off[f] : 0x7fffffff;
     if (f < F) sh.fr_vend[f] = ft.off[f] + ft.gh[f] * ft.gw[f];
   }
+  if (tid < 4) stats_init(sh.stats[tid >> 1][tid & 1]);
   __syncthreads();
   // tau comes from a selection only when there is a pool and TSG is on;
   // otherwise tau = NaN and every gate stays open
@@ -323,20 +471,21 @@ __global__ void __launch_bounds__(kSelThreads, 4) k_select(Problem p, const __gr
   uint32_t kt_gate = 0u;  // gate: rho <= tau, i.e. key (~float_key(rho)) >= kt_gate
   uint8_t* gate = a.gate.base ? a.gate.at(l) + hn : nullptr;
 
+  SelStats ks;  // of the keys this thread writes
   if (a.mode & kSelGate) {
+    stats_init(ks);
     float* rho = a.rho.at(l) + hn;
-    const float* rp = a.rho_part.at(l) + hn;
+    const uint32_t* rk = a.rho_key.at(l) + hn;
     const float* rn = a.rn.at(l) + hn;
-    const size_t slice = (size_t)p.hkv * n;
-    const int nsl = a.nchunk;
-    for (int s = 0; s < nsl; ++s) prefetch_l2(rp + (size_t)s * slice, 4, j0, j1);
+    prefetch_l2(rk, 4, j0, j1);
     prefetch_l2(rn, 4, j0, j1);
-    // rho of every token: pool tokens from the TSG slices and 1/|k_i|, NaN
+    // rho of every token: pool tokens from TSG's maxima and 1/|k_i|, NaN
     // elsewhere; the selection keys are complements (m-th smallest rho ==
     // m-th largest key), 0 marks a token outside the pool.  Finish Eq. 6
     // with the row's own term: times 1/|k_i| (cosine), nothing (dot), minus
     // |k_i|^2 (negative squared L2).
-    auto finish = [&](float m, float rnv) {
+    auto finish = [&](uint32_t key, float rnv) {
+      const float m = key_float(key);
       return a.tsg_metric == kTsgCosine ? m * rnv : (a.tsg_metric == kTsgDot ? m : m - 1.f / (rnv * rnv));
     };
     if (vec) {
@@ -344,65 +493,43 @@ __global__ void __launch_bounds__(kSelThreads, 4) k_select(Problem p, const __gr
           sh, F, j0, j1,
           [&](int t0, const int (&kinds)[4]) {
             RhoIn4 r;
-            const float ninf = -CUDART_INF_F;
-#pragma unroll
-            for (int s = 0; s < 4; ++s) r.s[s] = make_float4(ninf, ninf, ninf, ninf);
+            r.m = make_uint4(0u, 0u, 0u, 0u);
             r.rn = make_float4(0.f, 0.f, 0.f, 0.f);
             if (kinds[0] == kTokPool || kinds[1] == kTokPool || kinds[2] == kTokPool || kinds[3] == kTokPool) {
-              const float* src = rp + t0;
-#pragma unroll
-              for (int s = 0; s < 4; ++s)
-                if (s < nsl) r.s[s] = __ldg(reinterpret_cast<const float4*>(src + (size_t)s * slice));
-              for (int s = 4; s < nsl; ++s) {
-                const float4 x = __ldg(reinterpret_cast<const float4*>(src + (size_t)s * slice));
-                r.s[3] = make_float4(fmaxf(r.s[3].x, x.x), fmaxf(r.s[3].y, x.y), fmaxf(r.s[3].z, x.z),
-                                     fmaxf(r.s[3].w, x.w));
-              }
+              r.m = __ldg(reinterpret_cast<const uint4*>(rk + t0));
               r.rn = __ldg(reinterpret_cast<const float4*>(rn + t0));
             }
             return r;
           },
           [&](int t0, const int (&kinds)[4], const RhoIn4& v) {
-            const float m0 = fmaxf(fmaxf(v.s[0].x, v.s[1].x), fmaxf(v.s[2].x, v.s[3].x));
-            const float m1 = fmaxf(fmaxf(v.s[0].y, v.s[1].y), fmaxf(v.s[2].y, v.s[3].y));
-            const float m2 = fmaxf(fmaxf(v.s[0].z, v.s[1].z), fmaxf(v.s[2].z, v.s[3].z));
-            const float m3 = fmaxf(fmaxf(v.s[0].w, v.s[1].w), fmaxf(v.s[2].w, v.s[3].w));
-            const float r0 = kinds[0] == kTokPool ? finish(m0, v.rn.x) : CUDART_NAN_F;
-            const float r1 = kinds[1] == kTokPool ? finish(m1, v.rn.y) : CUDART_NAN_F;
-            const float r2 = kinds[2] == kTokPool ? finish(m2, v.rn.z) : CUDART_NAN_F;
-            const float r3 = kinds[3] == kTokPool ? finish(m3, v.rn.w) : CUDART_NAN_F;
+            const float r0 = kinds[0] == kTokPool ? finish(v.m.x, v.rn.x) : CUDART_NAN_F;
+            const float r1 = kinds[1] == kTokPool ? finish(v.m.y, v.rn.y) : CUDART_NAN_F;
+            const float r2 = kinds[2] == kTokPool ? finish(v.m.z, v.rn.z) : CUDART_NAN_F;
+            const float r3 = kinds[3] == kTokPool ? finish(v.m.w, v.rn.w) : CUDART_NAN_F;
             if (a.write_stages) *reinterpret_cast<float4*>(rho + t0) = make_float4(r0, r1, r2, r3);
-            *reinterpret_cast<uint4*>(keys + (t0 - j0)) =
-                make_uint4(kinds[0] == kTokPool ? ~float_key(r0) : 0u, kinds[1] == kTokPool ? ~float_key(r1) : 0u,
-                           kinds[2] == kTokPool ? ~float_key(r2) : 0u, kinds[3] == kTokPool ? ~float_key(r3) : 0u);
+            const uint4 kv = make_uint4(kinds[0] == kTokPool ? ~float_key(r0) : 0u,
+                                        kinds[1] == kTokPool ? ~float_key(r1) : 0u,
+                                        kinds[2] == kTokPool ? ~float_key(r2) : 0u,
+                                        kinds[3] == kTokPool ? ~float_key(r3) : 0u);
+            *reinterpret_cast<uint4*>(keys + (t0 - j0)) = kv;
+            stats_add(ks, kv.x, 0u);
+            stats_add(ks, kv.y, 0u);
+            stats_add(ks, kv.z, 0u);
+            stats_add(ks, kv.w, 0u);
           });
     } else
     for_tokens<2>(
         sh, F, j0, j1,
         [&](int t, int kind) {
-          // independent loads (no max between them), so that all of a
-          // batch's slices are in flight together
-          RhoIn r;
-#pragma unroll
-          for (int s = 0; s < 4; ++s) r.s[s] = -CUDART_INF_F;
-          r.rn = CUDART_NAN_F;
-          if (kind == kTokPool) {
-            const float* src = rp + t;
-#pragma unroll
-            for (int s = 0; s < 4; ++s)
-              if (s < nsl) r.s[s] = __ldg(src + (size_t)s * slice);
-            for (int s = 4; s < nsl; ++s) r.s[3] = fmaxf(r.s[3], __ldg(src + (size_t)s * slice));
-            r.rn = __ldg(rn + t);
-          }
-          return r;
+          return kind == kTokPool ? make_uint2(__ldg(rk + t), __float_as_uint(__ldg(rn + t))) : make_uint2(0u, 0u);
         },
-        [&](int t, int kind, const RhoIn& v) {
-          const float m = fmaxf(fmaxf(v.s[0], v.s[1]), fmaxf(v.s[2], v.s[3]));
-          const float r = kind == kTokPool ? finish(m, v.rn) : CUDART_NAN_F;
+        [&](int t, int kind, uint2 v) {
+          const float r = kind == kTokPool ? finish(v.x, __uint_as_float(v.y)) : CUDART_NAN_F;
           if (a.write_stages) rho[t] = r;
-          keys[t - j0] = kind == kTokPool ? ~float_key(r) : 0u;
+          const uint32_t key = kind == kTokPool ? ~float_key(r) : 0u;
+          keys[t - j0] = key;
+          stats_add(ks, key, 0u);
         });
-    __syncthreads();
     // the score phase's inputs arrive in L2 while tau is selected
     if ((a.mode & kSelTopk) && !a.base_uniform) prefetch_l2(a.a_base.at(l) + hn, 4, j0, j1);
     if ((a.mode & kSelTopk) && a.phi.base && a.css_enable) prefetch_l2(a.phi.at(l) + hn, 4, j0, j1);
@@ -412,13 +539,14 @@ __global__ void __launch_bounds__(kSelThreads, 4) k_select(Problem p, const __gr
         kt_gate = ~float_key(tau);
       } else {
         // the fused call needs only the gated set; the staged call reports tau
-        uint32_t need;
-        kt_gate = cluster_select_desc(cl, keys, len, (uint32_t)min(a.budget[l], pool), sh, pass, &need,
-                                      !a.write_stages);
+        const Selected g = cluster_select(ncta, keys, len, (uint32_t)min(a.budget[l], pool), 0u, ks, sh, 0, pass,
+                                          !a.write_stages);
+        kt_gate = g.need ? g.T : g.T + 1u;
         tau = key_float(~kt_gate);
       }
     }
     if (c == 0 && tid == 0) a.tau.at(l)[h] = tau;
+    __syncthreads();  // the keys are written, also without a select
     if (!(a.mode & kSelTopk)) {
       // gate only: Eq. 8 on the pool, open elsewhere
       for_tokens<2>(
@@ -466,6 +594,8 @@ __global__ void __launch_bounds__(kSelThreads, 4) k_select(Problem p, const __gr
       }
       return s;
     };
+    const uint32_t zero_key = float_key(0.f);  // a closed gate's score
+    stats_init(ks);
     if (vec) {
       for_tokens4(
           sh, F, j0, j1,
@@ -491,8 +621,12 @@ __global__ void __launch_bounds__(kSelThreads, 4) k_select(Problem p, const __gr
             const float s3 = score_of(t0 + 3, kinds[3], v.A.w, kinds[3] != kTokText ? v.P.w : 0.f,
                                       (float)(v.G >> 24));
             if (a.write_stages) *reinterpret_cast<float4*>(sc + t0) = make_float4(s0, s1, s2, s3);
-            *reinterpret_cast<uint4*>(keys + (t0 - j0)) =
-                make_uint4(float_key(s0), float_key(s1), float_key(s2), float_key(s3));
+            const uint4 kv = make_uint4(float_key(s0), float_key(s1), float_key(s2), float_key(s3));
+            *reinterpret_cast<uint4*>(keys + (t0 - j0)) = kv;
+            stats_add(ks, kv.x, zero_key);
+            stats_add(ks, kv.y, zero_key);
+            stats_add(ks, kv.z, zero_key);
+            stats_add(ks, kv.w, zero_key);
           });
     } else
     for_tokens<2>(
@@ -507,11 +641,12 @@ __global__ void __launch_bounds__(kSelThreads, 4) k_select(Problem p, const __gr
         [&](int t, int kind, float3 v) {
           const float s = score_of(t, kind, v.x, v.y, v.z);
           if (a.write_stages) sc[t] = s;
-          keys[t - j0] = float_key(s);
+          const uint32_t key = float_key(s);
+          keys[t - j0] = key;
+          stats_add(ks, key, zero_key);
         });
-    __syncthreads();
-    uint32_t need;
-    const uint32_t T = cluster_select_desc(cl, keys, len, (uint32_t)a.budget[l], sh, pass, &need, true);
+    const Selected top = cluster_select(ncta, keys, len, (uint32_t)a.budget[l], zero_key, ks, sh, 1, pass, true);
+    const uint32_t T = top.T, need = top.need;
     // Ordered compaction.  Thread tid owns the contiguous run [r0, r1) of
     // this CTA's keys (odd run length: conflict-free shared reads); one
     // block scan gives its (greater, equal) counts before the run, the
@@ -530,19 +665,15 @@ __global__ void __launch_bounds__(kSelThreads, 4) k_select(Problem p, const __gr
       sh.counts[0] = tot & 0xffffu;
       sh.counts[1] = tot >> 16;
     }
-    cl.sync();
-    if (tid == 0) {
-      uint32_t gb = 0, eb = 0;
-      for (int r = 0; r < c; ++r) {
-        const uint32_t* rc = cl.map_shared_rank(sh.counts, r);
-        gb += rc[0];
-        eb += rc[1];
-      }
-      sh.bcast[2] = gb;
-      sh.bcast[3] = eb;
+    cluster_barrier(cl, ncta);
+    uint32_t gb = 0, eb = 0;  // of the CTAs before this one
+    if ((tid & 31) < c) {
+      const uint32_t* rc = cl.map_shared_rank(sh.counts, tid & 31);
+      gb = rc[0];
+      eb = rc[1];
     }
-    __syncthreads();
-    uint32_t gt_before = sh.bcast[2] + (ex & 0xffffu), eq_before = sh.bcast[3] + (ex >> 16);
+    uint32_t gt_before = __reduce_add_sync(0xffffffffu, gb) + (ex & 0xffffu);
+    uint32_t eq_before = __reduce_add_sync(0xffffffffu, eb) + (ex >> 16);
     int32_t* out = a.idx[l] + (size_t)h * a.budget[l];
     // kept: every key > T, and the first `need` keys == T in index order;
     // a kept token's slot = kept tokens before it
@@ -557,17 +688,19 @@ __global__ void __launch_bounds__(kSelThreads, 4) k_select(Problem p, const __gr
       }
     }
   }
-  cl.sync();  // no CTA leaves while a peer may still read its shared memory
+  cluster_barrier(cl, ncta);  // no CTA leaves while a peer may still read its shared memory
 }
 
 int select_max_tokens() { return kSelMaxCluster * kSelMaxChunk; }
+
+static int select_chunk(int n, int cl) { return ((n + cl - 1) / cl + 3) & ~3; }
 
 static void select_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, const Problem& p, int cl,
                           cudaStream_t st) {
   *cfg = cudaLaunchConfig_t{};
   cfg->gridDim = dim3(cl, p.L * p.hkv, 1);
   cfg->blockDim = dim3(kSelThreads, 1, 1);
-  cfg->dynamicSmemBytes = (size_t)(((p.n + cl - 1) / cl + 3) & ~3) * 4;
+  cfg->dynamicSmemBytes = (size_t)select_chunk(p.n, cl) * 4;
   cfg->stream = st;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = cl;
@@ -577,11 +710,21 @@ static void select_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, co
   cfg->numAttrs = 1;
 }
 
+// Clusters of c CTAs, `occ` of them to an SM, that are resident at once on
+// device dev: what the occupancy query says, which depends on nothing else
+// here, asked once per (device, c, occ) -- a query takes the host 5 us, and a
+// launch compares up to nine cluster sizes.
+static cudaError_t clusters_fit(int dev, int c, int occ, const cudaLaunchConfig_t& cfg, int* fit) {
+  constexpr int kDevices = 64;
+  static std::atomic<int> known[kDevices][2 * kSelMaxCluster + 1][2048 / kSelThreads + 1];  // fit + 1; 0: not asked
+  std::atomic<int>* slot = dev < kDevices ? &known[dev][c][occ] : nullptr;
+  if (slot && (*fit = slot->load(std::memory_order_relaxed) - 1) >= 0) return cudaSuccess;
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(fit, k_select, &cfg);
+  if (e == cudaSuccess && slot) slot->store(*fit + 1, std::memory_order_relaxed);
+  return e;
+}
+
 cudaError_t launch_select(const Problem& p, const FrameTable& ft, const SelectArgs& a, cudaStream_t st) {
-  // Cluster size: the CTAs of a cluster split one (layer, head)'s tokens.
-  // Each CTA is latency-bound on its own chunk, so the estimated time is
-  // (waves of co-resident clusters) x (chunk length); the smallest cluster
-  // with the lowest estimate wins (fewer CTAs per cluster barrier).
   cudaError_t e = cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)(kSelMaxChunk * 4));
   if (e != cudaSuccess) return e;
@@ -590,39 +733,50 @@ cudaError_t launch_select(const Problem& p, const FrameTable& ft, const SelectAr
   e = cudaFuncSetAttribute(k_select, cudaFuncAttributePreferredSharedMemoryCarveout,
                            (int)cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
+  // clusters of 16 (non-portable) where the device takes them
+  const bool big = cudaFuncSetAttribute(k_select, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+  int nsm = 0, dev = 0, sm_smem = 0, cta_smem = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&cta_smem, cudaDevAttrReservedSharedMemoryPerBlock, dev)) != cudaSuccess) return e;
+  cta_smem += (int)sizeof(SelShared);
+  // Cluster size: the CTAs of a cluster split one (layer, head)'s tokens.
+  // Measured (one wave of clusters, GB300): 13 us for a lone CTA and about
+  // 16.5 + 0.55 per CTA for a cluster's barriers and exchanges, plus 1.5 ns per
+  // token of a CTA or, where CTAs share SMs, 1.2 ns per token of an SM.  The
+  // least sum over the waves wins, the smallest cluster among equals: 28 x 4
+  // heads of 53,600 tokens take clusters of 5, which are all resident at once
+  // (74 us; 8 need two waves, 108), 28 x 4 of 2,144 single CTAs (17 us; 2: 21,
+  // 4: 27), 28 x 2 of 20,000 clusters of 4 (29; 3: 32, 8: 39), 4 of 23,680
+  // clusters of 8 (24; 16: 29, 4: 30), 4 of 132,800 clusters of 16 (44; 8: 56).
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  int cl = 0, fit8 = 0;
-  long long best = 0;
+  int cl = 0;
+  double best = 0.0;
   const long long units = (long long)p.L * p.hkv;
-  for (int c = 1; c <= kSelMaxCluster; c <<= 1) {
-    const int ch = ((p.n + c - 1) / c + 3) & ~3;
+  for (int c = 1; c <= (big ? 2 : 1) * kSelMaxCluster; c = c < kSelMaxCluster ? c + 1 : 2 * c) {
+    const int ch = select_chunk(p.n, c);
     if (ch > kSelMaxChunk) continue;
     select_config(&cfg, attr, p, c, st);
+    const int occ = std::min(2048 / kSelThreads, sm_smem / ((cta_smem + 4 * ch + 127) & ~127));
+    if (occ < 1) continue;
     int fit = 0;
-    if ((e = cudaOccupancyMaxActiveClusters(&fit, k_select, &cfg)) != cudaSuccess) return e;
-    if (c == kSelMaxCluster) fit8 = fit;
-    if (fit < 1) continue;
-    const long long est = (units + fit - 1) / fit * ch;
-    if (cl == 0 || est < best) {
-      cl = c;
-      best = est;
+    if ((e = clusters_fit(dev, c, occ, cfg, &fit)) != cudaSuccess) {
+      if (c <= kSelMaxCluster) return e;
+      break;
     }
-  }
-  // A few (layer, head) problems (one layer, a couple of layers) leave most
-  // SMs idle even with clusters of 8: clusters of 16 (non-portable) halve
-  // each CTA's tokens.  Only while they take at most one CTA per SM (the
-  // 16-CTA barriers cost more once CTAs share SMs), so that batches keep
-  // their portable shape.
-  int nsm = 0, dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    nsm = 0;
-  if (cl == kSelMaxCluster && units <= fit8 && units * 2 * kSelMaxCluster <= nsm &&
-      cudaFuncSetAttribute(k_select, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-    const int c = 2 * kSelMaxCluster;
-    select_config(&cfg, attr, p, c, st);
-    int fit = 0;
-    if (cudaOccupancyMaxActiveClusters(&fit, k_select, &cfg) == cudaSuccess && fit >= units) cl = c;
+    if (fit < 1) continue;
+    const double fixed = c == 1 ? 13.0 : 16.5 + 0.55 * c;
+    double cost = 0.0;
+    for (long long left = units; left > 0; left -= fit) {
+      const double per_sm = (double)std::min<long long>(left, fit) * c * ch / nsm;
+      cost += fixed + std::max(1.5e-3 * ch, 1.2e-3 * per_sm);
+    }
+    if (cl == 0 || cost < best) {
+      cl = c;
+      best = cost;
+    }
   }
   (void)cudaGetLastError();  // a refused non-portable query leaves no error behind
   if (cl == 0) return cudaErrorNotSupported;

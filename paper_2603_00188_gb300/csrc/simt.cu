@@ -35,13 +35,13 @@ __device__ __forceinline__ void unpack16(const uint4& w, float (&f)[16 / sizeof(
 // grid.y = layer.
 template <typename T>
 __global__ void __launch_bounds__(256) k_inv_norms(const __grid_constant__ LayerPtrs io, int n, int hkv,
-                                                   Strided<float> rn_all, Strided<float> rc_all, int cur_off,
-                                                   int cur_len, int cur_pad) {
+                                                   NormsOut norms, int cur_off, int cur_len) {
   constexpr int kChunks = kD * (int)sizeof(T) / 16;
   constexpr int kPer = 16 / (int)sizeof(T);
   const int l = blockIdx.y;
   const T* k = static_cast<const T*>(io.k[l]);
-  float* rn = rn_all.at(l);
+  float* rn = norms.rn.at(l);
+  uint32_t* rho = norms.rho_key.base ? norms.rho_key.at(l) : nullptr;
   const long long rows = (long long)n * hkv;
   for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < rows;
        r += (long long)gridDim.x * blockDim.x) {
@@ -60,12 +60,13 @@ __global__ void __launch_bounds__(256) k_inv_norms(const __grid_constant__ Layer
     const long long j = r / hkv, h = r - j * hkv;
     const float v = 1.0f / fmaxf(sqrtf(sn), 1e-8f);
     rn[h * n + j] = v;
-    if (j >= cur_off && j < cur_off + cur_len) rc_all.at(l)[h * cur_pad + (j - cur_off)] = v;
+    if (rho) rho[h * n + j] = 0u;
+    if (j >= cur_off && j < cur_off + cur_len) norms.rn_cur.at(l)[h * norms.cur_pad + (j - cur_off)] = v;
   }
 }
 
-cudaError_t launch_inv_norms(const Problem& p, const FrameTable& ft, const LayerPtrs& io, Strided<float> rn,
-                             Strided<float> rn_cur, int cur_pad, cudaStream_t st) {
+cudaError_t launch_inv_norms(const Problem& p, const FrameTable& ft, const LayerPtrs& io, const NormsOut& norms,
+                             cudaStream_t st) {
   long long rows = (long long)p.n * p.hkv;
   long long blocks = (rows + 255) / 256;
   long long cap = (152 * 8 + p.L - 1) / p.L;
@@ -73,9 +74,9 @@ cudaError_t launch_inv_norms(const Problem& p, const FrameTable& ft, const Layer
   TimingScope ts("inv_norms", st);
   dim3 grid((unsigned)blocks, p.L);
   if (p.dtype == kBF16)
-    k_inv_norms<__nv_bfloat16><<<grid, 256, 0, st>>>(io, p.n, p.hkv, rn, rn_cur, ft.cur_off, ft.cur_len, cur_pad);
+    k_inv_norms<__nv_bfloat16><<<grid, 256, 0, st>>>(io, p.n, p.hkv, norms, ft.cur_off, ft.cur_len);
   else
-    k_inv_norms<float><<<grid, 256, 0, st>>>(io, p.n, p.hkv, rn, rn_cur, ft.cur_off, ft.cur_len, cur_pad);
+    k_inv_norms<float><<<grid, 256, 0, st>>>(io, p.n, p.hkv, norms, ft.cur_off, ft.cur_len);
   return cudaGetLastError();
 }
 
@@ -114,8 +115,7 @@ struct CssGeom {
 template <typename T>
 __global__ void __launch_bounds__(kCssThreads) k_css(const __grid_constant__ LayerPtrs io,
                                                      const __grid_constant__ FrameTable ft, int hkv,
-                                                     Strided<float> phi_all, Strided<float> rn_all,
-                                                     Strided<float> rc_all, int cur_pad) {
+                                                     Strided<float> phi_all, NormsOut norms) {
   using Gm = CssGeom<T>;
   constexpr int kChunks = kD * (int)sizeof(T) / 16;
   constexpr int kPer = 16 / (int)sizeof(T);
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(kCssThreads) k_css(const __grid_constant__ Lay
   if (f >= ft.n_frames) return;
   const T* k = static_cast<const T*>(io.k[l]);
   float* phi = phi_all.at(l);
-  float* rn_out = rn_all.at(l);
+  float* rn_out = norms.rn.at(l);
   const int gh = ft.gh[f], gw = ft.gw[f], off = ft.off[f];
   int RB, CB;
   Gm::tile(gh, gw, RB, CB);
@@ -214,7 +214,8 @@ __global__ void __launch_bounds__(kCssThreads) k_css(const __grid_constant__ Lay
     const int j = off + u * gw + v;
     phi[(size_t)h * n + j] = cnt ? 1.0f - sum / (float)cnt : 0.0f;
     rn_out[(size_t)h * n + j] = r0;
-    if (f == ft.n_frames - 1) rc_all.at(l)[(size_t)h * cur_pad + (j - off)] = r0;
+    if (norms.rho_key.base) norms.rho_key.at(l)[(size_t)h * n + j] = 0u;
+    if (f == ft.n_frames - 1) norms.rn_cur.at(l)[(size_t)h * norms.cur_pad + (j - off)] = r0;
   }
 }
 
@@ -230,8 +231,7 @@ __global__ void k_fill_text_nan(const __grid_constant__ FrameTable ft, int hkv, 
 
 template <typename T>
 static cudaError_t css_launch_t(const Problem& p, const FrameTable& ft, const LayerPtrs& io,
-                                Strided<float> phi, Strided<float> rn, Strided<float> rn_cur, int cur_pad,
-                                cudaStream_t st) {
+                                Strided<float> phi, const NormsOut& norms, cudaStream_t st) {
   using Gm = CssGeom<T>;
   int tmax = 0, cmax = 0;
   for (int f = 0; f < ft.n_frames; ++f) {
@@ -245,15 +245,14 @@ static cudaError_t css_launch_t(const Problem& p, const FrameTable& ft, const La
   cudaError_t e = cudaFuncSetAttribute(k_css<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   TimingScope ts("css", st);
-  k_css<T><<<dim3(tmax, ft.n_frames, p.L * p.hkv), kCssThreads, smem, st>>>(io, ft, p.hkv, phi, rn, rn_cur,
-                                                                             cur_pad);
+  k_css<T><<<dim3(tmax, ft.n_frames, p.L * p.hkv), kCssThreads, smem, st>>>(io, ft, p.hkv, phi, norms);
   return cudaGetLastError();
 }
 
 cudaError_t launch_css(const Problem& p, const FrameTable& ft, const LayerPtrs& io, Strided<float> phi,
-                       Strided<float> rn, Strided<float> rn_cur, int cur_pad, cudaStream_t st) {
-  if (p.dtype == kBF16) return css_launch_t<__nv_bfloat16>(p, ft, io, phi, rn, rn_cur, cur_pad, st);
-  return css_launch_t<float>(p, ft, io, phi, rn, rn_cur, cur_pad, st);
+                       const NormsOut& norms, cudaStream_t st) {
+  if (p.dtype == kBF16) return css_launch_t<__nv_bfloat16>(p, ft, io, phi, norms, st);
+  return css_launch_t<float>(p, ft, io, phi, norms, st);
 }
 
 // ------------------------------------------------------- CSS, k x k box
@@ -281,8 +280,7 @@ struct BoxGeom {
 template <typename T, int R>
 __global__ void __launch_bounds__(kBoxThreads) k_css_box(const __grid_constant__ LayerPtrs io,
                                                          const __grid_constant__ FrameTable ft, int hkv,
-                                                         Strided<float> phi_all, Strided<float> rn_all,
-                                                         Strided<float> rc_all, int cur_pad) {
+                                                         Strided<float> phi_all, NormsOut norms) {
   using Gm = BoxGeom<T, R>;
   constexpr int kChunks = kD * (int)sizeof(T) / 16;
   constexpr int kPer = 16 / (int)sizeof(T);
@@ -331,8 +329,9 @@ __global__ void __launch_bounds__(kBoxThreads) k_css_box(const __grid_constant__
       r = 1.0f / fmaxf(sqrtf(sn), 1e-8f);
       if (a >= R && a < R + kBoxRows && b >= R && b < R + kBoxCols) {
         const int j = off + u * gw + v;
-        rn_all.at(l)[(size_t)h * n + j] = r;
-        if (f == ft.n_frames - 1) rc_all.at(l)[(size_t)h * cur_pad + (j - off)] = r;
+        norms.rn.at(l)[(size_t)h * n + j] = r;
+        if (norms.rho_key.base) norms.rho_key.at(l)[(size_t)h * n + j] = 0u;
+        if (f == ft.n_frames - 1) norms.rn_cur.at(l)[(size_t)h * norms.cur_pad + (j - off)] = r;
       }
     }
     rn[cell] = r;
@@ -399,7 +398,7 @@ __global__ void __launch_bounds__(kBoxThreads) k_css_box(const __grid_constant__
 
 template <typename T, int R>
 static cudaError_t css_box_t(const Problem& p, const FrameTable& ft, const LayerPtrs& io, Strided<float> phi,
-                             Strided<float> rn, Strided<float> rn_cur, int cur_pad, cudaStream_t st) {
+                             const NormsOut& norms, cudaStream_t st) {
   using Gm = BoxGeom<T, R>;
   cudaError_t e = cudaFuncSetAttribute(k_css_box<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, Gm::smem);
   if (e != cudaSuccess) return e;
@@ -410,29 +409,27 @@ static cudaError_t css_box_t(const Problem& p, const FrameTable& ft, const Layer
   }
   TimingScope ts("css_box", st);
   dim3 grid((unsigned)tiles, (unsigned)(ft.n_frames > 0 ? ft.n_frames : 1), (unsigned)(p.L * p.hkv));
-  k_css_box<T, R><<<grid, kBoxThreads, Gm::smem, st>>>(io, ft, p.hkv, phi, rn, rn_cur, cur_pad);
+  k_css_box<T, R><<<grid, kBoxThreads, Gm::smem, st>>>(io, ft, p.hkv, phi, norms);
   return cudaGetLastError();
 }
 
 template <typename T>
 static cudaError_t css_box_r(int radius, const Problem& p, const FrameTable& ft, const LayerPtrs& io,
-                             Strided<float> phi, Strided<float> rn, Strided<float> rn_cur, int cur_pad,
-                             cudaStream_t st) {
+                             Strided<float> phi, const NormsOut& norms, cudaStream_t st) {
   switch (radius) {
-    case 1: return css_box_t<T, 1>(p, ft, io, phi, rn, rn_cur, cur_pad, st);
-    case 2: return css_box_t<T, 2>(p, ft, io, phi, rn, rn_cur, cur_pad, st);
-    case 3: return css_box_t<T, 3>(p, ft, io, phi, rn, rn_cur, cur_pad, st);
-    case 4: return css_box_t<T, 4>(p, ft, io, phi, rn, rn_cur, cur_pad, st);
+    case 1: return css_box_t<T, 1>(p, ft, io, phi, norms, st);
+    case 2: return css_box_t<T, 2>(p, ft, io, phi, norms, st);
+    case 3: return css_box_t<T, 3>(p, ft, io, phi, norms, st);
+    case 4: return css_box_t<T, 4>(p, ft, io, phi, norms, st);
     default: return cudaErrorInvalidValue;
   }
 }
 
 cudaError_t launch_css_box(const Problem& p, const FrameTable& ft, const LayerPtrs& io, int size,
-                           Strided<float> phi, Strided<float> rn, Strided<float> rn_cur, int cur_pad,
-                           cudaStream_t st) {
+                           Strided<float> phi, const NormsOut& norms, cudaStream_t st) {
   if (ft.n_frames == 0) return cudaSuccess;
-  if (p.dtype == kBF16) return css_box_r<__nv_bfloat16>(size / 2, p, ft, io, phi, rn, rn_cur, cur_pad, st);
-  return css_box_r<float>(size / 2, p, ft, io, phi, rn, rn_cur, cur_pad, st);
+  if (p.dtype == kBF16) return css_box_r<__nv_bfloat16>(size / 2, p, ft, io, phi, norms, st);
+  return css_box_r<float>(size / 2, p, ft, io, phi, norms, st);
 }
 
 cudaError_t launch_fill_text_nan(const Problem& p, const FrameTable& ft, float* phi, cudaStream_t st) {
@@ -761,13 +758,13 @@ cudaError_t launch_score(const Problem& p, const LayerPtrs& io, Strided<float2> 
 
 // ------------------------------------------------------------------ TSG
 // fp32 path of Eq. 6: a tile of 64 historical tokens against the current
-// frame's keys of one column slice, streamed in tiles of 64.  Writes slice
-// blockIdx.z of rho_part.  grid = (half row tile, layer*Hkv + head, slice).
+// frame's keys of one column slice, streamed in tiles of 64; the slices fold
+// into rho_key.  grid = (half row tile, layer*Hkv + head, slice).
 constexpr int kTsgSimtSmem = (2 * kTileFloats + 2 * kTileRows) * 4;
 
 __global__ void __launch_bounds__(kTileThreads, kTilesPerSm)
     k_tsg_simt(const __grid_constant__ LayerPtrs io, const __grid_constant__ FrameTable ft, int hkv,
-               Strided<const float> rn_all, Strided<float> rho_all, int slice_cols, int metric) {
+               Strided<const float> rn_all, Strided<uint32_t> rho_all, int slice_cols, int metric) {
   extern __shared__ float4 tile_smem[];
   float* hs = reinterpret_cast<float*>(tile_smem);
   float* cs = hs + kTileFloats;
@@ -818,29 +815,28 @@ __global__ void __launch_bounds__(kTileThreads, kTilesPerSm)
 #pragma unroll
     for (int i = 0; i < kTA; ++i) cs[ty + 8 * i] = best[i];
   __syncthreads();
-  float* rho_part = rho_all.at(l) + ((size_t)blockIdx.z * hkv + h) * n;
+  uint32_t* rho_key = rho_all.at(l) + (size_t)h * n;
   if (tx == 0)
 #pragma unroll
     for (int i = 0; i < kTA; ++i) {
       const int tok = i0 + ty + 8 * i;
-      if (tok < fend) rho_part[tok] = fmaxf(best[i], cs[ty + 8 * i]);
+      if (tok < fend) atomicMax(rho_key + tok, float_key(fmaxf(best[i], cs[ty + 8 * i])));
     }
 }
 
-// Column slices of the fp32 TSG pass (1..kTsgSimtSlices): the count whose
-// CTAs, three to an SM, take the least time in whole waves, a wave costing
-// its column tiles plus about one for the row tile's load.  The slices fold
-// by maximum, so the count changes no result.
-int tsg_simt_slices(const Problem& p, const FrameTable& ft) {
-  if (ft.n_frames < 2) return 1;
+// Column slices of the fp32 TSG pass: the count whose CTAs, three to an SM,
+// take the least time in whole waves, a wave costing its column tiles plus
+// about one for the row tile's load.  The slices fold by maximum, so the
+// count changes no result.
+static int tsg_simt_slices(const Problem& p, const FrameTable& ft) {
   const long long rows = 2LL * ft.tile0[ft.n_frames - 1] * p.L * p.hkv;
   const int tiles = (ft.cur_len + kTileRows - 1) / kTileRows;
   const long long slots = 152 * kTilesPerSm;
   int best = 1;
   long long best_cost = 0;
-  for (int s = 1; s <= kTsgSimtSlices; ++s) {
+  for (int s = 1; s <= tiles && s <= 16; ++s) {
     const int per = (tiles + s - 1) / s;
-    if (s > 1 && (s - 1) * per >= tiles) break;  // an empty slice
+    if ((s - 1) * per >= tiles) continue;  // an empty slice
     const long long cost = ((rows * s + slots - 1) / slots) * (per + 1);
     if (s == 1 || cost < best_cost) {
       best = s;
@@ -851,7 +847,7 @@ int tsg_simt_slices(const Problem& p, const FrameTable& ft) {
 }
 
 cudaError_t launch_tsg(const Problem& p, const FrameTable& ft, const LayerPtrs& io, Strided<const float> rn,
-                       Strided<float> rho_part, int metric, cudaStream_t st) {
+                       Strided<uint32_t> rho_key, int metric, cudaStream_t st) {
   const int tiles = ft.n_frames >= 2 ? ft.tile0[ft.n_frames - 1] : 0;
   if (tiles == 0) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(k_tsg_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, kTsgSimtSmem);
@@ -860,7 +856,7 @@ cudaError_t launch_tsg(const Problem& p, const FrameTable& ft, const LayerPtrs& 
   const int ctiles = (ft.cur_len + kTileRows - 1) / kTileRows;
   const int slice_cols = (ctiles + slices - 1) / slices * kTileRows;
   TimingScope ts("tsg_simt", st);
-  k_tsg_simt<<<dim3(2 * tiles, p.L * p.hkv, slices), kTileThreads, kTsgSimtSmem, st>>>(io, ft, p.hkv, rn, rho_part,
+  k_tsg_simt<<<dim3(2 * tiles, p.L * p.hkv, slices), kTileThreads, kTsgSimtSmem, st>>>(io, ft, p.hkv, rn, rho_key,
                                                                                       slice_cols, metric);
   return cudaGetLastError();
 }

@@ -70,8 +70,8 @@ __device__ __forceinline__ void tsg_tile_next(const FrameTable& ft, int t, int& 
 // of head h stay in shared memory (128 KB); historical row tiles of 128
 // tokens stream through two 32 KB stages.  TMEM holds the 128 x 512 fp32
 // product as two 256-column accumulator stages; epilogue group g owns stage g
-// and writes slice 2*chunk+g of rho_part: max_j acc_ij * rn_j.  Columns past
-// the current frame carry rn = NaN, which fmaxf ignores.
+// and folds max_j acc_ij * rn_j over them into rho_key.  Columns past the
+// current frame carry rn = NaN, which fmaxf ignores.
 constexpr int kTsgB = 0;                  // [2][512][128 B]
 constexpr int kTsgAStages = 3;
 constexpr int kTsgA = 131072;                              // [3 stages][2][128][128 B]
@@ -86,7 +86,7 @@ constexpr int kTsgSmem = 232448;                           // the per-CTA maximu
 template <int METRIC>
 __global__ void __launch_bounds__(kThreads, 1)
     k_tsg_umma(const __grid_constant__ KMaps maps, const __grid_constant__ FrameTable ft,
-               Strided<const float> rc_all, int cur_pad, Strided<float> rho_all, int hkv, uint32_t* err) {
+               Strided<const float> rc_all, int cur_pad, Strided<uint32_t> rho_all, int hkv, uint32_t* err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = align1024(smem_raw);
   if ((int)(sm - smem_raw) + kTsgUsed > kTsgSmem) {  // uniform: the layout would not fit
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int chunk = blockIdx.y, l = blockIdx.z / hkv, h = blockIdx.z % hkv, n = ft.n_tokens;
   const CUtensorMap& kmap = maps.m[l];
   const float* rn_cur = rc_all.at(l) + (size_t)h * cur_pad;  // 16-byte aligned rows
-  float* rho_part = rho_all.at(l);
+  uint32_t* rho_key = rho_all.at(l) + (size_t)h * n;
   const int n_tiles = ft.tsg_tiles;
   const int col0 = chunk * 512;
   const int valid = min(512, ft.cur_len - col0);
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         int tok0, fend;
         tsg_tile_next(ft, t, tf, tok0, fend);
         const int tok = tok0 + quarter * 32 + lane;
-        if (tok < fend) rho_part[((size_t)(2 * chunk + g) * hkv + h) * n + tok] = mx;
+        if (tok < fend) atomicMax(rho_key + tok, float_key(mx));
       }
     }
   }
@@ -942,8 +942,7 @@ struct CssGeom {
 };
 
 struct CssDots {
-  Strided<float> rn, dE, dS, dSE, dSW, rn_cur;
-  int cur_pad;
+  Strided<float> dE, dS, dSE, dSW;
 };
 
 // Frame f and first token t0 of CSS tile t (the tiles of frame f are
@@ -957,7 +956,7 @@ __device__ __forceinline__ void css_tile_next(const FrameTable& ft, int t, int& 
 
 __global__ void __launch_bounds__(kThreads, 1)
     k_css_umma(const __grid_constant__ KMaps maps, const __grid_constant__ FrameTable ft, int hkv,
-               CssDots out, CssGeom geo, uint32_t* err) {
+               CssDots out, NormsOut norms, CssGeom geo, uint32_t* err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = align1024(smem_raw);
   const int S = geo.stages, SB = geo.stage_bytes, half_bytes = geo.cap_rows * 128;
@@ -1056,12 +1055,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int g = (warp - 2) >> 2, quarter = warp & 3;
     float* stg = reinterpret_cast<float*>(sm + off_stg) + (size_t)(warp - 2) * 32 * kCssStgRow + lane * kCssStgRow;
     const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + g * 256 + quarter * 32;
-    float* rn_o = out.rn.at(l) + (size_t)h * n;
+    float* rn_o = norms.rn.at(l) + (size_t)h * n;
+    uint32_t* rho_o = norms.rho_key.base ? norms.rho_key.at(l) + (size_t)h * n : nullptr;
     float* e_o = out.dE.at(l) + (size_t)h * n;
     float* s_o = out.dS.at(l) + (size_t)h * n;
     float* se_o = out.dSE.at(l) + (size_t)h * n;
     float* sw_o = out.dSW.at(l) + (size_t)h * n;
-    float* rc_o = out.rn_cur.at(l) + (size_t)h * out.cur_pad;
+    float* rc_o = norms.rn_cur.at(l) + (size_t)h * norms.cur_pad;
     int f = 0;
     for (int it = g; it < ntiles; it += 2) {
       const uint32_t ua = (uint32_t)(it >> 1);
@@ -1110,6 +1110,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (tok < ft.off[f] + ft.gh[f] * gw) {
         const float r = 1.0f / fmaxf(sqrtf(val[0]), 1e-8f);
         rn_o[tok] = r;
+        if (rho_o) rho_o[tok] = 0u;
         e_o[tok] = val[1];
         sw_o[tok] = val[2];
         s_o[tok] = val[3];
@@ -1133,7 +1134,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // are done once per run.  grid = (run block, frame, layer*Hkv + head).
 constexpr int kPhiRun = 4;
 __global__ void __launch_bounds__(256) k_css_phi(const __grid_constant__ FrameTable ft, int hkv, CssDots d,
-                                                 Strided<float> phi_all) {
+                                                 Strided<const float> rn_all, Strided<float> phi_all) {
   const int f = blockIdx.y, l = blockIdx.z / hkv, h = blockIdx.z % hkv, n = ft.n_tokens;
   if (f >= ft.n_frames) return;
   const int gh = ft.gh[f], gw = ft.gw[f], off = ft.off[f];
@@ -1142,7 +1143,7 @@ __global__ void __launch_bounds__(256) k_css_phi(const __grid_constant__ FrameTa
   if (slot >= gh * runs) return;
   const int u = slot / runs, v0 = (slot - u * runs) * kPhiRun;
   const size_t hn = (size_t)h * n;
-  const float* rn = d.rn.at(l) + hn;
+  const float* rn = rn_all.at(l) + hn;
   const float* e = d.dE.at(l) + hn;
   const float* s = d.dS.at(l) + hn;
   const float* se = d.dSE.at(l) + hn;
@@ -1361,7 +1362,7 @@ int score_nsplit_max(const Problem& p) {
 int score_nsplit(const Problem& p) { return score_nsplit_max(p); }
 
 cudaError_t launch_tsg_umma(const Problem& p, const FrameTable& ft, const LayerPtrs& io,
-                            Strided<const float> rn_cur, int cur_pad, Strided<float> rho_part, int metric,
+                            Strided<const float> rn_cur, int cur_pad, Strided<uint32_t> rho_key, int metric,
                             uint32_t* err, cudaStream_t st) {
   if (ft.n_frames < 2) return cudaSuccess;
   const int n_tiles = ft.tsg_tiles;
@@ -1377,7 +1378,7 @@ cudaError_t launch_tsg_umma(const Problem& p, const FrameTable& ft, const LayerP
   const int gx = pick_split(groups, n_tiles, sm_count());
   dim3 grid(gx, nchunk, p.L * p.hkv);
   TimingScope ts("tsg_umma", st);
-  kern<<<grid, kThreads, kTsgSmem, st>>>(local, ft, rn_cur, cur_pad, rho_part, p.hkv, err);
+  kern<<<grid, kThreads, kTsgSmem, st>>>(local, ft, rn_cur, cur_pad, rho_key, p.hkv, err);
   return cudaGetLastError();
 }
 
@@ -1428,9 +1429,8 @@ bool css_umma_supported(const FrameTable& ft) {
 }
 
 cudaError_t launch_css_umma(const Problem& p, const FrameTable& ft, const LayerPtrs& io, Strided<float> phi,
-                            Strided<float> rn, Strided<float> rn_cur, int cur_pad, Strided<float> dE,
-                            Strided<float> dS, Strided<float> dSE, Strided<float> dSW, uint32_t* err,
-                            cudaStream_t st, bool with_phi) {
+                            const NormsOut& norms, Strided<float> dE, Strided<float> dS, Strided<float> dSE,
+                            Strided<float> dSW, uint32_t* err, cudaStream_t st, bool with_phi) {
   const int tiles = ft.ctile0[ft.n_frames];
   if (tiles == 0) return cudaSuccess;
   KMaps maps;
@@ -1448,39 +1448,26 @@ cudaError_t launch_css_umma(const Problem& p, const FrameTable& ft, const LayerP
   if ((e = cudaFuncSetAttribute(k_css_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, geo.smem)) !=
       cudaSuccess)
     return e;
-  CssDots d;
-  d.rn = rn;
-  d.dE = dE;
-  d.dS = dS;
-  d.dSE = dSE;
-  d.dSW = dSW;
-  d.rn_cur = rn_cur;
-  d.cur_pad = cur_pad;
+  const CssDots d = {dE, dS, dSE, dSW};
   const int gx = pick_split(p.L * p.hkv, tiles, sm_count());
   {
     TimingScope ts("css_umma", st);
-    k_css_umma<<<dim3(gx, p.L * p.hkv), kThreads, geo.smem, st>>>(maps, ft, p.hkv, d, geo, err);
+    k_css_umma<<<dim3(gx, p.L * p.hkv), kThreads, geo.smem, st>>>(maps, ft, p.hkv, d, norms, geo, err);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  return with_phi ? launch_css_phi(p, ft, phi, rn, rn_cur, cur_pad, dE, dS, dSE, dSW, st) : cudaSuccess;
+  if (!with_phi) return cudaSuccess;
+  return launch_css_phi(p, ft, phi, strided<const float>(norms.rn.base, norms.rn.stride), dE, dS, dSE, dSW, st);
 }
 
-cudaError_t launch_css_phi(const Problem& p, const FrameTable& ft, Strided<float> phi, Strided<float> rn,
-                           Strided<float> rn_cur, int cur_pad, Strided<float> dE, Strided<float> dS,
-                           Strided<float> dSE, Strided<float> dSW, cudaStream_t st) {
+cudaError_t launch_css_phi(const Problem& p, const FrameTable& ft, Strided<float> phi, Strided<const float> rn,
+                           Strided<float> dE, Strided<float> dS, Strided<float> dSE, Strided<float> dSW,
+                           cudaStream_t st) {
   if (ft.ctile0[ft.n_frames] == 0) return cudaSuccess;
-  CssDots d;
-  d.rn = rn;
-  d.dE = dE;
-  d.dS = dS;
-  d.dSE = dSE;
-  d.dSW = dSW;
-  d.rn_cur = rn_cur;
-  d.cur_pad = cur_pad;
+  const CssDots d = {dE, dS, dSE, dSW};
   int cmax = 1;  // the most kPhiRun-cell runs of any frame
   for (int f = 0; f < ft.n_frames; ++f) cmax = max(cmax, ft.gh[f] * ((ft.gw[f] + kPhiRun - 1) / kPhiRun));
   TimingScope ts("css_phi", st);
-  k_css_phi<<<dim3((cmax + 255) / 256, ft.n_frames, p.L * p.hkv), 256, 0, st>>>(ft, p.hkv, d, phi);
+  k_css_phi<<<dim3((cmax + 255) / 256, ft.n_frames, p.L * p.hkv), 256, 0, st>>>(ft, p.hkv, d, rn, phi);
   return cudaGetLastError();
 }
 
