@@ -12,6 +12,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+from array import array
 
 import numpy as np
 import torch
@@ -72,7 +73,7 @@ class KernelTime(ctypes.Structure):
     _fields_ = [("name", ctypes.c_char * 32), ("launches", ctypes.c_int32), ("total_ms", ctypes.c_double)]
 
 
-_P = ctypes.c_void_p
+_P = ctypes.c_void_p  # also takes a plain address, which costs no object
 _S = ctypes.c_int32
 _sig = {
     "stlite_budget": (ctypes.c_int32, [ctypes.c_int32, ctypes.c_double, ctypes.c_int32]),
@@ -94,8 +95,7 @@ _sig = {
     "stlite_status_string": (ctypes.c_char_p, [ctypes.c_int32]),
     "stlite_score_noalloc": (_S, [ctypes.POINTER(Shape), _P, _P, _P, _P]),
     "stlite_compress_layers": (_S, [ctypes.POINTER(Shape), ctypes.POINTER(Frames), ctypes.POINTER(Params),
-                                    ctypes.c_int32, ctypes.POINTER(LayerIO), ctypes.POINTER(ctypes.c_int32), _P,
-                                    ctypes.c_size_t, _P]),
+                                    ctypes.c_int32, _P, ctypes.POINTER(ctypes.c_int32), _P, ctypes.c_size_t, _P]),
     "stlite_compress_varlen": (_S, [ctypes.POINTER(Shape), ctypes.c_int32, ctypes.POINTER(ctypes.c_int32),
                                     ctypes.POINTER(Frames), ctypes.POINTER(Params), _P, _P, _P, _P, _P, _P,
                                     ctypes.POINTER(ctypes.c_int32), _P, ctypes.c_size_t, _P]),
@@ -105,22 +105,20 @@ _sig = {
     "stlite_decode_attention": (_S, [ctypes.POINTER(Shape), _P, _P, _P, _P, _P, ctypes.c_size_t, _P]),
     "stlite_decode_workspace_size": (_S, [ctypes.POINTER(Shape), ctypes.POINTER(ctypes.c_size_t)]),
     "stlite_compress_layers_budgets": (_S, [ctypes.POINTER(Shape), ctypes.POINTER(Frames), ctypes.POINTER(Params),
-                                            ctypes.c_int32, ctypes.POINTER(LayerIO), ctypes.POINTER(ctypes.c_int32),
-                                            _P, ctypes.c_size_t, _P]),
+                                            ctypes.c_int32, _P, ctypes.POINTER(ctypes.c_int32), _P, ctypes.c_size_t,
+                                            _P]),
     "stlite_spatial_saliency_size": (_S, [ctypes.POINTER(Shape), ctypes.POINTER(Frames), _P, ctypes.c_int32, _P, _P,
                                           ctypes.c_size_t, _P]),
     "stlite_compress_varlen_layers": (_S, [ctypes.POINTER(Shape), ctypes.c_int32, ctypes.POINTER(ctypes.c_int32),
-                                           ctypes.POINTER(Frames), ctypes.POINTER(Params), ctypes.c_int32,
-                                           ctypes.POINTER(LayerIO), ctypes.POINTER(ctypes.c_int32), _P,
-                                           ctypes.c_size_t, _P]),
+                                           ctypes.POINTER(Frames), ctypes.POINTER(Params), ctypes.c_int32, _P,
+                                           ctypes.POINTER(ctypes.c_int32), _P, ctypes.c_size_t, _P]),
     "stlite_hierarchical_budgets": (_S, [ctypes.c_int32, ctypes.POINTER(ctypes.c_double), ctypes.c_int64,
                                          ctypes.c_int32, ctypes.POINTER(ctypes.c_int32)]),
     "stlite_prompt_score": (_S, [ctypes.POINTER(Shape), ctypes.c_int32, ctypes.c_int32, _P, _P, _P, _P,
                                  ctypes.c_size_t, _P]),
     "stlite_prompt_workspace_size": (_S, [ctypes.POINTER(Shape), ctypes.c_int32, ctypes.POINTER(ctypes.c_size_t)]),
     "stlite_selftest_wait_timeout": (_S, [_P, ctypes.c_int64, _P]),
-    "stlite_decode_attention_layers": (_S, [ctypes.POINTER(Shape), ctypes.c_int32, ctypes.POINTER(DecodeIO), _P,
-                                            ctypes.c_size_t, _P]),
+    "stlite_decode_attention_layers": (_S, [ctypes.POINTER(Shape), ctypes.c_int32, _P, _P, ctypes.c_size_t, _P]),
     "stlite_decode_layers_workspace_size": (_S, [ctypes.POINTER(Shape), ctypes.c_int32,
                                                  ctypes.POINTER(ctypes.c_size_t)]),
 }
@@ -142,13 +140,16 @@ def _check(status: int, where: str):
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
+
+
+_DTYPE = {torch.bfloat16: STLITE_BF16, torch.float32: STLITE_F32}
 
 
 def make_shape(q, k) -> Shape:
@@ -156,8 +157,23 @@ def make_shape(q, k) -> Shape:
     n, hkv, d2 = k.shape
     if d != d2:
         raise ValueError("q and k head_dim differ")
-    dt = {torch.bfloat16: STLITE_BF16, torch.float32: STLITE_F32}[k.dtype]
-    return Shape(n, hq, hkv, d, w, dt)
+    return Shape(n, hq, hkv, d, w, _DTYPE[k.dtype])
+
+
+def _layer_table(layers):
+    """The stlite_layer_io array of (q, k, v, k_out, v_out, idx_out) tuples."""
+    return array("Q", [p for q, k, v, ko, vo, ix in layers for p in (
+        q.data_ptr(), k.data_ptr(), v.data_ptr(), ko.data_ptr(), vo.data_ptr(), ix.data_ptr())])
+
+
+def _decode_table(layers):
+    """The stlite_decode_io array of (q, k, v, out) tuples."""
+    return array("Q", [p for q, k, v, o in layers for p in (
+        q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr())])
+
+
+def _address(table) -> int:
+    return table.buffer_info()[0]
 
 
 class FrameSpec:
@@ -268,10 +284,10 @@ def stlite_compress_layers(layers, frames, params, ws, stream=None) -> int:
     q0, k0 = layers[0][0], layers[0][1]
     sh = make_shape(q0, k0)
     fs = _frames(frames)
-    arr = (LayerIO * len(layers))(*[LayerIO(*(t.data_ptr() for t in lay)) for lay in layers])
+    arr = _layer_table(layers)
     b = ctypes.c_int32(0)
     _check(_lib.stlite_compress_layers(ctypes.byref(sh), ctypes.byref(fs.c), ctypes.byref(params), len(layers),
-                                       arr, ctypes.byref(b), _ptr(ws), ws.numel(), _stream(stream)),
+                                       _address(arr), ctypes.byref(b), _ptr(ws), ws.numel(), _stream(stream)),
            "stlite_compress_layers")
     return int(b.value)
 
@@ -283,10 +299,11 @@ def stlite_compress_layers_budgets(layers, frames, params, budgets, ws, stream=N
     q0, k0 = layers[0][0], layers[0][1]
     sh = make_shape(q0, k0)
     fs = _frames(frames)
-    arr = (LayerIO * len(layers))(*[LayerIO(*(t.data_ptr() for t in lay)) for lay in layers])
+    arr = _layer_table(layers)
     bud = (ctypes.c_int32 * len(layers))(*[int(b) for b in budgets])
     _check(_lib.stlite_compress_layers_budgets(ctypes.byref(sh), ctypes.byref(fs.c), ctypes.byref(params),
-                                               len(layers), arr, bud, _ptr(ws), ws.numel(), _stream(stream)),
+                                               len(layers), _address(arr), bud, _ptr(ws), ws.numel(),
+                                               _stream(stream)),
            "stlite_compress_layers_budgets")
 
 
@@ -344,12 +361,12 @@ def stlite_compress_varlen_layers(layers, cu_seqlens, frames_list, params, ws, s
     q0, k0 = layers[0][0], layers[0][1]
     sh = make_shape(q0[0] if q0.dim() == 4 else q0, k0)
     cu, specs, arr = _varlen_args(cu_seqlens, frames_list)
-    lio = (LayerIO * len(layers))(*[LayerIO(*(t.data_ptr() for t in lay)) for lay in layers])
+    lio = _layer_table(layers)
     cb = np.zeros(n_seqs + 1, dtype=np.int32)
     ip = ctypes.POINTER(ctypes.c_int32)
     _check(_lib.stlite_compress_varlen_layers(ctypes.byref(sh), n_seqs, cu.ctypes.data_as(ip), arr,
-                                              ctypes.byref(params), len(layers), lio, cb.ctypes.data_as(ip),
-                                              _ptr(ws), ws.numel(), _stream(stream)),
+                                              ctypes.byref(params), len(layers), _address(lio),
+                                              cb.ctypes.data_as(ip), _ptr(ws), ws.numel(), _stream(stream)),
            "stlite_compress_varlen_layers")
     return cb
 
@@ -383,8 +400,7 @@ def prompt_shape(q_prompt, k) -> Shape:
     n, hkv, d2 = k.shape
     if d != d2:
         raise ValueError("q and k head_dim differ")
-    dt = {torch.bfloat16: STLITE_BF16, torch.float32: STLITE_F32}[k.dtype]
-    return Shape(n, hq, hkv, d, 1, dt)
+    return Shape(n, hq, hkv, d, 1, _DTYPE[k.dtype])
 
 
 def stlite_prompt_workspace_size(shape: Shape, n_prompt: int) -> int:
@@ -422,8 +438,8 @@ def stlite_decode_attention_layers(layers, ws, stream=None):
     """layers: list of (q, k, v, out) device tensors, one tuple per layer
     (same shapes)."""
     sh = make_shape(layers[0][0], layers[0][1])
-    arr = (DecodeIO * len(layers))(*[DecodeIO(*(t.data_ptr() for t in lay)) for lay in layers])
-    _check(_lib.stlite_decode_attention_layers(ctypes.byref(sh), len(layers), arr, _ptr(ws), ws.numel(),
+    arr = _decode_table(layers)
+    _check(_lib.stlite_decode_attention_layers(ctypes.byref(sh), len(layers), _address(arr), _ptr(ws), ws.numel(),
                                                _stream(stream)), "stlite_decode_attention_layers")
 
 
