@@ -14,6 +14,8 @@
 // wait is bounded.
 #include <cudaTypedefs.h>
 
+#include <algorithm>
+
 #include "kernels.cuh"
 #include "ptx.cuh"
 
@@ -1298,25 +1300,26 @@ static int sm_count() {
   return c > 0 ? c : 148;
 }
 
-// CTAs per work unit (1..cap): one wave when the units are fewer than the
-// SMs, else the split among 1..4 that fills whole waves best.
-static int pick_split(int units, int cap, int slots) {
-  // Splits s of each unit so that units * s CTAs (one per SM) fill whole
-  // waves as nearly as possible; among equal fills the fewest CTAs win.
-  if (cap < 1) cap = 1;
+// CTAs per work unit (1..cap) for CTAs that take an SM each: the split whose
+// waves cost least, a CTA costing `fixed` tiles for its prologue (TMEM,
+// barriers, the resident operand, the first copies: 5-6 us) and its share of
+// the unit's tiles; among equals the fewest CTAs.  Many tiles per unit want
+// full waves (112 units of 419 tiles: 4 CTAs each, 2.95 waves); few want few
+// prologues (112 units of 17: one CTA each, 0.74 of a wave, instead of 2.95
+// waves of four or five tiles: row statistics 44 -> 31 us, column sums 33 ->
+// 25, CSS 28 -> 23; 56 units of 150: 5 CTAs each instead of 8, column sums 60
+// -> 55).
+static int pick_split(int units, int cap, int slots, int tiles, int fixed) {
   const int even = (slots + units - 1) / units;
-  int smax = 4 * even;
-  if (smax < 4) smax = 4;
-  if (smax > cap) smax = cap;
+  const int smax = std::min(std::max(cap, 1), std::max(4, 4 * even));
   int best = 1;
-  double best_eff = 0.0;
+  long long best_cost = 0;
   for (int s = 1; s <= smax; ++s) {
-    const long long ctas = (long long)units * s;
-    const long long waves = (ctas + slots - 1) / slots;
-    const double eff = (double)ctas / (double)(waves * slots);
-    if (eff > best_eff + 0.02) {
+    const long long waves = ((long long)units * s + slots - 1) / slots;
+    const long long cost = waves * (fixed + (tiles + s - 1) / s);
+    if (s == 1 || cost < best_cost) {
       best = s;
-      best_eff = eff;
+      best_cost = cost;
     }
   }
   return best;
@@ -1355,8 +1358,21 @@ int score_nsplit_max(const Problem& p) {
     if (per_t < 2) per_t = 2;
     return (tiles + per_t - 1) / per_t;
   }
-  int s = pick_split(p.hkv, tiles, 2 * 152);
-  return s < 1 ? 1 : s;
+  // fp32: the split of a head's tiles, at most four times what two CTAs per
+  // SM take, that fills whole waves of them best
+  const int slots = 2 * 152, even = (slots + p.hkv - 1) / p.hkv;
+  const int smax = std::min(tiles, std::max(4, 4 * even));
+  int best = 1;
+  double best_eff = 0.0;
+  for (int s = 1; s <= smax; ++s) {
+    const long long ctas = (long long)p.hkv * s, waves = (ctas + slots - 1) / slots;
+    const double eff = (double)ctas / (double)(waves * slots);
+    if (eff > best_eff + 0.02) {
+      best = s;
+      best_eff = eff;
+    }
+  }
+  return best;
 }
 
 int score_nsplit(const Problem& p) { return score_nsplit_max(p); }
@@ -1375,7 +1391,7 @@ cudaError_t launch_tsg_umma(const Problem& p, const FrameTable& ft, const LayerP
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTsgSmem);
   if (e != cudaSuccess) return e;
   const int groups = nchunk * p.L * p.hkv;
-  const int gx = pick_split(groups, n_tiles, sm_count());
+  const int gx = pick_split(groups, n_tiles, sm_count(), n_tiles, 3);
   dim3 grid(gx, nchunk, p.L * p.hkv);
   TimingScope ts("tsg_umma", st);
   kern<<<grid, kThreads, kTsgSmem, st>>>(local, ft, rn_cur, cur_pad, rho_key, p.hkv, err);
@@ -1403,7 +1419,7 @@ cudaError_t launch_score_umma(const Problem& p, const LayerPtrs& io, Strided<flo
     TimingScope ts("rowstats_umma", st);
     // CTAs per (layer, head, row half): whole waves for the batch, each
     // taking cps consecutive splits
-    const int cph0 = pick_split(p.L * p.hkv * L1.NMH, nsplit, sm_count());
+    const int cph0 = pick_split(p.L * p.hkv * L1.NMH, nsplit, sm_count(), score_tiles(p), 3);
     const int cps = (nsplit + cph0 - 1) / cph0;
     const int cph = (nsplit + cps - 1) / cps;
     rs_kernel<<<dim3(cph * L1.NMH, p.L * p.hkv), kScoreThreads, L1.total, st>>>(m1, io, p, nsplit, cps, rowpart,
@@ -1416,7 +1432,7 @@ cudaError_t launch_score_umma(const Problem& p, const LayerPtrs& io, Strided<flo
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int tiles = (p.n + 127) / 128;
-  const int gx = pick_split(p.L * p.hkv, tiles, sm_count());
+  const int gx = pick_split(p.L * p.hkv, tiles, sm_count(), tiles, 6);
   TimingScope ts("colsum_umma", st);
   cs_kernel<<<dim3(gx, p.L * p.hkv), kCsThreads, L2.total, st>>>(m2, io, p, rowpart, nsplit, a_base, err);
   return cudaGetLastError();
@@ -1449,7 +1465,7 @@ cudaError_t launch_css_umma(const Problem& p, const FrameTable& ft, const LayerP
       cudaSuccess)
     return e;
   const CssDots d = {dE, dS, dSE, dSW};
-  const int gx = pick_split(p.L * p.hkv, tiles, sm_count());
+  const int gx = pick_split(p.L * p.hkv, tiles, sm_count(), tiles, 6);
   {
     TimingScope ts("css_umma", st);
     k_css_umma<<<dim3(gx, p.L * p.hkv), kThreads, geo.smem, st>>>(maps, ft, p.hkv, d, norms, geo, err);
