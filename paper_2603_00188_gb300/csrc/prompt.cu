@@ -6,29 +6,42 @@
 //   C[j] = (1/G) sum_{g in group h} sum_{p >= j} softmax_{j' <= p}(q_{p,g} . k_{j',h} / sqrt(d))_j
 // full base A = C; Mean Attention A = C / #{prompt rows that attend to j}.
 //
-//   k_prompt_rowstats  pass 1: one CTA per 128-row m-tile of query rows
-//                      (P1 = floor(128 / G) whole positions, G rows each);
-//                      key tiles of 256 stream up to the tile's last
-//                      position; per row the running max and sum of
-//                      exponentials under the causal mask, merged over four
-//                      epilogue groups into bias_r = -m_r - log2(G l_r).
-//   k_prompt_colsum    pass 2: one CTA per 128-key tile, the tile resident
-//                      in shared memory as the A operand; chunks of P2 =
-//                      floor(256 / G) positions (G P2 rows) stream as the
-//                      B operand from the first chunk that can see the
-//                      tile; each key sums 2^(x c + bias_r) over the rows
-//                      that attend to it.  Every key's sum is formed in one
-//                      CTA, in a fixed order: no atomics, no reduction pass.
+//   k_prompt_rowstats  pass 1: persistent CTAs over the 128-row m-tiles of
+//                      query rows (P1 = floor(128 / G) whole positions, G rows
+//                      each), longest first; per m-tile key tiles of 256
+//                      stream up to its last position; per row the running
+//                      max and sum of exponentials under the causal mask,
+//                      merged over four epilogue groups into bias_r = -m_r -
+//                      log2(G l_r).
+//   k_prompt_colsum    pass 2: a cluster of CTAs per 128-key tile, the tile
+//                      resident in shared memory as the A operand; chunks of
+//                      P2 = floor(256 / G) positions (G P2 rows) stream as the
+//                      B operand from the first chunk that can see the tile,
+//                      the cluster's CTAs taking them in turn; each key sums
+//                      2^(x c + bias_r) over the rows that attend to it, and
+//                      the CTAs' sums are added in rank order: no atomics, no
+//                      reduction pass.
 //
 // Query rows come straight from q [nq][Hq][128] through a 3-D TMA box (d,
 // the group's G heads, positions): its lines land in shared memory in
 // (position, head) order, which is the row order r = position * G + g.
 // Same warp roles as the window-score passes: warp 0 TMA, warp 1 MMA, four
 // groups of four epilogue warps; every mbarrier wait is bounded.
+//
+// Both passes are bound by their epilogues (0.9 and 1.1 us per 128 x 256 item,
+// the MMA alone 0.66).  8,576 positions, 28 query heads (one layer), with one
+// CTA per m-tile and per key tile, the biases in the query rows' stages and a
+// kernel that filled the bias array first: 6 + 210 + 255 us; now 196 + 241.
+#include <cooperative_groups.h>
 #include <cudaTypedefs.h>
+
+#include <algorithm>
+#include <cmath>
 
 #include "kernels.cuh"
 #include "ptx.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace stl {
 
@@ -39,25 +52,29 @@ constexpr int kPrThreads = (2 + 4 * kPrGroups) * 32;
 constexpr int kPrMaxReg = 96;
 constexpr float kPrLog2e = 1.4426950408889634f;
 
-// pass 1: Q m-tile [2 halves][128 rows][128 B], two key stages of 256 keys
+// pass 1: two Q m-tiles [2 halves][128 rows][128 B] (the next one loads
+// while this one is worked on), two key stages of 256 keys
 constexpr int kP1Q = 0;
-constexpr int kP1K = 32768;
+constexpr int kP1K = 2 * 32768;
 constexpr int kP1KStage = 65536;
 constexpr int kP1Stages = 2;
-constexpr int kP1Bar = kP1K + kP1Stages * kP1KStage;  // 8 mbarriers, slot, abort
-constexpr int kP1Xch = kP1Bar + 128;                   // float2 [4 groups][128 rows]
-constexpr int kP1Smem = kP1Xch + kPrGroups * 128 * 8 + 1024;
+constexpr int kP1Bar = kP1K + kP1Stages * kP1KStage;  // 13 mbarriers, slot, abort
+constexpr int kP1Xch = kP1Bar + 128;                   // float2 [2][4 groups][128 rows]
+constexpr int kP1Smem = kP1Xch + 2 * kPrGroups * 128 * 8 + 1024;
 
 // pass 2: key tile [2 halves][128 keys][128 B], two Q stages of 256 rows,
-// the stages' row biases, the groups' partial sums
+// four stages of row biases, the groups' partial sums, the CTA's sums
 constexpr int kP2K = 0;
 constexpr int kP2Q = 32768;
 constexpr int kP2QStage = 65536;
 constexpr int kP2Stages = 2;
+constexpr int kP2BStages = 4;
 constexpr int kP2Bias = kP2Q + kP2Stages * kP2QStage;  // float [stages][256]
-constexpr int kP2Bar = kP2Bias + kP2Stages * 1024;
-constexpr int kP2Xch = kP2Bar + 128;                    // float [4 groups][128 keys]
-constexpr int kP2Smem = kP2Xch + kPrGroups * 128 * 4 + 1024;
+constexpr int kP2Bar = kP2Bias + kP2BStages * 1024;    // 18 mbarriers, slot, abort
+constexpr int kP2Xch = kP2Bar + 256;                    // float [4 groups][128 keys]
+constexpr int kP2Sum = kP2Xch + kPrGroups * 128 * 4;    // float [128 keys]
+constexpr int kP2Smem = kP2Sum + 128 * 4 + 1024;
+constexpr int kP2MaxSplit = 8;                          // CTAs per key tile (one cluster)
 
 __device__ __forceinline__ uint8_t* pr_align1024(uint8_t* p) {
   uint32_t a = smem_u32(p);
@@ -94,9 +111,13 @@ struct PromptArgs {
 
 // bias [Hkv][n_ch][crp]: entry of row (relative position pr, head g of the
 // group) at chunk pr / P2, offset (pr % P2) G + g; every other entry -inf.
-__global__ void k_prompt_bias_fill(float* bias, size_t count) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
-    bias[i] = -CUDART_INF_F;
+// Those others: the ends of the chunks' rows, and the last chunk's positions
+// past the prompt (a few values per chunk, shared out over the grid).
+__device__ __forceinline__ void prompt_bias_pad(const PromptArgs& a, float* bias) {
+  for (int c = blockIdx.x; c < a.hkv * a.n_ch; c += gridDim.x) {
+    const int real = a.G * min(a.p2, a.nq - c % a.n_ch * a.p2);
+    for (int i = real + threadIdx.x; i < a.crp; i += blockDim.x) bias[(size_t)c * a.crp + i] = -CUDART_INF_F;
+  }
 }
 
 __global__ void __maxnreg__(kPrMaxReg)
@@ -104,21 +125,19 @@ __global__ void __maxnreg__(kPrMaxReg)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = pr_align1024(smem_raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = blockIdx.x % a.hkv;
-  const int mt = a.n_mt - 1 - (int)(blockIdx.x / a.hkv);  // longest rows first
-  const int p_first = a.n - a.nq;
-  const int pr0 = mt * a.p1;                               // first relative position of the tile
-  const int npos = min(a.p1, a.nq - pr0);
-  const int rows = npos * a.G;
-  const int pa = p_first + pr0;                            // first absolute position
-  const int kend = pa + npos;                              // keys [0, kend) are visible to some row
-  const int ntiles = (kend + 255) / 256;
+  // work item i: KV head i % hkv, m-tile n_mt - 1 - i / hkv (longest rows
+  // first); CTA b takes items b, b + grid, ...  An item's rows are positions
+  // [pr0, pr0 + npos), its keys [0, p_first + pr0 + npos).
+  const int n_items = a.n_mt * a.hkv, p_first = a.n - a.nq;
+  auto item_pr0 = [&](int i) { return (a.n_mt - 1 - i / a.hkv) * a.p1; };
+  auto item_tiles = [&](int pr0) { return (p_first + pr0 + min(a.p1, a.nq - pr0) + 255) / 256; };
   const uint32_t sQ = smem_u32(sm + kP1Q), sK = smem_u32(sm + kP1K);
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kP1Bar);
   const uint32_t b_kfull = smem_u32(&bars[0]), b_kempty = smem_u32(&bars[kP1Stages]);
   const uint32_t b_accfull = smem_u32(&bars[2 * kP1Stages]), b_accempty = smem_u32(&bars[2 * kP1Stages + 2]);
-  const uint32_t b_q = smem_u32(&bars[2 * kP1Stages + 4]), b_done = smem_u32(&bars[2 * kP1Stages + 5]);
-  uint32_t* slot = reinterpret_cast<uint32_t*>(sm + kP1Bar + 8 * (2 * kP1Stages + 6));
+  const uint32_t b_qfull = smem_u32(&bars[2 * kP1Stages + 4]), b_qempty = smem_u32(&bars[2 * kP1Stages + 6]);
+  const uint32_t b_done = smem_u32(&bars[2 * kP1Stages + 8]);
+  uint32_t* slot = reinterpret_cast<uint32_t*>(sm + kP1Bar + 8 * (2 * kP1Stages + 9));
   volatile uint32_t* abort_flag = slot + 1;
   float2* xch = reinterpret_cast<float2*>(sm + kP1Xch);
   const float c = kPrLog2e * rsqrtf((float)kD);
@@ -131,8 +150,9 @@ __global__ void __maxnreg__(kPrMaxReg)
     for (int i = 0; i < 2; ++i) {
       mbar_init(b_accfull + 8 * i, 1);
       mbar_init(b_accempty + 8 * i, 4 * kPrGroups);
+      mbar_init(b_qfull + 8 * i, 1);
+      mbar_init(b_qempty + 8 * i, 1);
     }
-    mbar_init(b_q, 1);
     mbar_init(b_done, 1);
     *abort_flag = 0u;
     fence_mbar_init();
@@ -143,6 +163,7 @@ __global__ void __maxnreg__(kPrMaxReg)
     tmem_alloc(smem_u32(slot), 512);
     tmem_relinquish();
   }
+  prompt_bias_pad(a, bias);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -150,23 +171,33 @@ __global__ void __maxnreg__(kPrMaxReg)
 
   if (warp == 0) {
     if (lane == 0) {
-      // the m-tile's rows: positions [pr0, pr0 + P1) of the group's G heads
+      // an item's rows: positions [pr0, pr0 + P1) of the group's G heads
       const uint32_t qbytes = 2u * 128u * (uint32_t)(a.G * a.p1);
-      mbar_arrive_expect_tx(b_q, qbytes);
-      tma_load_3d(sQ, &maps.q1, b_q, 0, h * a.G, pr0);
-      tma_load_3d(sQ + 16384, &maps.q1, b_q, 64, h * a.G, pr0);
-      int issued[kP1Stages] = {0, 0};
-      int ks = 0;
+      int issued[kP1Stages] = {0, 0}, q_issued[2] = {0, 0};
+      int ks = 0, qi = 0;  // key stage; items so far
       uint32_t kp = 0u;
-      for (int it = 0; it < ntiles; ++it, ks = ks + 1 == kP1Stages ? 0 : ks + 1, kp += ks == 0 ? 1u : 0u) {
-        if (!mbar_wait(b_kempty + 8 * ks, (kp & 1u) ^ 1u, err, abort_flag)) break;
-        mbar_arrive_expect_tx(b_kfull + 8 * ks, (uint32_t)kP1KStage);
-        tma_load_3d(sK + ks * kP1KStage, &maps.k1, b_kfull + 8 * ks, 0, h, it * 256);
-        tma_load_3d(sK + ks * kP1KStage + 32768, &maps.k1, b_kfull + 8 * ks, 64, h, it * 256);
-        ++issued[ks];
+      bool ok = true;
+      for (int i = blockIdx.x; ok && i < n_items; i += gridDim.x, ++qi) {
+        const int qs = qi & 1, h = i % a.hkv, pr0 = item_pr0(i), ntiles = item_tiles(pr0);
+        if (!mbar_wait(b_qempty + 8 * qs, ((uint32_t)(qi >> 1) & 1u) ^ 1u, err, abort_flag)) break;
+        mbar_arrive_expect_tx(b_qfull + 8 * qs, qbytes);
+        tma_load_3d(sQ + qs * 32768, &maps.q1, b_qfull + 8 * qs, 0, h * a.G, pr0);
+        tma_load_3d(sQ + qs * 32768 + 16384, &maps.q1, b_qfull + 8 * qs, 64, h * a.G, pr0);
+        ++q_issued[qs];
+        for (int it = 0; it < ntiles; ++it, ks = ks + 1 == kP1Stages ? 0 : ks + 1, kp += ks == 0 ? 1u : 0u) {
+          if (!mbar_wait(b_kempty + 8 * ks, (kp & 1u) ^ 1u, err, abort_flag)) {
+            ok = false;
+            break;
+          }
+          mbar_arrive_expect_tx(b_kfull + 8 * ks, (uint32_t)kP1KStage);
+          tma_load_3d(sK + ks * kP1KStage, &maps.k1, b_kfull + 8 * ks, 0, h, it * 256);
+          tma_load_3d(sK + ks * kP1KStage + 32768, &maps.k1, b_kfull + 8 * ks, 64, h, it * 256);
+          ++issued[ks];
+        }
       }
       if (*abort_flag) {
-        mbar_wait_drain(b_q, 0);
+        for (int s = 0; s < 2; ++s)
+          if (q_issued[s]) mbar_wait_drain(b_qfull + 8 * s, (uint32_t)(q_issued[s] - 1) & 1u);
         for (int s = 0; s < kP1Stages; ++s)
           if (issued[s]) mbar_wait_drain(b_kfull + 8 * s, (uint32_t)(issued[s] - 1) & 1u);
       }
@@ -174,37 +205,53 @@ __global__ void __maxnreg__(kPrMaxReg)
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16(128, 256);
-      bool ok = mbar_wait(b_q, 0, err, abort_flag);
-      int ks = 0;
+      bool ok = true;
+      int ks = 0, qi = 0, u = 0;  // key stage; items, key tiles so far
       uint32_t kp = 0u;
-      for (int it = 0; ok && it < ntiles; ++it, ks = ks + 1 == kP1Stages ? 0 : ks + 1, kp += ks == 0 ? 1u : 0u) {
-        if (!mbar_wait(b_kfull + 8 * ks, kp & 1u, err, abort_flag)) break;
-        const int as = it & 1;
-        if (!mbar_wait(b_accempty + 8 * as, ((uint32_t)(it >> 1) & 1u) ^ 1u, err, abort_flag)) break;
-        tc_fence_after();
+      for (int i = blockIdx.x; ok && i < n_items; i += gridDim.x, ++qi) {
+        const int qs = qi & 1, ntiles = item_tiles(item_pr0(i));
+        if (!mbar_wait(b_qfull + 8 * qs, (uint32_t)(qi >> 1) & 1u, err, abort_flag)) break;
+        for (int it = 0; it < ntiles;
+             ++it, ++u, ks = ks + 1 == kP1Stages ? 0 : ks + 1, kp += ks == 0 ? 1u : 0u) {
+          const int as = u & 1;
+          if (!mbar_wait(b_kfull + 8 * ks, kp & 1u, err, abort_flag) ||
+              !mbar_wait(b_accempty + 8 * as, ((uint32_t)(u >> 1) & 1u) ^ 1u, err, abort_flag)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const uint32_t kb = k >> 2, koff = (k & 3) * 32;
-          const uint64_t ad = desc_sw128(sQ + kb * 16384 + koff);
-          const uint64_t bd = desc_sw128(sK + ks * kP1KStage + kb * 32768 + koff);
-          umma_bf16(tmem + as * 256, ad, bd, idesc, k > 0 ? 1u : 0u);
+          for (int k = 0; k < 8; ++k) {
+            const uint32_t kb = k >> 2, koff = (k & 3) * 32;
+            const uint64_t ad = desc_sw128(sQ + qs * 32768 + kb * 16384 + koff);
+            const uint64_t bd = desc_sw128(sK + ks * kP1KStage + kb * 32768 + koff);
+            umma_bf16(tmem + as * 256, ad, bd, idesc, k > 0 ? 1u : 0u);
+          }
+          umma_commit(b_accfull + 8 * as);
+          umma_commit(b_kempty + 8 * ks);
         }
-        umma_commit(b_accfull + 8 * as);
-        umma_commit(b_kempty + 8 * ks);
+        if (ok) umma_commit(b_qempty + 8 * qs);
       }
       umma_commit(b_done);
       mbar_wait_drain(b_done, 0);
     }
   } else {
-    // group g drains key columns [64 g, 64 g + 64) of every item; the
+    // group g drains key columns [64 g, 64 g + 64) of every key tile; the
     // thread owns query row `row` (TMEM lane) at absolute position pos
     const int g = (warp - 2) >> 2, quarter = warp & 3, row = quarter * 32 + lane;
-    const int pos = pa + row / a.G;
     const uint32_t lanebase = tmem + ((uint32_t)(quarter * 32) << 16) + g * 64;
+    bool live = true;  // after a wait gave up every warp still meets the others at each item's end
+    int u = 0, xb = 0;
+    for (int i = blockIdx.x; i < n_items; i += gridDim.x, xb ^= 1) {
+    const int h = i % a.hkv, pr0 = item_pr0(i), ntiles = item_tiles(pr0);
+    const int pa = p_first + pr0, rows = min(a.p1, a.nq - pr0) * a.G, pos = pa + row / a.G;
     float m = -CUDART_INF_F, l = 0.f;
-    for (int it = 0; it < ntiles; ++it) {
-      const int as = it & 1;
-      if (!warp_wait(b_accfull + 8 * as, (uint32_t)(it >> 1) & 1u, err, abort_flag)) break;
+    for (int it = 0; live && it < ntiles; ++it, ++u) {
+      const int as = u & 1;
+      if (!warp_wait(b_accfull + 8 * as, (uint32_t)(u >> 1) & 1u, err, abort_flag)) {
+        live = false;
+        break;
+      }
       tc_fence_after();
       float v[64];
       tmem_ld64(lanebase + as * 256, v);
@@ -258,13 +305,15 @@ __global__ void __maxnreg__(kPrMaxReg)
         }
       }
     }
-    // merge the four groups' states per row in group order
-    xch[g * 128 + row] = make_float2(m, l);
+    // merge the four groups' states per row in group order (two exchange
+    // buffers in turn: one is rewritten after the other's barrier)
+    float2* xp = xch + xb * kPrGroups * 128;
+    xp[g * 128 + row] = make_float2(m, l);
     epilogue_sync();
-    if (g == 0 && row < rows && !*abort_flag) {
-      float mm = xch[row].x, ll = xch[row].y;
+    if (g == 0 && row < rows && live && !*abort_flag) {
+      float mm = xp[row].x, ll = xp[row].y;
       for (int o = 1; o < kPrGroups; ++o) {
-        const float2 s = xch[o * 128 + row];
+        const float2 s = xp[o * 128 + row];
         const float mn = fmaxf(mm, s.x);
         if (mn == -CUDART_INF_F) continue;
         const float x = mm == -CUDART_INF_F ? 0.f : ll * exp2f((mm - mn) * c);
@@ -275,6 +324,7 @@ __global__ void __maxnreg__(kPrMaxReg)
       const int prel = pr0 + row / a.G, gq = row - (row / a.G) * a.G;
       const size_t at = ((size_t)h * a.n_ch + prel / a.p2) * a.crp + (size_t)(prel % a.p2) * a.G + gq;
       bias[at] = -mm * c - log2f((float)a.G * ll);
+    }
     }
   }
   tc_fence_before();
@@ -291,20 +341,27 @@ __global__ void __maxnreg__(kPrMaxReg)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = pr_align1024(smem_raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = blockIdx.x % a.hkv, kt = blockIdx.x / a.hkv;  // keys seen by the most rows first
+  // a cluster of `split` CTAs per key tile: rank r takes every split-th chunk
+  // (keys seen by the most rows first)
+  cg::cluster_group cl = cg::this_cluster();
+  const int split = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int unit = blockIdx.x / split, h = unit % a.hkv, kt = unit / a.hkv;
   const int j0 = kt * 128;
   const int p_first = a.n - a.nq;
-  const int cstart = j0 <= p_first ? 0 : (j0 - p_first) / a.p2;
-  const int nitems = a.n_ch - cstart;
+  const int cstart = (j0 <= p_first ? 0 : (j0 - p_first) / a.p2) + rank;
+  const int nitems = cstart < a.n_ch ? (a.n_ch - cstart + split - 1) / split : 0;
   const uint32_t sK = smem_u32(sm + kP2K), sQ = smem_u32(sm + kP2Q);
   float* bias_s = reinterpret_cast<float*>(sm + kP2Bias);
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kP2Bar);
   const uint32_t b_qfull = smem_u32(&bars[0]), b_qempty = smem_u32(&bars[kP2Stages]);
   const uint32_t b_accfull = smem_u32(&bars[2 * kP2Stages]), b_accempty = smem_u32(&bars[2 * kP2Stages + 2]);
   const uint32_t b_k = smem_u32(&bars[2 * kP2Stages + 4]), b_done = smem_u32(&bars[2 * kP2Stages + 5]);
-  uint32_t* slot = reinterpret_cast<uint32_t*>(sm + kP2Bar + 8 * (2 * kP2Stages + 6));
+  const uint32_t b_bfull = smem_u32(&bars[2 * kP2Stages + 6]);
+  const uint32_t b_bempty = smem_u32(&bars[2 * kP2Stages + 6 + kP2BStages]);
+  uint32_t* slot = reinterpret_cast<uint32_t*>(sm + kP2Bar + 8 * (2 * kP2Stages + 6 + 2 * kP2BStages));
   volatile uint32_t* abort_flag = slot + 1;
   float* xch = reinterpret_cast<float*>(sm + kP2Xch);
+  float* sum_s = reinterpret_cast<float*>(sm + kP2Sum);
   const float c = kPrLog2e * rsqrtf((float)kD);
   const int qrows = a.G * a.p2;  // real lines of a chunk; lines up to 256 stay zero
 
@@ -315,13 +372,19 @@ __global__ void __maxnreg__(kPrMaxReg)
     const int s = e / (2 * per_half), rem = e % (2 * per_half), kb = rem / per_half, w = rem % per_half;
     *reinterpret_cast<uint4*>(sm + kP2Q + s * kP2QStage + kb * 32768 + qrows * 128 + w * 16) = make_uint4(0, 0, 0, 0);
   }
-  for (int e = threadIdx.x; e < kP2Stages * 256; e += blockDim.x)
+  for (int e = threadIdx.x; e < kP2BStages * 256; e += blockDim.x)
     if ((e & 255) >= a.crp) bias_s[e] = -CUDART_INF_F;
   fence_proxy_async_smem();
   if (threadIdx.x == 0) {
     for (int i = 0; i < kP2Stages; ++i) {
       mbar_init(b_qfull + 8 * i, 1);
-      mbar_init(b_qempty + 8 * i, 1 + 4 * kPrGroups);  // the MMA's commit and every epilogue warp (bias)
+      mbar_init(b_qempty + 8 * i, 1);
+    }
+    // the biases have a ring of their own: the query rows' stage is free as
+    // soon as its MMA is done, not when the epilogue has read its biases
+    for (int i = 0; i < kP2BStages; ++i) {
+      mbar_init(b_bfull + 8 * i, 1);
+      mbar_init(b_bempty + 8 * i, 4 * kPrGroups);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(b_accfull + 8 * i, 1);
@@ -349,24 +412,28 @@ __global__ void __maxnreg__(kPrMaxReg)
       mbar_arrive_expect_tx(b_k, 32768u);
       tma_load_3d(sK, &maps.k2, b_k, 0, h, j0);
       tma_load_3d(sK + 16384, &maps.k2, b_k, 64, h, j0);
-      const uint32_t qbytes = 2u * 128u * (uint32_t)qrows + 4u * (uint32_t)a.crp;
-      int issued[kP2Stages] = {0, 0};
+      const uint32_t qbytes = 2u * 128u * (uint32_t)qrows, bbytes = 4u * (uint32_t)a.crp;
+      int issued[kP2Stages] = {0, 0}, b_issued[kP2BStages] = {0, 0, 0, 0};
       int ks = 0;
       uint32_t kp = 0u;
       for (int it = 0; it < nitems; ++it, ks = ks + 1 == kP2Stages ? 0 : ks + 1, kp += ks == 0 ? 1u : 0u) {
         if (!mbar_wait(b_qempty + 8 * ks, (kp & 1u) ^ 1u, err, abort_flag)) break;
-        const int ch = cstart + it;
+        const int ch = cstart + it * split, bs = it % kP2BStages;
         mbar_arrive_expect_tx(b_qfull + 8 * ks, qbytes);
         tma_load_3d(sQ + ks * kP2QStage, &maps.q2, b_qfull + 8 * ks, 0, h * a.G, ch * a.p2);
         tma_load_3d(sQ + ks * kP2QStage + 32768, &maps.q2, b_qfull + 8 * ks, 64, h * a.G, ch * a.p2);
-        bulk_g2s(smem_u32(bias_s + ks * 256), bias_h + (size_t)ch * a.crp, 4u * (uint32_t)a.crp,
-                 b_qfull + 8 * ks);
         ++issued[ks];
+        if (!mbar_wait(b_bempty + 8 * bs, ((uint32_t)(it / kP2BStages) & 1u) ^ 1u, err, abort_flag)) break;
+        mbar_arrive_expect_tx(b_bfull + 8 * bs, bbytes);
+        bulk_g2s(smem_u32(bias_s + bs * 256), bias_h + (size_t)ch * a.crp, bbytes, b_bfull + 8 * bs);
+        ++b_issued[bs];
       }
       if (*abort_flag) {
         mbar_wait_drain(b_k, 0);
         for (int s = 0; s < kP2Stages; ++s)
           if (issued[s]) mbar_wait_drain(b_qfull + 8 * s, (uint32_t)(issued[s] - 1) & 1u);
+        for (int s = 0; s < kP2BStages; ++s)
+          if (b_issued[s]) mbar_wait_drain(b_bfull + 8 * s, (uint32_t)(b_issued[s] - 1) & 1u);
       }
     }
   } else if (warp == 1) {
@@ -402,9 +469,8 @@ __global__ void __maxnreg__(kPrMaxReg)
     const int j = j0 + row;
     const uint32_t lanebase = tmem + ((uint32_t)(quarter * 32) << 16) + g * 64;
     float sum = 0.f, comp = 0.f;  // compensated running total over the items
-    int ks = 0;
-    for (int it = 0; it < nitems; ++it, ks = ks + 1 == kP2Stages ? 0 : ks + 1) {
-      const int as = it & 1;
+    for (int it = 0; it < nitems; ++it) {
+      const int as = it & 1, bs = it % kP2BStages;
       if (!warp_wait(b_accfull + 8 * as, (uint32_t)(it >> 1) & 1u, err, abort_flag)) break;
       tc_fence_after();
       float v[64];
@@ -412,8 +478,9 @@ __global__ void __maxnreg__(kPrMaxReg)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(b_accempty + 8 * as);
-      const float4* b4 = reinterpret_cast<const float4*>(bias_s + ks * 256 + g * 64);
-      const int p0 = p_first + (cstart + it) * a.p2;
+      if (!warp_wait(b_bfull + 8 * bs, (uint32_t)(it / kP2BStages) & 1u, err, abort_flag)) break;
+      const float4* b4 = reinterpret_cast<const float4*>(bias_s + bs * 256 + g * 64);
+      const int p0 = p_first + (cstart + it * split) * a.p2;
       float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
       if (p0 >= j0 + 127) {
         // every row of the chunk sees every key of the tile: exponent
@@ -442,9 +509,9 @@ __global__ void __maxnreg__(kPrMaxReg)
           s3 += 4 * i + 3 >= colmin ? ex2_approx(fmaf(v[4 * i + 3], c, b.w)) : 0.f;
         }
       }
-      // this stage's biases are read: count the warp out of the stage
+      // this stage's biases are read: count the warp out of it
       __syncwarp();
-      if (lane == 0) mbar_arrive(b_qempty + 8 * ks);
+      if (lane == 0) mbar_arrive(b_bempty + 8 * bs);
       const float y = ((s0 + s1) + (s2 + s3)) - comp;
       const float t = sum + y;
       comp = (t - sum) - y;
@@ -452,11 +519,7 @@ __global__ void __maxnreg__(kPrMaxReg)
     }
     xch[g * 128 + row] = sum;
     epilogue_sync();
-    if (g == 0 && j < a.n && !*abort_flag) {
-      float acc = (xch[row] + xch[128 + row]) + (xch[256 + row] + xch[384 + row]);
-      if (a.mode == 1) acc /= (float)min(a.nq, a.n - j);
-      a_out[(size_t)h * a.n + j] = acc;
-    }
+    if (g == 0) sum_s[row] = (xch[row] + xch[128 + row]) + (xch[256 + row] + xch[384 + row]);
   }
   tc_fence_before();
   __syncthreads();
@@ -464,6 +527,20 @@ __global__ void __maxnreg__(kPrMaxReg)
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
+  // the cluster's sums in rank order (after a wait gave up, the keys stay unwritten)
+  if (split > 1) cl.sync();
+  if (rank == 0 && threadIdx.x < 128 && j0 + (int)threadIdx.x < a.n) {
+    const int j = j0 + threadIdx.x;
+    float acc = sum_s[threadIdx.x];
+    bool whole = !*abort_flag;
+    for (int r = 1; r < split; ++r) {
+      acc += cl.map_shared_rank(sum_s, r)[threadIdx.x];
+      whole = whole && !*cl.map_shared_rank(slot + 1, r);
+    }
+    if (a.mode == 1) acc /= (float)min(a.nq, a.n - j);
+    if (whole) a_out[(size_t)h * a.n + j] = acc;
+  }
+  if (split > 1) cl.sync();  // no CTA leaves while rank 0 may still read its sums
 }
 
 // ---- fp32 caches: the same two passes on the CUDA cores --------------------
@@ -633,6 +710,30 @@ PromptArgs prompt_args(int n, int nq, int hq, int hkv, int mode) {
 
 }  // namespace
 
+// CTAs per key tile of pass 2.  A tile's chunks cannot be shared between
+// waves, so the pass ends with the CTA of the most chunks (the first keys'
+// tiles: every chunk) or, with many tiles, when the SMs have worked off all of
+// them: about total / SMs + longest / 2 chunks, plus 6 per CTA an SM runs.
+static int prompt_split(const PromptArgs& a, int nsm) {
+  const long long tiles = (a.n + 127) / 128;
+  long long chunks = 0;
+  for (long long t = 0; t < tiles; ++t) {
+    const long long j0 = t * 128, pf = a.n - a.nq;
+    chunks += a.n_ch - (j0 <= pf ? 0 : (j0 - pf) / a.p2);
+  }
+  int best = 1;
+  double best_cost = 0.0;
+  for (int s = 1; s <= kP2MaxSplit && s <= std::max(1, a.n_ch); s <<= 1) {
+    const double ctas = (double)tiles * a.hkv * s, longest = (double)a.n_ch / s;
+    const double cost = std::max((double)chunks * a.hkv / nsm + longest / 2, longest) + 6.0 * std::ceil(ctas / nsm);
+    if (s == 1 || cost < best_cost) {
+      best = s;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
 size_t prompt_bias_bytes(int n, int nq, int hq, int hkv) {
   const PromptArgs a = prompt_args(n, nq, hq, hkv, 0);
   return (size_t)hkv * a.n_ch * a.crp * 4;
@@ -643,14 +744,7 @@ cudaError_t launch_prompt_score(DType dt, const void* q, const void* k, int n, i
   const PromptArgs a = prompt_args(n, nq, hq, hkv, mode);
   if (a.p1 < 1) return cudaErrorNotSupported;
   if (dt == kF32) {
-    const size_t nbias = (size_t)hkv * a.n_ch * a.crp;
-    const size_t blocks = (nbias + 255) / 256;
     cudaError_t e;
-    {
-      TimingScope ts("prompt_bias_fill", st);
-      k_prompt_bias_fill<<<(unsigned)(blocks < 1024 ? blocks : 1024), 256, 0, st>>>(bias, nbias);
-    }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const float* qf = static_cast<const float*>(q);
     const float* kf = static_cast<const float*>(k);
     {
@@ -676,20 +770,28 @@ cudaError_t launch_prompt_score(DType dt, const void* q, const void* k, int n, i
   if ((e = cudaFuncSetAttribute(k_prompt_colsum, cudaFuncAttributeMaxDynamicSharedMemorySize, kP2Smem)) !=
       cudaSuccess)
     return e;
-  const size_t nbias = (size_t)hkv * a.n_ch * a.crp;
-  {
-    TimingScope ts("prompt_bias_fill", st);
-    const size_t blocks = (nbias + 255) / 256;
-    k_prompt_bias_fill<<<(unsigned)(blocks < 1024 ? blocks : 1024), 256, 0, st>>>(bias, nbias);
-  }
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  int nsm = 0, dev = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   {
     TimingScope ts("prompt_rowstats", st);
-    k_prompt_rowstats<<<(unsigned)(a.n_mt * hkv), kPrThreads, kP1Smem, st>>>(maps, a, bias, err);
+    k_prompt_rowstats<<<(unsigned)std::min(nsm, a.n_mt * hkv), kPrThreads, kP1Smem, st>>>(maps, a, bias, err);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  const int split = prompt_split(a, nsm);
+  cfg.gridDim = dim3((unsigned)((n + 127) / 128 * hkv * split));
+  cfg.blockDim = dim3(kPrThreads);
+  cfg.dynamicSmemBytes = kP2Smem;
+  cfg.stream = st;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)split;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
   TimingScope ts("prompt_colsum", st);
-  k_prompt_colsum<<<(unsigned)(((n + 127) / 128) * hkv), kPrThreads, kP2Smem, st>>>(maps, a, bias, a_out, err);
+  if ((e = cudaLaunchKernelEx(&cfg, k_prompt_colsum, maps, a, (const float*)bias, a_out, err)) != cudaSuccess) return e;
   return cudaGetLastError();
 }
 

@@ -163,3 +163,21 @@ def test_prompt_full_size_bench_layer(st):
     ora = oracle.prompt_abase(exact64(qp[n - tail:]), exact64(k), oracle.PROMPT_FULL, threads=oracle.host_threads())
     for h in range(H):
         assert_within(f[h, n - tail:], ora[h, n - tail:], a_bound(ora[h, n - tail:]), "full base, last keys, head %d" % h)
+
+
+@pytest.mark.parametrize("n,n_prompt,hq,hkv", [(130, 130, 5, 1), (1500, 1500, 10, 2), (1500, 40, 10, 2),
+                                               (2500, 2500, 8, 8), (700, 700, 384, 3), (129, 1, 7, 7)])
+def test_prompt_splits_and_pads(st, n, n_prompt, hq, hkv):
+    # one to eight CTAs per key tile (some without a chunk), m-tiles that follow
+    # one another in a CTA, chunks whose rows end short of 256 or of a multiple
+    # of four (G = 5, 128), a one-row prompt
+    gen = torch.Generator().manual_seed(n + hq)
+    q = torch.randn((n_prompt, hq, 128), generator=gen).to(torch.bfloat16).cuda()
+    k = torch.randn((n, hkv, 128), generator=gen).to(torch.bfloat16).cuda()
+    for base, mode in ((st.STLITE_PROMPT_FULL, oracle.PROMPT_FULL), (st.STLITE_PROMPT_MEAN, oracle.PROMPT_MEAN)):
+        a, ws = st.prompt_score(q, k, base)
+        torch.cuda.synchronize()
+        ora = oracle.prompt_abase(exact64(q), exact64(k), mode, threads=oracle.host_threads())
+        for h in range(hkv):
+            assert_within(a[h].cpu().numpy(), ora[h], a_bound(ora[h]), "head %d" % h)
+        assert st.stlite_device_status(ws) == st.STLITE_OK
