@@ -87,6 +87,13 @@ __device__ __forceinline__ bool mbar_wait_drain(uint32_t bar, uint32_t parity) {
   return true;
 }
 
+// 16-byte asynchronous copy global -> shared (both addresses 16-byte aligned),
+// and the wait for all of this thread's.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // ------------------------------------------------------------------ TMA
 // 3-D tiled load into this CTA's shared memory, completing on `bar` with the
 // box's byte count.  The innermost coordinate c0 is a multiple of 64 elements

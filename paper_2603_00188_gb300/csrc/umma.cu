@@ -36,19 +36,24 @@ struct KMaps {
 
 // Q rows [r0, r0 + rows) of KV head h into shared memory in the K-major
 // 128B-swizzle layout [2 K-halves][rows][128 B]; query row r = window row *
-// G + group member; rows past R are zero.
+// G + group member; rows past R are zero.  Asynchronous copies, all of them in
+// flight together (a thread has six to eight): one memory latency instead of
+// one per load.
 __device__ __forceinline__ void load_q_sw128(uint8_t* sq, int rows, const __nv_bfloat16* q,
                                              const Problem& p, int h, int r0 = 0) {
   const int G = p.G(), R = p.R();
+  const uint32_t base = smem_u32(sq);
   for (int e = threadIdx.x; e < rows * 16; e += blockDim.x) {
-    int row = e >> 4, c16 = e & 15, kb = c16 >> 3, cc = c16 & 7;
-    uint4 val = make_uint4(0, 0, 0, 0);
+    const int row = e >> 4, c16 = e & 15, kb = c16 >> 3, cc = c16 & 7;
+    const uint32_t off = (uint32_t)kb * rows * 128 + row * 128 + ((cc ^ (row & 7)) << 4);
     if (r0 + row < R) {
-      int wr = (r0 + row) / G, g = (r0 + row) - wr * G;
-      val = __ldg(reinterpret_cast<const uint4*>(q + ((size_t)wr * p.hq + h * G + g) * kD + c16 * 8));
+      const int wr = (r0 + row) / G, g = (r0 + row) - wr * G;
+      cp_async16(base + off, q + ((size_t)wr * p.hq + h * G + g) * kD + c16 * 8);
+    } else {
+      *reinterpret_cast<uint4*>(sq + off) = make_uint4(0, 0, 0, 0);
     }
-    *reinterpret_cast<uint4*>(sq + (size_t)kb * rows * 128 + row * 128 + ((cc ^ (row & 7)) << 4)) = val;
   }
+  cp_async_wait_all();
   fence_proxy_async_smem();
 }
 
@@ -413,6 +418,14 @@ __global__ void __maxnreg__(kScoreMaxReg)
   uint32_t* xcnt = reinterpret_cast<uint32_t*>(sm + L.off_xch + kRsXBuf * kScoreGroups * MT * 128 * 8);
   const float c = kLog2eF * rsqrtf((float)kD);
 
+  int early = 0;  // key tiles loaded before the setup barrier (thread 0)
+  auto load_k = [&](int it, int s) {
+    const int tok = j0 + it * KN;
+    mbar_arrive_expect_tx(b_kfull + 8 * s, (uint32_t)L.k_stage_bytes);
+    tma_load_3d(sK + s * L.k_stage_bytes, &kmap, b_kfull + 8 * s, 0, h, tok);
+    tma_load_3d(sK + s * L.k_stage_bytes + KN * 128, &kmap, b_kfull + 8 * s, 64, h, tok);
+  };
+
   if (threadIdx.x == 0) {
     for (int i = 0; i < S; ++i) {
       mbar_init(b_kfull + 8 * i, 1);
@@ -427,6 +440,9 @@ __global__ void __maxnreg__(kScoreMaxReg)
     for (int i = 0; i < kRsXBuf * 4; ++i) xcnt[i] = 0u;
     fence_mbar_init();
     tma_prefetch_desc(&kmap);
+    // the first copies fly while the CTA sets up
+    fence_proxy_async_smem();
+    for (; early < S && early < ntiles; ++early) load_k(early, early);
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(slot), 512);
@@ -461,18 +477,13 @@ __global__ void __maxnreg__(kScoreMaxReg)
 
   if (warp == 0) {
     if (lane == 0) {
-      int issued[kMaxKStages] = {0, 0, 0, 0};
-      int ks = 0;        // stage of tile it (it % S), counted instead of divided
-      uint32_t kp = 0u;  // passes over the ring (it / S)
-      for (int it = 0; it < ntiles; ++it, ks = ks + 1 == S ? 0 : ks + 1, kp += ks == 0u ? 1u : 0u) {
-        const int s = ks;
-        const uint32_t u = kp;
-        if (!mbar_wait(b_kempty + 8 * s, (u & 1u) ^ 1u, err, abort_flag)) break;
-        const int tok = j0 + it * KN;
-        mbar_arrive_expect_tx(b_kfull + 8 * s, (uint32_t)L.k_stage_bytes);
-        tma_load_3d(sK + s * L.k_stage_bytes, &kmap, b_kfull + 8 * s, 0, h, tok);
-        tma_load_3d(sK + s * L.k_stage_bytes + KN * 128, &kmap, b_kfull + 8 * s, 64, h, tok);
-        ++issued[s];
+      int issued[kMaxKStages], ks = early == S ? 0 : early;
+      uint32_t kp = early == S ? 1u : 0u;
+      for (int i = 0; i < kMaxKStages; ++i) issued[i] = i < early ? 1 : 0;
+      for (int it = early; it < ntiles; ++it, ks = ks + 1 == S ? 0 : ks + 1, kp += ks == 0 ? 1u : 0u) {
+        if (!mbar_wait(b_kempty + 8 * ks, (kp & 1u) ^ 1u, err, abort_flag)) break;
+        load_k(it, ks);
+        ++issued[ks];
       }
       if (*abort_flag)
         for (int s = 0; s < S; ++s)
@@ -715,6 +726,16 @@ __global__ void __maxnreg__(kScoreMaxReg)
   const uint32_t b_xfull = smem_u32(sm + L.off_xch + kCsXBuf * kScoreGroups * 128 * 4);
   const uint32_t b_xfree = b_xfull + 8 * kCsXBuf;
 
+  int ntiles = 0;
+  for (int t = blockIdx.x; t < ntiles_all; t += gridDim.x) ++ntiles;
+  int early = 0;  // key tiles loaded before the setup barrier (thread 0)
+  auto load_k = [&](int it, int s) {
+    const int tok = (blockIdx.x + it * gridDim.x) * 128;
+    mbar_arrive_expect_tx(b_kfull + 8 * s, 32768);
+    tma_load_3d(sK + s * 32768, &kmap, b_kfull + 8 * s, 0, h, tok);
+    tma_load_3d(sK + s * 32768 + 16384, &kmap, b_kfull + 8 * s, 64, h, tok);
+  };
+
   if (threadIdx.x == 0) {
     for (int i = 0; i < S; ++i) {
       mbar_init(b_kfull + 8 * i, 1);
@@ -732,6 +753,9 @@ __global__ void __maxnreg__(kScoreMaxReg)
     *abort_flag = 0u;
     fence_mbar_init();
     tma_prefetch_desc(&kmap);
+    // the first copies fly while the CTA sets up
+    fence_proxy_async_smem();
+    for (; early < S && early < ntiles; ++early) load_k(early, early);
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(slot), (uint32_t)L.tmem_cols);
@@ -747,23 +771,16 @@ __global__ void __maxnreg__(kScoreMaxReg)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *slot;
-  int ntiles = 0;
-  for (int t = blockIdx.x; t < ntiles_all; t += gridDim.x) ++ntiles;
 
   if (warp == 0) {
     if (lane == 0) {
-      int issued[kMaxKStages] = {0, 0, 0, 0};
-      int ks = 0;
-      uint32_t kp = 0u;
-      for (int it = 0; it < ntiles; ++it, ks = ks + 1 == S ? 0 : ks + 1, kp += ks == 0u ? 1u : 0u) {
-        const int s = ks;
-        const uint32_t u = kp;
-        if (!mbar_wait(b_kempty + 8 * s, (u & 1u) ^ 1u, err, abort_flag)) break;
-        const int tok = (blockIdx.x + it * gridDim.x) * 128;
-        mbar_arrive_expect_tx(b_kfull + 8 * s, 32768);
-        tma_load_3d(sK + s * 32768, &kmap, b_kfull + 8 * s, 0, h, tok);
-        tma_load_3d(sK + s * 32768 + 16384, &kmap, b_kfull + 8 * s, 64, h, tok);
-        ++issued[s];
+      int issued[kMaxKStages], ks = early == S ? 0 : early;
+      uint32_t kp = early == S ? 1u : 0u;
+      for (int i = 0; i < kMaxKStages; ++i) issued[i] = i < early ? 1 : 0;
+      for (int it = early; it < ntiles; ++it, ks = ks + 1 == S ? 0 : ks + 1, kp += ks == 0 ? 1u : 0u) {
+        if (!mbar_wait(b_kempty + 8 * ks, (kp & 1u) ^ 1u, err, abort_flag)) break;
+        load_k(it, ks);
+        ++issued[ks];
       }
       if (*abort_flag)
         for (int s = 0; s < S; ++s)
@@ -981,6 +998,16 @@ __global__ void __launch_bounds__(kThreads, 1)
   volatile uint32_t* abort_flag = slot + 1;
   int ntiles = 0;
   for (int t = blockIdx.x; t < ntiles_all; t += gridDim.x) ++ntiles;
+  int early = 0, lf = 0;  // tiles loaded before the setup barrier (thread 0); the frame of the last one loaded
+  auto load_k = [&](int it, int s) {
+    int t0;
+    css_tile_next(ft, blockIdx.x + it * gridDim.x, lf, t0);
+    const int nbox = (((128 + ft.gw[lf] + 1 + 15) & ~15) + 63) / 64;  // 64-row boxes covering NB rows
+    mbar_arrive_expect_tx(b_kfull + 8 * s, (uint32_t)(2 * nbox * 64 * 128));
+    for (int kb = 0; kb < 2; ++kb)
+      for (int r = 0; r < nbox; ++r)
+        tma_load_3d(sB + s * SB + kb * half_bytes + r * 8192, &kmap, b_kfull + 8 * s, kb * 64, h, t0 + r * 64);
+  };
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < S; ++i) {
@@ -995,6 +1022,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     *abort_flag = 0u;
     fence_mbar_init();
     tma_prefetch_desc(&kmap);
+    // the first copies fly while the CTA sets up
+    fence_proxy_async_smem();
+    for (; early < S && early < ntiles; ++early) load_k(early, early);
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(slot), 512);
@@ -1007,22 +1037,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (warp == 0) {
     if (lane == 0) {
-      int issued[kCssMaxStages] = {0, 0, 0, 0};
-      int f = 0, ks = 0;
-      uint32_t kp = 0u;
-      for (int it = 0; it < ntiles; ++it, ks = ks + 1 == S ? 0 : ks + 1, kp += ks == 0u ? 1u : 0u) {
-        const int s = ks;
-        const uint32_t u = kp;
-        if (!mbar_wait(b_kempty + 8 * s, (u & 1u) ^ 1u, err, abort_flag)) break;
-        int t0;
-        css_tile_next(ft, blockIdx.x + it * gridDim.x, f, t0);
-        const int nbox = (((128 + ft.gw[f] + 1 + 15) & ~15) + 63) / 64;  // 64-row boxes covering NB rows
-        mbar_arrive_expect_tx(b_kfull + 8 * s, (uint32_t)(2 * nbox * 64 * 128));
-        for (int kb = 0; kb < 2; ++kb)
-          for (int r = 0; r < nbox; ++r)
-            tma_load_3d(sB + s * SB + kb * half_bytes + r * 8192, &kmap, b_kfull + 8 * s, kb * 64, h,
-                        t0 + r * 64);
-        ++issued[s];
+      int issued[kCssMaxStages], ks = early == S ? 0 : early;
+      uint32_t kp = early == S ? 1u : 0u;
+      for (int i = 0; i < kCssMaxStages; ++i) issued[i] = i < early ? 1 : 0;
+      for (int it = early; it < ntiles; ++it, ks = ks + 1 == S ? 0 : ks + 1, kp += ks == 0 ? 1u : 0u) {
+        if (!mbar_wait(b_kempty + 8 * ks, (kp & 1u) ^ 1u, err, abort_flag)) break;
+        load_k(it, ks);
+        ++issued[ks];
       }
       if (*abort_flag)
         for (int s = 0; s < S; ++s)
@@ -1391,7 +1412,7 @@ cudaError_t launch_tsg_umma(const Problem& p, const FrameTable& ft, const LayerP
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTsgSmem);
   if (e != cudaSuccess) return e;
   const int groups = nchunk * p.L * p.hkv;
-  const int gx = pick_split(groups, n_tiles, sm_count(), n_tiles, 3);
+  const int gx = pick_split(groups, n_tiles, sm_count(), n_tiles, 4);
   dim3 grid(gx, nchunk, p.L * p.hkv);
   TimingScope ts("tsg_umma", st);
   kern<<<grid, kThreads, kTsgSmem, st>>>(local, ft, rn_cur, cur_pad, rho_key, p.hkv, err);
