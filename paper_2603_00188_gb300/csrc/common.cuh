@@ -113,6 +113,15 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
   return t;
 }
 
+// Programmatic dependent launch (launch_after): a kernel launched that way may
+// start while its predecessor in the stream still runs; pdl_wait returns once
+// the predecessor has completed and its writes are visible, and pdl_trigger
+// lets a successor start.  Every thread of such a kernel waits before it
+// touches global memory, so a kernel completes after its predecessor does and
+// the order of the stream holds for whatever follows.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void record_error(uint32_t* err, uint32_t bits) {
   if (err) atomicOr(err, bits);
 }

@@ -56,6 +56,8 @@ __global__ void __launch_bounds__(kDecThreads, 2) k_decode_split(const __grid_co
                                                               int hq, int hkv, int per, float* part_o_all,
                                                               float2* part_ml_all) {
   extern __shared__ float4 dec_smem[];
+  pdl_trigger();
+  pdl_wait();
   const int split = blockIdx.x, h = blockIdx.y, r = blockIdx.z % w, layer = blockIdx.z / w, nsplit = gridDim.x;
   const T* __restrict__ q = static_cast<const T*>(b.q[layer]);
   const T* __restrict__ k = static_cast<const T*>(b.k[layer]);
@@ -276,8 +278,12 @@ __global__ void __launch_bounds__(kDecMmaThreads, 1)
     for (int i = 0; i < kDecStages; ++i) mbar_init(b_full + 8 * i, 1);
     *abort_flag = 0u;
     fence_mbar_init();
+    tma_prefetch_desc(&kmap);
+    tma_prefetch_desc(&vmap);
   }
   __syncthreads();
+  pdl_trigger();
+  pdl_wait();
   // keys and values of tile it into stage it % kDecStages (one thread)
   auto issue = [&](int it) {
     const int s = it % kDecStages;
@@ -441,60 +447,61 @@ __global__ void __launch_bounds__(kDecMmaThreads, 1)
   }
 }
 
-// out[r][g][c] = merge over the splits.  grid (hq, w), one thread per
-// dimension: the splits' weights exp2(m_s - M) and the normaliser are formed
-// once in shared memory, then every thread sums its dimension over the splits
-// with eight partial loads in flight.
+// out[r][g][c] = merge over the splits.  grid (hq, w * layers), four slices of
+// 128 threads, one dimension each: the splits' weights exp2(m_s - M) and the
+// normaliser are formed in shared memory by one split (or two) per thread
+// while slice k's first eight partials (splits k, k + 4, ...) are on their way.
+// A merge is two or three memory latencies, nothing else: with one slice that
+// loaded the partials after the weights, eight at a time, it took twice as
+// long.
 constexpr int kDecMaxSplits = 1024;
-__global__ void __launch_bounds__(kD) k_decode_combine(const __grid_constant__ DecBatch b, const float* part_o_all,
-                                                       const float2* part_ml_all, int nsplit, int hq, int w) {
+constexpr int kCmbSlices = 4, kCmbThreads = kCmbSlices * kD, kCmbWarps = kCmbThreads / 32;
+static_assert(kDecMaxSplits <= 2 * kCmbThreads, "two splits per thread");
+__global__ void __launch_bounds__(kCmbThreads) k_decode_combine(const __grid_constant__ DecBatch b,
+                                                                const float* part_o_all, const float2* part_ml_all,
+                                                                int nsplit, int hq, int w) {
   __shared__ float wts[kDecMaxSplits];
-  __shared__ float red[kD / 32];
-  __shared__ float bc[2];
-  const int g = blockIdx.x, r = blockIdx.y % w, layer = blockIdx.y / w, c = threadIdx.x, lane = c & 31, wp = c >> 5;
-  const float* part_o = part_o_all + (size_t)layer * nsplit * w * hq * kD;
-  const float2* part_ml = part_ml_all + (size_t)layer * nsplit * w * hq;
-  float* out = b.out[layer];
-  float mx = -CUDART_INF_F;
-  for (int s = c; s < nsplit; s += kD) mx = fmaxf(mx, part_ml[((size_t)s * w + r) * hq + g].x);
-  mx = warp_max(mx);
-  if (lane == 0) red[wp] = mx;
+  __shared__ float red[2][kCmbWarps];
+  __shared__ float acc[kCmbSlices - 1][kD];
+  const int g = blockIdx.x, r = blockIdx.y % w, layer = blockIdx.y / w;
+  const int t = threadIdx.x, c = t & (kD - 1), k = t / kD, lane = t & 31, wp = t >> 5;
+  const size_t rows = (size_t)w * hq;  // partial rows of one split
+  const float* part_o = part_o_all + ((size_t)layer * nsplit * rows + (size_t)r * hq + g) * kD + c;
+  const float2* part_ml = part_ml_all + (size_t)layer * nsplit * rows + (size_t)r * hq + g;
+  pdl_trigger();
+  pdl_wait();
+  float x[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) x[u] = k + kCmbSlices * u < nsplit ? part_o[(size_t)(k + kCmbSlices * u) * rows * kD] : 0.f;
+  const float2 none = make_float2(-CUDART_INF_F, 0.f);
+  const float2 ml0 = t < nsplit ? part_ml[(size_t)t * rows] : none;
+  const float2 ml1 = t + kCmbThreads < nsplit ? part_ml[(size_t)(t + kCmbThreads) * rows] : none;
+  const float mx = warp_max(fmaxf(ml0.x, ml1.x));
+  if (lane == 0) red[0][wp] = mx;
   __syncthreads();
-  if (c == 0) {
-    float M = red[0];
-    for (int i = 1; i < kD / 32; ++i) M = fmaxf(M, red[i]);
-    bc[0] = M;
-  }
+  const float M = warp_max(red[0][lane % kCmbWarps]);
+  const float a0 = weight(ml0.x, M), a1 = weight(ml1.x, M);
+  if (t < nsplit) wts[t] = a0;
+  if (t + kCmbThreads < nsplit) wts[t + kCmbThreads] = a1;
+  const float ls = warp_sum(fmaf(ml0.y, a0, ml1.y * a1));
+  if (lane == 0) red[1][wp] = ls;
   __syncthreads();
-  const float M = bc[0];
-  float ls = 0.f;
-  for (int s = c; s < nsplit; s += kD) {
-    const float2 ml = part_ml[((size_t)s * w + r) * hq + g];
-    const float a = weight(ml.x, M);
-    wts[s] = a;
-    ls = fmaf(ml.y, a, ls);
-  }
-  ls = warp_sum(ls);
-  __syncthreads();  // red is reused
-  if (lane == 0) red[wp] = ls;
-  __syncthreads();
-  if (c == 0) {
-    float L = 0.f;
-    for (int i = 0; i < kD / 32; ++i) L += red[i];
-    bc[1] = L;
-  }
-  __syncthreads();
+  const float L = warp_sum(lane < kCmbWarps ? red[1][lane] : 0.f);
   float O = 0.f;
-  int s = 0;
-  for (; s + 8 <= nsplit; s += 8) {
-    float x[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = part_o[(((size_t)(s + u) * w + r) * hq + g) * kD + c];
+  for (int u = 0; u < 8; ++u)
+    if (k + kCmbSlices * u < nsplit) O = fmaf(x[u], wts[k + kCmbSlices * u], O);
+  for (int s0 = k + 8 * kCmbSlices; s0 < nsplit; s0 += 8 * kCmbSlices) {
 #pragma unroll
-    for (int u = 0; u < 8; ++u) O = fmaf(x[u], wts[s + u], O);
+    for (int u = 0; u < 8; ++u)
+      x[u] = s0 + kCmbSlices * u < nsplit ? part_o[(size_t)(s0 + kCmbSlices * u) * rows * kD] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (s0 + kCmbSlices * u < nsplit) O = fmaf(x[u], wts[s0 + kCmbSlices * u], O);
   }
-  for (; s < nsplit; ++s) O = fmaf(part_o[(((size_t)s * w + r) * hq + g) * kD + c], wts[s], O);
-  out[((size_t)r * hq + g) * kD + c] = O / bc[1];
+  if (k > 0) acc[k - 1][c] = O;
+  __syncthreads();
+  if (k == 0) b.out[layer][((size_t)r * hq + g) * kD + c] = ((O + acc[0][c]) + (acc[1][c] + acc[2][c])) / L;
 }
 
 int decode_splits(int n, int hkv, int w, int layers) {
@@ -555,8 +562,8 @@ cudaError_t launch_decode(DType dt, const DecBatch& b, int layers, int n, int hq
       constexpr int NT = decltype(nt)::value;
       e = cudaFuncSetAttribute(k_decode_mma<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, dec_mma_smem(NT));
       if (e != cudaSuccess) return;
-      k_decode_mma<NT><<<grid, kDecMmaThreads, dec_mma_smem(NT), st>>>(maps, b, w, n, hq, hkv, per, part_o,
-                                                                       part_ml, err);
+      e = launch_after(k_decode_mma<NT>, grid, kDecMmaThreads, dec_mma_smem(NT), st, maps, b, w, n, hq, hkv, per,
+                       part_o, part_ml, err);
     };
     TimingScope ts("decode_split", st);
     if (G <= 8)
@@ -570,7 +577,7 @@ cudaError_t launch_decode(DType dt, const DecBatch& b, int layers, int n, int hq
       constexpr int GM = decltype(gm)::value;
       e = cudaFuncSetAttribute(k_decode_split<float, GM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return;
-      k_decode_split<float, GM><<<grid, kDecThreads, smem, st>>>(b, w, n, hq, hkv, per, part_o, part_ml);
+      e = launch_after(k_decode_split<float, GM>, grid, kDecThreads, smem, st, b, w, n, hq, hkv, per, part_o, part_ml);
     };
     TimingScope ts("decode_split", st);
     if (G <= 4)
@@ -583,8 +590,8 @@ cudaError_t launch_decode(DType dt, const DecBatch& b, int layers, int n, int hq
   if (e != cudaSuccess) return e;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   TimingScope ts("decode_combine", st);
-  k_decode_combine<<<dim3(hq, w * layers), kD, 0, st>>>(b, part_o, part_ml, nsplit, hq, w);
-  return cudaGetLastError();
+  e = launch_after(k_decode_combine, dim3(hq, w * layers), kCmbThreads, 0, st, b, part_o, part_ml, nsplit, hq, w);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace stl

@@ -100,6 +100,23 @@ class TimingScope {
   cudaEvent_t start_;
 };
 
+// Launches `kern` so that it may start before its predecessor in the stream
+// has completed (see pdl_wait, which it calls).
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // ---- launchers ----------------------------------------------------------
 // What a kernel that forms the inverse key norms writes: rn[l][h][j] = 1 /
 // max(|k_l[j,h]|, 1e-8); the current frame's also to rn_cur[l][h][j -
