@@ -91,6 +91,45 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// Folds one split partial (m2, l2) of the window score's row statistics into
+// (m, l): the running max in log2 units and the sum of 2^(x - max).
+// Symmetric in its two arguments, bit for bit (max and a two-term sum commute).
+__device__ __forceinline__ void fold_partial(float& m, float& l, float m2, float l2) {
+  if (!(l2 > 0.f)) return;
+  if (!(l > 0.f)) {
+    m = m2;
+    l = l2;
+    return;
+  }
+  const float mn = fmaxf(m, m2);
+  l = l * exp2f(m - mn) + l2 * exp2f(m2 - mn);
+  m = mn;
+}
+
+// The bias -m - log2(G l) of one query row from its splits' partials pp[0],
+// pp[R], pp[2 R], ..., by four neighbouring lanes (whole warps call it): lane q
+// folds splits q, q + 4, q + 8, ... (eight loads in flight), then the four
+// lanes' states are folded pairwise with shuffles, so that every lane holds
+// the same bits.  The order depends on the split count alone.
+__device__ __forceinline__ float row_bias4(const float2* pp, int R, int nsplit, float G) {
+  const int q = threadIdx.x & 3;
+  float m = -CUDART_INF_F, l = 0.f;
+  for (int s0 = q; s0 < nsplit; s0 += 32) {
+    float2 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      v[u] = s0 + 4 * u < nsplit ? pp[(size_t)(s0 + 4 * u) * R] : make_float2(-CUDART_INF_F, 0.f);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) fold_partial(m, l, v[u].x, v[u].y);
+  }
+#pragma unroll
+  for (int o = 1; o < 4; o <<= 1) {
+    const float m2 = __shfl_xor_sync(0xffffffffu, m, o), l2 = __shfl_xor_sync(0xffffffffu, l, o);
+    fold_partial(m, l, m2, l2);
+  }
+  return -m - log2f(G * l);
+}
+
 __device__ __forceinline__ float dot4(float4 a, float4 b) {
   return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, a.w * b.w)));
 }

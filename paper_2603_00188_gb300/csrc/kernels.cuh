@@ -100,8 +100,9 @@ class TimingScope {
   cudaEvent_t start_;
 };
 
-// Launches `kern` so that it may start before its predecessor in the stream
-// has completed (see pdl_wait, which it calls).
+// Launches `kern` so that it may start once every CTA of its predecessor in
+// the stream has called pdl_trigger (see pdl_wait, which kern calls before it
+// touches anything the predecessor writes, reads or was ordered after).
 template <typename... P, typename... A>
 cudaError_t launch_after(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -144,7 +145,7 @@ int score_nsplit(const Problem& p);
 int score_nsplit_max(const Problem& p);
 // Merges pass 1's split partials into the row bias -m_r - log2(G l_r) that
 // follows them in rowpart ([Hkv][R] float per layer).
-void launch_row_bias(const Problem& p, int nsplit, Strided<float2> rowpart, cudaStream_t st);
+cudaError_t launch_row_bias(const Problem& p, int nsplit, Strided<float2> rowpart, cudaStream_t st);
 
 // TSG row maxima: rho_key[l][h][i] = max over the current frame's columns j
 // of k_i.k_j * rn_j, for historical visual tokens i (Eq. 6 before the 1/|k_i|

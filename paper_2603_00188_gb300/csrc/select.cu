@@ -449,6 +449,7 @@ __global__ void __launch_bounds__(kSelThreads, 4) k_select(Problem p, const __gr
   cg::cluster_group cl = cg::this_cluster();
   const int ncta = (int)cl.num_blocks(), c = (int)cl.block_rank();
   const int l = blockIdx.y / p.hkv, h = blockIdx.y % p.hkv, n = p.n, tid = threadIdx.x;
+  pdl_trigger();
   const int chunk = ((n + ncta - 1) / ncta + 3) & ~3;  // four-token groups never straddle two CTAs
   const int j0 = min(n, c * chunk), j1 = min(n, j0 + chunk), len = j1 - j0;
   const bool vec = (n & 3) == 0;  // every row base [Hkv][N] is 16-byte aligned
@@ -794,6 +795,7 @@ cudaError_t launch_select(const Problem& p, const FrameTable& ft, const SelectAr
 // grid.y = layer.
 template <int CPR>
 __global__ void __launch_bounds__(256) k_gather(const __grid_constant__ LayerPtrs io, int n, int hkv) {
+  pdl_wait();
   const int l = blockIdx.y;
   const int budget = io.budget[l];
   const int32_t* idx = io.idx[l];
@@ -846,11 +848,8 @@ cudaError_t launch_gather(const Problem& p, const LayerPtrs& io, cudaStream_t st
   if (blocks < 1) blocks = 1;
   TimingScope ts("gather", st);
   dim3 grid((unsigned)blocks, p.L);
-  if (cpr == 16)
-    k_gather<16><<<grid, 256, 0, st>>>(io, p.n, p.hkv);
-  else
-    k_gather<32><<<grid, 256, 0, st>>>(io, p.n, p.hkv);
-  return cudaGetLastError();
+  const cudaError_t e = launch_after(cpr == 16 ? k_gather<16> : k_gather<32>, grid, 256, 0, st, io, p.n, p.hkv);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace stl

@@ -53,6 +53,9 @@ __device__ __forceinline__ void load_q_sw128(uint8_t* sq, int rows, const __nv_b
       *reinterpret_cast<uint4*>(sq + off) = make_uint4(0, 0, 0, 0);
     }
   }
+}
+// The copies of load_q_sw128 (this thread's) have landed, for the tensor core.
+__device__ __forceinline__ void load_q_done() {
   cp_async_wait_all();
   fence_proxy_async_smem();
 }
@@ -449,6 +452,8 @@ __global__ void __maxnreg__(kScoreMaxReg)
     tmem_relinquish();
   }
   load_q_sw128(sm, MT * 128, q, p, h, r0);
+  load_q_done();
+  pdl_trigger();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -696,11 +701,12 @@ __host__ __device__ inline CsLayout cs_layout(int R) {
 }
 
 // NH: column halves per key tile (cs_layout's nh), a template parameter so
-// that the one-half loop compiles away.
+// that the one-half loop compiles away.  merged: k_row_bias has merged the
+// splits' row statistics; otherwise every CTA does so for itself.
 template <int NH>
 __global__ void __maxnreg__(kScoreMaxReg)
     k_colsum_umma(const __grid_constant__ KMaps maps, const __grid_constant__ LayerPtrs io, Problem p,
-                  Strided<float2> part_all, int nsplit, Strided<float> a_all, uint32_t* err) {
+                  Strided<float2> part_all, int nsplit, int merged, Strided<float> a_all, uint32_t* err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = align1024(smem_raw);
   const CsLayout L = cs_layout(p.R());
@@ -762,11 +768,22 @@ __global__ void __maxnreg__(kScoreMaxReg)
     tmem_relinquish();
   }
   load_q_sw128(sm, NQ, q, p, h);
-  // pass 1's merged row statistics: bias_r = -m_r - log2(G l_r), so that
-  // 2^(x c + bias_r) is the softmax probability divided by G (padded rows
-  // get -inf and add exact zeros)
-  const float* bias_g = reinterpret_cast<const float*>(part + (size_t)p.hkv * nsplit * R) + (size_t)h * R;
-  for (int r = threadIdx.x; r < NQ; r += blockDim.x) bias_s[r] = r < R ? bias_g[r] : -CUDART_INF_F;
+  // what follows needs the row statistics; the copies above do not
+  pdl_wait();
+  // pass 1's row statistics, the splits merged: bias_r = -m_r - log2(G l_r),
+  // so that 2^(x c + bias_r) is the softmax probability divided by G (padded
+  // rows get -inf and add exact zeros)
+  if (merged) {
+    const float* bias_g = reinterpret_cast<const float*>(part + (size_t)p.hkv * nsplit * R) + (size_t)h * R;
+    for (int r = threadIdx.x; r < NQ; r += kCsThreads) bias_s[r] = r < R ? bias_g[r] : -CUDART_INF_F;
+  } else {
+    for (int e4 = threadIdx.x; e4 < 4 * NQ; e4 += kCsThreads) {  // NQ a multiple of 32: whole warps
+      const int r = e4 >> 2;
+      const float b = row_bias4(part + (size_t)h * nsplit * R + min(r, R - 1), R, nsplit, (float)p.G());
+      if ((e4 & 3) == 0) bias_s[r] = r < R ? b : -CUDART_INF_F;
+    }
+  }
+  load_q_done();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1447,16 +1464,20 @@ cudaError_t launch_score_umma(const Problem& p, const LayerPtrs& io, Strided<flo
                                                                                err);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  {
-    TimingScope ts("row_bias", st);
-    launch_row_bias(p, nsplit, rowpart, st);
-  }
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int tiles = (p.n + 127) / 128;
   const int gx = pick_split(p.L * p.hkv, tiles, sm_count(), tiles, 6);
+  // One wave of CTAs merges the splits' row statistics itself, beside its first
+  // copies (a merge launch of its own costs 6 us); with several waves that work
+  // would be done over (28 layers of 53,600 tokens: the step 0.5 % slower).
+  const int merged = (long long)gx * p.L * p.hkv > sm_count();
+  if (merged) {
+    TimingScope ts("row_bias", st);
+    if ((e = launch_row_bias(p, nsplit, rowpart, st)) != cudaSuccess) return e;
+  }
   TimingScope ts("colsum_umma", st);
-  cs_kernel<<<dim3(gx, p.L * p.hkv), kCsThreads, L2.total, st>>>(m2, io, p, rowpart, nsplit, a_base, err);
-  return cudaGetLastError();
+  e = launch_after(cs_kernel, dim3(gx, p.L * p.hkv), kCsThreads, L2.total, st, m2, io, p, rowpart, nsplit,
+                   merged, a_base, err);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 bool css_umma_supported(const FrameTable& ft) {
