@@ -293,7 +293,7 @@ __device__ __forceinline__ void add2(float& a0, float& a1, float b0, float b1) {
       : "f"(b0), "f"(b1));
 }
 
-// max(a, b, c) in one instruction (inputs here are never NaN).
+// max(a, b, c) in one instruction; NaN inputs are ignored (PTX max without .NaN).
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float d;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));

@@ -226,9 +226,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!warp_wait(b_accfull + 8 * g, (uint32_t)it & 1u, err, abort_flag)) break;
         tc_fence_after();
         float mx = -CUDART_INF_F;
-        if (valid_g == 256) {
-          // full stage: no masked column, packed products and 3-input max
-          // into eight independent running maxima (short dependency chains)
+        if (valid_g > 192) {
+          // (nearly) full stage: packed products and 3-input max into eight
+          // independent running maxima (short dependency chains); a column
+          // past the frame carries rn = NaN, and the maximum ignores NaN,
+          // whatever is left in its TMEM column
           float m[8];
 #pragma unroll
           for (int i = 0; i < 8; ++i) m[i] = -CUDART_INF_F;
