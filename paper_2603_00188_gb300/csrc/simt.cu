@@ -2,7 +2,11 @@
 // of window scoring and TSG (fp32 inputs cannot use the bf16 tensor-core
 // path without losing the exactness of the products).  Every kernel covers a
 // batch of layers: the layer index is the high part of one grid dimension.
+#include <cooperative_groups.h>
+
 #include "kernels.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace stl {
 
@@ -646,15 +650,19 @@ cudaError_t launch_row_bias(const Problem& p, int nsplit, Strided<float2> rowpar
 // ---------------------------------------------------------- column sums
 // Window score, second pass (fp32): a[h][j] = sum_r 2^(x_rj + bias_r).  The
 // key tile stays, the query rows stream; a thread sums its eight keys over
-// the rows it sees, the sixteen threads of a key add theirs at the end.
-// grid = (key tile, layer*Hkv + head).
+// the rows it sees, the sixteen threads of a key add theirs at the end.  A
+// cluster of CTAs may share a key tile: each takes every split-th tile of
+// query rows, and their sums are added in rank order.
+// grid = (key tile * split, layer*Hkv + head).
 __global__ void __launch_bounds__(kTileThreads, kTilesPerSm)
     k_colsum_simt(const __grid_constant__ LayerPtrs io, Problem p, int nsplit, Strided<float2> part_all,
                   Strided<float> a_all) {
   extern __shared__ float4 tile_smem[];
   float* ks = reinterpret_cast<float*>(tile_smem);
   float* qs = ks + kTileFloats;
-  const int l = blockIdx.y / p.hkv, h = blockIdx.y % p.hkv, j0 = blockIdx.x * kTileRows;
+  cg::cluster_group cl = cg::this_cluster();
+  const int split = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int l = blockIdx.y / p.hkv, h = blockIdx.y % p.hkv, j0 = (int)blockIdx.x / split * kTileRows;
   const float* q = static_cast<const float*>(io.q[l]);
   const float* k = static_cast<const float*>(io.k[l]);
   const int R = p.R(), ty = tile_ty(), tx = tile_tx();
@@ -664,7 +672,7 @@ __global__ void __launch_bounds__(kTileThreads, kTilesPerSm)
   float acc[kTA];
 #pragma unroll
   for (int i = 0; i < kTA; ++i) acc[i] = 0.f;
-  for (int rt = 0; rt < R; rt += kTileRows) {
+  for (int rt = rank * kTileRows; rt < R; rt += split * kTileRows) {
     const int nr = min(kTileRows, R - rt);
     tile_load(qs, nr, [&](int r) { return q_row(q, p, h, rt + r); });
     float bs[kTB];
@@ -686,16 +694,37 @@ __global__ void __launch_bounds__(kTileThreads, kTilesPerSm)
   for (int i = 0; i < kTA; ++i)
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+  tile_ready();  // also for a CTA without query rows, whose key copies are still in flight
   if (tx == 8)
 #pragma unroll
     for (int i = 0; i < kTA; ++i) qs[ty + 8 * i] = acc[i];
   __syncthreads();
   if (tx == 0)
 #pragma unroll
-    for (int i = 0; i < kTA; ++i) {
-      const int j = j0 + ty + 8 * i;
-      if (j < p.n) a_all.at(l)[(size_t)h * p.n + j] = acc[i] + qs[ty + 8 * i];
-    }
+    for (int i = 0; i < kTA; ++i) qs[ty + 8 * i] += acc[i];
+  if (split > 1)
+    cl.sync();
+  else
+    __syncthreads();
+  const int j = j0 + threadIdx.x;
+  if (rank == 0 && threadIdx.x < kTileRows && j < p.n) {
+    float sum = qs[threadIdx.x];
+    for (int r = 1; r < split; ++r) sum += cl.map_shared_rank(qs, r)[threadIdx.x];
+    a_all.at(l)[(size_t)h * p.n + j] = sum;
+  }
+  if (split > 1) cl.sync();  // no CTA leaves while rank 0 may still read its sums
+}
+
+// CTAs per key tile: as many as there are tiles of query rows, while those of
+// one layer all fit at once (1,152 keys of 4 heads: 72 key tiles for 456
+// places; one CTA each worked off four tiles of query rows alone on its SM).
+// It fixes how the sums are grouped, so it depends on the layer's shape alone.
+static int colsum_simt_split(const Problem& p) {
+  const long long tiles = (long long)((p.n + kTileRows - 1) / kTileRows) * p.hkv;
+  const int rows = (p.R() + kTileRows - 1) / kTileRows;
+  int s = 1;
+  while (2 * s <= rows && 2 * s <= 8 && tiles * 2 * s <= 152 * kTilesPerSm) s *= 2;
+  return s;
 }
 
 cudaError_t launch_score(const Problem& p, const LayerPtrs& io, Strided<float2> rowpart, int nsplit,
@@ -705,7 +734,18 @@ cudaError_t launch_score(const Problem& p, const LayerPtrs& io, Strided<float2> 
   e = cudaFuncSetAttribute(k_colsum_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, kScoreSimtSmem);
   if (e != cudaSuccess) return e;
   dim3 g1(nsplit, p.L * p.hkv, (p.R() + kTileRows - 1) / kTileRows);
-  dim3 g2((p.n + kTileRows - 1) / kTileRows, p.L * p.hkv);
+  const int split = colsum_simt_split(p);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  cfg.gridDim = dim3((p.n + kTileRows - 1) / kTileRows * split, p.L * p.hkv);
+  cfg.blockDim = dim3(kTileThreads);
+  cfg.dynamicSmemBytes = kScoreSimtSmem;
+  cfg.stream = st;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)split;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
   {
     TimingScope ts("rowstats_simt", st);
     k_rowstats_simt<<<g1, kTileThreads, kScoreSimtSmem, st>>>(io, p, nsplit, rowpart);
@@ -716,8 +756,8 @@ cudaError_t launch_score(const Problem& p, const LayerPtrs& io, Strided<float2> 
     if ((e = launch_row_bias(p, nsplit, rowpart, st)) != cudaSuccess) return e;
   }
   TimingScope ts("colsum_simt", st);
-  k_colsum_simt<<<g2, kTileThreads, kScoreSimtSmem, st>>>(io, p, nsplit, rowpart, a_base);
-  return cudaGetLastError();
+  e = cudaLaunchKernelEx(&cfg, k_colsum_simt, io, p, nsplit, rowpart, a_base);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ TSG
