@@ -393,7 +393,10 @@ cudaError_t run_css_phi(const Ctx& c, Strided<float> phi, cudaStream_t st) {
 // tensor-core one (so that every path sees the same bits), else from the
 // norms kernel (whose arithmetic matches the CUDA-core CSS kernel's).
 cudaError_t run_norms(const Ctx& c, const LayerPtrs& io) {
-  if (use_tensor_cores(c.p) && css_umma_supported(c.ft)) return run_css(c, io, c.view<float>(c.plan.phi), true);
+  if (use_tensor_cores(c.p) && css_umma_supported(c.ft)) {
+    bool deferred;  // leaves Phi, which nobody asks for (7 us of a 14-frame layer's gate)
+    return run_css(c, io, c.view<float>(c.plan.phi), true, 3, true, &deferred);
+  }
   return launch_inv_norms(c.p, c.ft, io, norms_out(c, true), c.st);
 }
 
