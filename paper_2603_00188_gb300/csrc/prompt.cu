@@ -713,8 +713,10 @@ PromptArgs prompt_args(int n, int nq, int hq, int hkv, int mode) {
 // CTAs per key tile of pass 2.  A tile's chunks cannot be shared between
 // waves, so the pass ends with the CTA of the most chunks (the first keys'
 // tiles: every chunk) or, with many tiles, when the SMs have worked off all of
-// them: about total / SMs + longest / 2 chunks, plus 6 per CTA an SM runs.
-static int prompt_split(const PromptArgs& a, int nsm) {
+// them: about total / SMs + longest / 2 chunks, plus 6 per CTA an SM runs.  It
+// fixes how the sums are grouped, so it depends on the shape alone (152 SMs).
+static int prompt_split(const PromptArgs& a) {
+  constexpr int nsm = 152;
   const long long tiles = (a.n + 127) / 128;
   long long chunks = 0;
   for (long long t = 0; t < tiles; ++t) {
@@ -780,7 +782,7 @@ cudaError_t launch_prompt_score(DType dt, const void* q, const void* k, int n, i
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
-  const int split = prompt_split(a, nsm);
+  const int split = prompt_split(a);
   cfg.gridDim = dim3((unsigned)((n + 127) / 128 * hkv * split));
   cfg.blockDim = dim3(kPrThreads);
   cfg.dynamicSmemBytes = kP2Smem;
