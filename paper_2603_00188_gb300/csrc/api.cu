@@ -366,8 +366,9 @@ NormsOut norms_out(const Ctx& c, bool tsg) {
 // size ablation, on the box-sum kernel).
 // defer_phi: the tensor-core CSS leaves Phi to a later run_css_phi and sets
 // *deferred (the other kernels produce Phi themselves).
+// text_nan (tensor-core CSS): Phi = NaN for text tokens.
 cudaError_t run_css(const Ctx& c, const LayerPtrs& io, Strided<float> phi, bool tsg, int size = 3,
-                    bool defer_phi = false, bool* deferred = nullptr) {
+                    bool defer_phi = false, bool* deferred = nullptr, bool text_nan = false) {
   const NormsOut norms = norms_out(c, tsg);
   if (deferred) *deferred = false;
   if (size > 3) return launch_css_box(c.p, c.ft, io, size, phi, norms, c.st);
@@ -376,7 +377,8 @@ cudaError_t run_css(const Ctx& c, const LayerPtrs& io, Strided<float> phi, bool 
     const size_t hn4 = (size_t)c.p.hkv * c.p.n * 4;
     Strided<float> dE = c.view<float>(c.plan.dots), dS = c.view<float>(c.plan.dots + hn4);
     Strided<float> dSE = c.view<float>(c.plan.dots + 2 * hn4), dSW = c.view<float>(c.plan.dots + 3 * hn4);
-    return launch_css_umma(c.p, c.ft, io, phi, norms, dE, dS, dSE, dSW, c.err, c.st, !(defer_phi && deferred));
+    return launch_css_umma(c.p, c.ft, io, phi, norms, dE, dS, dSE, dSW, c.err, c.st, !(defer_phi && deferred),
+                           text_nan);
   }
   return launch_css(c.p, c.ft, io, phi, norms, c.st);
 }
@@ -558,6 +560,8 @@ stlite_status stlite_spatial_saliency(const stlite_shape* shape, const stlite_fr
   if (s != STLITE_OK) return s;
   if (!k || !phi || !aligned16(k) || !aligned16(phi)) return STLITE_EINVAL;
   const LayerPtrs io = single_layer(nullptr, k, nullptr, nullptr, nullptr, nullptr);
+  if (use_tensor_cores(c.p) && css_umma_supported(c.ft) && c.ft.n_frames > 0)
+    return cuda_status(run_css(c, io, one(phi), false, 3, false, nullptr, true));
   cudaError_t e = run_css(c, io, one(phi), false);
   if (e == cudaSuccess) e = launch_fill_text_nan(c.p, c.ft, phi, c.st);
   return cuda_status(e);

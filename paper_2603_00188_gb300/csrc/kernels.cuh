@@ -172,12 +172,14 @@ cudaError_t launch_css(const Problem& p, const FrameTable& ft, const LayerPtrs& 
 bool css_umma_supported(const FrameTable& ft);
 cudaError_t launch_css_umma(const Problem& p, const FrameTable& ft, const LayerPtrs& io, Strided<float> phi,
                             const NormsOut& norms, Strided<float> dE, Strided<float> dS, Strided<float> dSE,
-                            Strided<float> dSW, uint32_t* err, cudaStream_t st, bool with_phi = true);
+                            Strided<float> dSW, uint32_t* err, cudaStream_t st, bool with_phi = true,
+                            bool text_nan = false);
 // Phi of the CSS dots (the second kernel of launch_css_umma, on its own;
-// the caller orders it after the dots are written).
+// the caller orders it after the dots are written).  text_nan: Phi = NaN for
+// every text token, too.
 cudaError_t launch_css_phi(const Problem& p, const FrameTable& ft, Strided<float> phi, Strided<const float> rn,
                            Strided<float> dE, Strided<float> dS, Strided<float> dSE, Strided<float> dSW,
-                           cudaStream_t st);
+                           cudaStream_t st, bool text_nan = false);
 // CSS over the size x size neighbourhood (size 3, 5, 7 or 9; 3 is the
 // method's Moore neighbourhood) on the CUDA cores, through box sums of the
 // normalised keys; any grid width.  Writes phi and the norms' outputs as

@@ -1176,12 +1176,19 @@ __global__ void __launch_bounds__(kThreads, 1)
 // are done once per run.  grid = (run block, frame, layer*Hkv + head).
 constexpr int kPhiRun = 4;
 __global__ void __launch_bounds__(256) k_css_phi(const __grid_constant__ FrameTable ft, int hkv, CssDots d,
-                                                 Strided<const float> rn_all, Strided<float> phi_all) {
+                                                 Strided<const float> rn_all, Strided<float> phi_all,
+                                                 int text_nan) {
   const int f = blockIdx.y, l = blockIdx.z / hkv, h = blockIdx.z % hkv, n = ft.n_tokens;
   if (f >= ft.n_frames) return;
   const int gh = ft.gh[f], gw = ft.gw[f], off = ft.off[f];
   const int runs = (gw + kPhiRun - 1) / kPhiRun;  // runs per grid row
   const int slot = blockIdx.x * blockDim.x + threadIdx.x;
+  if (text_nan) {  // the text after the frame, and before the first one
+    float* row = phi_all.at(l) + (size_t)h * n;
+    const int end = f + 1 < ft.n_frames ? ft.off[f + 1] : n, step = gridDim.x * blockDim.x;
+    for (int j = off + gh * gw + slot; j < end; j += step) row[j] = CUDART_NAN_F;
+    for (int j = slot; f == 0 && j < off; j += step) row[j] = CUDART_NAN_F;
+  }
   if (slot >= gh * runs) return;
   const int u = slot / runs, v0 = (slot - u * runs) * kPhiRun;
   const size_t hn = (size_t)h * n;
@@ -1490,7 +1497,7 @@ bool css_umma_supported(const FrameTable& ft) {
 
 cudaError_t launch_css_umma(const Problem& p, const FrameTable& ft, const LayerPtrs& io, Strided<float> phi,
                             const NormsOut& norms, Strided<float> dE, Strided<float> dS, Strided<float> dSE,
-                            Strided<float> dSW, uint32_t* err, cudaStream_t st, bool with_phi) {
+                            Strided<float> dSW, uint32_t* err, cudaStream_t st, bool with_phi, bool text_nan) {
   const int tiles = ft.ctile0[ft.n_frames];
   if (tiles == 0) return cudaSuccess;
   KMaps maps;
@@ -1516,18 +1523,20 @@ cudaError_t launch_css_umma(const Problem& p, const FrameTable& ft, const LayerP
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (!with_phi) return cudaSuccess;
-  return launch_css_phi(p, ft, phi, strided<const float>(norms.rn.base, norms.rn.stride), dE, dS, dSE, dSW, st);
+  return launch_css_phi(p, ft, phi, strided<const float>(norms.rn.base, norms.rn.stride), dE, dS, dSE, dSW, st,
+                        text_nan);
 }
 
 cudaError_t launch_css_phi(const Problem& p, const FrameTable& ft, Strided<float> phi, Strided<const float> rn,
                            Strided<float> dE, Strided<float> dS, Strided<float> dSE, Strided<float> dSW,
-                           cudaStream_t st) {
+                           cudaStream_t st, bool text_nan) {
   if (ft.ctile0[ft.n_frames] == 0) return cudaSuccess;
   const CssDots d = {dE, dS, dSE, dSW};
   int cmax = 1;  // the most kPhiRun-cell runs of any frame
   for (int f = 0; f < ft.n_frames; ++f) cmax = max(cmax, ft.gh[f] * ((ft.gw[f] + kPhiRun - 1) / kPhiRun));
   TimingScope ts("css_phi", st);
-  k_css_phi<<<dim3((cmax + 255) / 256, ft.n_frames, p.L * p.hkv), 256, 0, st>>>(ft, p.hkv, d, rn, phi);
+  k_css_phi<<<dim3((cmax + 255) / 256, ft.n_frames, p.L * p.hkv), 256, 0, st>>>(ft, p.hkv, d, rn, phi,
+                                                                                        text_nan ? 1 : 0);
   return cudaGetLastError();
 }
 
