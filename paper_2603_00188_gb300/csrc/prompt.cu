@@ -40,6 +40,7 @@
 
 #include "kernels.cuh"
 #include "ptx.cuh"
+#include "tile.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -544,120 +545,121 @@ __global__ void __maxnreg__(kPrMaxReg)
 }
 
 // ---- fp32 caches: the same two passes on the CUDA cores --------------------
-// Pass 1: one CTA of 128 threads per (query row, KV head); each thread keeps
-// an online (max, sum of 2^(x c - max c)) over its strided keys j <= pos, and
-// the block merges the threads' states in a fixed order.
-constexpr int kPrSimtRows = 128;
-__global__ void __launch_bounds__(kPrSimtRows) k_prompt_rowstats_simt(const float* __restrict__ q,
-                                                                     const float* __restrict__ k, PromptArgs a,
-                                                                     float* bias) {
-  __shared__ float qs[kD];
-  __shared__ float2 st[kPrSimtRows];
-  const int row = blockIdx.x, h = blockIdx.y, tid = threadIdx.x;
-  const int prel = row / a.G, gq = row - prel * a.G;
-  const int pos = a.n - a.nq + prel;
-  const float c = kPrLog2e * rsqrtf((float)kD);
-  qs[tid] = q[((size_t)prel * a.hq + h * a.G + gq) * kD + tid];
-  __syncthreads();
-  float m = -CUDART_INF_F, l = 0.f;
-  for (int j = tid; j <= pos; j += kPrSimtRows) {
-    const float4* kr = reinterpret_cast<const float4*>(k + ((size_t)j * a.hkv + h) * kD);
-    float d = 0.f;
-#pragma unroll 8
-    for (int e = 0; e < kD / 4; ++e) {
-      const float4 kv = __ldg(kr + e);
-      d = fmaf(kv.x, qs[4 * e], d);
-      d = fmaf(kv.y, qs[4 * e + 1], d);
-      d = fmaf(kv.z, qs[4 * e + 2], d);
-      d = fmaf(kv.w, qs[4 * e + 3], d);
-    }
-    const float x = d * c;
-    if (x > m) {
-      l = (m == -CUDART_INF_F ? 0.f : l * exp2f(m - x)) + 1.f;
-      m = x;
-    } else {
-      l += exp2f(x - m);
-    }
-  }
-  st[tid] = make_float2(m, l);
-  __syncthreads();
-  if (tid == 0) {
-    float mm = -CUDART_INF_F, ll = 0.f;
-    for (int t = 0; t < kPrSimtRows; ++t) {
-      const float2 s = st[t];
-      const float mn = fmaxf(mm, s.x);
-      if (mn == -CUDART_INF_F) continue;
-      ll = (mm == -CUDART_INF_F ? 0.f : ll * exp2f(mm - mn)) + (s.x == -CUDART_INF_F ? 0.f : s.y * exp2f(s.x - mn));
-      mm = mn;
-    }
-    const size_t at = ((size_t)h * a.n_ch + prel / a.p2) * a.crp + (size_t)(prel % a.p2) * a.G + gq;
-    bias[at] = -mm - log2f((float)a.G * ll);
-  }
+// Both are products of 64 x 64 tiles (tile.cuh).  1,152 positions of 28 heads:
+// row statistics 175 us, column sums 221; with a CTA per query row, each thread
+// reading keys from global memory, and one product at a time per thread from
+// shared memory they took 2,116 and 2,422.
+constexpr int kPrSimtSmem = 2 * kTileFloats * 4;
+
+// Query row r (position r / G of the prompt, head r % G of KV head h's group).
+__device__ __forceinline__ const float* prompt_row(const float* q, const PromptArgs& a, int h, int r) {
+  const int prel = r / a.G;
+  return q + ((size_t)prel * a.hq + h * a.G + (r - prel * a.G)) * kD;
+}
+// Where its bias lies.
+__device__ __forceinline__ size_t prompt_bias_at(const PromptArgs& a, int h, int r) {
+  const int prel = r / a.G;
+  return ((size_t)h * a.n_ch + prel / a.p2) * a.crp + (size_t)(prel % a.p2) * a.G + (r - prel * a.G);
 }
 
-// Pass 2: one CTA of 256 threads per (32-key tile, KV head).  The tile's keys
-// and, in turn, tiles of query rows (with their biases) sit in shared
-// memory (32-row tiles); thread t sums 2^(x c + bias_r) for key t % 32 over rows t / 32 + 8 i
-// that attend to it, and the eight partial sums of a key are added in a
-// fixed order.
-constexpr int kPrSimtKeys = 32, kPrSimtRowTile = 32, kPrSimtThreads = 256;
-__global__ void __launch_bounds__(kPrSimtThreads) k_prompt_colsum_simt(const float* __restrict__ q,
-                                                                      const float* __restrict__ k, PromptArgs a,
-                                                                      const float* bias, float* a_out) {
-  __shared__ float ks[kPrSimtKeys][kD + 1];
-  __shared__ float qs[kPrSimtRowTile][kD + 1];
-  __shared__ float bs[kPrSimtRowTile];
-  __shared__ float part[kPrSimtThreads];
-  const int h = blockIdx.y, tid = threadIdx.x, j0 = blockIdx.x * kPrSimtKeys;
-  const int kk = tid % kPrSimtKeys, rsub = tid / kPrSimtKeys;
-  const int j = j0 + kk;
-  const int p_first = a.n - a.nq;
+// Pass 1: a CTA per (64 query rows, KV head), longest rows first.
+__global__ void __launch_bounds__(kTileThreads, kTilesPerSm) k_prompt_rowstats_simt(const float* __restrict__ q,
+                                                                                   const float* __restrict__ k,
+                                                                                   PromptArgs a, float* bias) {
+  extern __shared__ float4 tile_smem[];
+  float* qs = reinterpret_cast<float*>(tile_smem);
+  float* ks = qs + kTileFloats;
+  const int h = blockIdx.y, r0 = (int)(gridDim.x - 1 - blockIdx.x) * kTileRows, rows = a.nq * a.G;
+  const int nr = min(kTileRows, rows - r0), p_first = a.n - a.nq, ty = tile_ty(), tx = tile_tx();
   const float c = kPrLog2e * rsqrtf((float)kD);
-  for (int e = tid; e < kPrSimtKeys * kD; e += kPrSimtThreads) {
-    const int r = e / kD, d = e % kD;
-    ks[r][d] = j0 + r < a.n ? k[((size_t)(j0 + r) * a.hkv + h) * kD + d] : 0.f;
+  tile_load(qs, nr, [&](int r) { return prompt_row(q, a, h, r0 + r); });
+  float m[kTA], l[kTA];
+  int pos[kTA];  // last key of the thread's rows
+#pragma unroll
+  for (int i = 0; i < kTA; ++i) {
+    m[i] = -CUDART_INF_F;
+    l[i] = 0.f;
+    pos[i] = p_first + (r0 + min(ty + 8 * i, nr - 1)) / a.G;
   }
-  const int rows = a.nq * a.G;
+  const int kend = p_first + (r0 + nr - 1) / a.G + 1;  // keys that some row sees
+  for (int j0 = 0; j0 < kend; j0 += kTileRows) {
+    tile_load(ks, min(kTileRows, kend - j0), [&](int r) { return k + ((size_t)(j0 + r) * a.hkv + h) * kD; });
+    tile_ready();
+    float d[kTA][kTB];
+    tile_dots(qs, ks, d);
+#pragma unroll
+    for (int i = 0; i < kTA; ++i) {
+#pragma unroll
+      for (int j = 0; j < kTB; ++j) d[i][j] = j0 + tx + 16 * j <= pos[i] ? d[i][j] * c : -CUDART_INF_F;
+      fold_scores(m[i], l[i], d[i]);
+    }
+    __syncthreads();  // the key tile is rewritten
+  }
+  merge_rows(m, l, ks);
+  if (tx == 0)
+#pragma unroll
+    for (int i = 0; i < kTA; ++i) {
+      const int r = ty + 8 * i;
+      if (r < nr) bias[prompt_bias_at(a, h, r0 + r)] = -m[i] - log2f((float)a.G * l[i]);
+    }
+}
+
+// Pass 2: a cluster of CTAs per (64 keys, KV head), each taking every split-th
+// tile of the query rows that can see the keys; their sums are added in rank
+// order.
+__global__ void __launch_bounds__(kTileThreads, kTilesPerSm) k_prompt_colsum_simt(const float* __restrict__ q,
+                                                                                 const float* __restrict__ k,
+                                                                                 PromptArgs a, const float* bias,
+                                                                                 float* a_out) {
+  extern __shared__ float4 tile_smem[];
+  float* ks = reinterpret_cast<float*>(tile_smem);
+  float* qs = ks + kTileFloats;
+  cg::cluster_group cl = cg::this_cluster();
+  const int split = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int h = blockIdx.y, j0 = (int)blockIdx.x / split * kTileRows, rows = a.nq * a.G;
+  const int p_first = a.n - a.nq, ty = tile_ty(), tx = tile_tx();
+  const float c = kPrLog2e * rsqrtf((float)kD);
   const int r_start = j0 <= p_first ? 0 : (j0 - p_first) * a.G;  // rows before it see no key of the tile
-  float acc = 0.f;
-  for (int r0 = r_start; r0 < rows; r0 += kPrSimtRowTile) {
-    __syncthreads();
-    for (int e = tid; e < kPrSimtRowTile * kD; e += kPrSimtThreads) {
-      const int r = e / kD, d = e % kD, row = r0 + r;
-      float v = 0.f;
-      if (row < rows) {
-        const int prel = row / a.G, gq = row - prel * a.G;
-        v = q[((size_t)prel * a.hq + h * a.G + gq) * kD + d];
-      }
-      qs[r][d] = v;
+  tile_load(ks, min(kTileRows, a.n - j0), [&](int r) { return k + ((size_t)(j0 + r) * a.hkv + h) * kD; });
+  float acc[kTA];
+#pragma unroll
+  for (int i = 0; i < kTA; ++i) acc[i] = 0.f;
+  for (int rt = r_start + rank * kTileRows; rt < rows; rt += split * kTileRows) {
+    const int nr = min(kTileRows, rows - rt);
+    tile_load(qs, nr, [&](int r) { return prompt_row(q, a, h, rt + r); });
+    float bs[kTB];
+    int pos[kTB];  // last key of the thread's rows; -1: no row
+#pragma unroll
+    for (int j = 0; j < kTB; ++j) {
+      const int r = tx + 16 * j;
+      bs[j] = r < nr ? __ldg(bias + prompt_bias_at(a, h, rt + r)) : 0.f;
+      pos[j] = r < nr ? p_first + (rt + r) / a.G : -1;
     }
-    for (int r = tid; r < kPrSimtRowTile; r += kPrSimtThreads) {
-      const int row = r0 + r;
-      float b = -CUDART_INF_F;
-      if (row < rows) {
-        const int prel = row / a.G, gq = row - prel * a.G;
-        b = bias[((size_t)h * a.n_ch + prel / a.p2) * a.crp + (size_t)(prel % a.p2) * a.G + gq];
-      }
-      bs[r] = b;
+    tile_ready();
+    float d[kTA][kTB];
+    tile_dots(ks, qs, d);
+#pragma unroll
+    for (int i = 0; i < kTA; ++i) {
+      float sum = 0.f;
+#pragma unroll
+      for (int j = 0; j < kTB; ++j) sum += j0 + ty + 8 * i <= pos[j] ? exp2f(fmaf(d[i][j], c, bs[j])) : 0.f;
+      acc[i] += sum;
     }
-    __syncthreads();
-    for (int r = rsub; r < kPrSimtRowTile; r += kPrSimtThreads / kPrSimtKeys) {
-      const int row = r0 + r;
-      if (row >= rows || p_first + row / a.G < j) continue;  // past the rows, or before key j
-      float d = 0.f;
-#pragma unroll 8
-      for (int e = 0; e < kD; ++e) d = fmaf(ks[kk][e], qs[r][e], d);
-      acc += exp2f(fmaf(d, c, bs[r]));
-    }
+    __syncthreads();  // the query tile is rewritten
   }
-  part[tid] = acc;
-  __syncthreads();
-  if (rsub == 0 && j < a.n) {
-    float s = 0.f;
-    for (int t = 0; t < kPrSimtThreads / kPrSimtKeys; ++t) s += part[t * kPrSimtKeys + kk];
-    if (a.mode == 1) s /= (float)min(a.nq, a.n - j);
-    a_out[(size_t)h * a.n + j] = s;
+  sum_rows(acc, qs);
+  if (split > 1)
+    cl.sync();
+  else
+    __syncthreads();
+  const int j = j0 + threadIdx.x;
+  if (rank == 0 && threadIdx.x < kTileRows && j < a.n) {
+    float sum = qs[threadIdx.x];
+    for (int r = 1; r < split; ++r) sum += cl.map_shared_rank(qs, r)[threadIdx.x];
+    if (a.mode == 1) sum /= (float)min(a.nq, a.n - j);
+    a_out[(size_t)h * a.n + j] = sum;
   }
+  if (split > 1) cl.sync();  // no CTA leaves while rank 0 may still read its sums
 }
 
 // ---- host --------------------------------------------------------------
@@ -749,16 +751,37 @@ cudaError_t launch_prompt_score(DType dt, const void* q, const void* k, int n, i
     cudaError_t e;
     const float* qf = static_cast<const float*>(q);
     const float* kf = static_cast<const float*>(k);
+    const int rows = nq * a.G, ktiles = (n + kTileRows - 1) / kTileRows, rtiles = (rows + kTileRows - 1) / kTileRows;
+    if ((e = cudaFuncSetAttribute(k_prompt_rowstats_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, kPrSimtSmem)) !=
+            cudaSuccess ||
+        (e = cudaFuncSetAttribute(k_prompt_colsum_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, kPrSimtSmem)) !=
+            cudaSuccess)
+      return e;
     {
       TimingScope ts("prompt_rowstats_simt", st);
-      k_prompt_rowstats_simt<<<dim3((unsigned)(nq * a.G), hkv), kPrSimtRows, 0, st>>>(qf, kf, a, bias);
+      k_prompt_rowstats_simt<<<dim3((unsigned)rtiles, hkv), kTileThreads, kPrSimtSmem, st>>>(qf, kf, a, bias);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // CTAs per key tile: while the CTAs fill the SMs less than four times (the
+    // first tiles see every row, the last ones few), at most one per row tile
+    int split = 1;
+    while (2 * split <= rtiles && 2 * split <= kP2MaxSplit &&
+           (long long)ktiles * hkv * 2 * split <= 4 * 152 * kTilesPerSm)
+      split *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3((unsigned)(ktiles * split), hkv);
+    cfg.blockDim = dim3(kTileThreads);
+    cfg.dynamicSmemBytes = kPrSimtSmem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)split;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
     TimingScope ts("prompt_colsum_simt", st);
-    k_prompt_colsum_simt<<<dim3((unsigned)((n + kPrSimtKeys - 1) / kPrSimtKeys), hkv), kPrSimtThreads, 0, st>>>(
-        qf, kf, a, bias, a_out);
-    (void)err;
-    return cudaGetLastError();
+    e = cudaLaunchKernelEx(&cfg, k_prompt_colsum_simt, qf, kf, a, (const float*)bias, a_out);
+    return e != cudaSuccess ? e : cudaGetLastError();
   }
   PromptMaps maps;
   cudaError_t e = make_prompt_qmap(&maps.q1, q, nq, hq, a.G, a.p1);

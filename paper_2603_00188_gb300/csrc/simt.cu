@@ -5,6 +5,7 @@
 #include <cooperative_groups.h>
 
 #include "kernels.cuh"
+#include "tile.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -444,91 +445,6 @@ cudaError_t launch_fill_text_nan(const Problem& p, const FrameTable& ft, float* 
   return cudaGetLastError();
 }
 
-// ------------------------------------------------ fp32 tile products
-// The fp32 passes below are products of two sets of 128-wide rows, bound by
-// the FMA pipe.  A CTA of 128 threads forms the 64 x 64 dot products of two
-// row sets in shared memory (rows padded to 132 floats, so that a warp's four
-// rows of A or eight of B lie in different banks), eight x four per thread:
-// per four dimensions, twelve 16-byte shared loads feed 64 packed
-// multiply-adds.  67.6 KB let three CTAs share an SM; one's copies hide behind
-// the others' products.  Even and odd dimensions accumulate apart (the two
-// halves of fma.rn.f32x2), each in ascending order, and are added last.
-// The product alone reaches 50 TFLOP/s of the FMA pipe's 76 (8 x 8 per thread:
-// 52, but two CTAs of half the warps; 4 x 8: 48; unpacked fmaf: the same).
-// One layer of 5 frames of 36 x 64 (11,840 keys, 4 heads of 224 query rows),
-// against one dot product per thread with both operands read from shared
-// memory for every multiply-add: TSG 2,036 -> 483 us (45 TFLOP/s), row
-// statistics 389 -> 94, column sums 466 -> 89; 1,152 keys: 201 -> 15, 90 -> 18
-// and 195 -> 29.
-constexpr int kTileRows = 64;
-constexpr int kTileThreads = 128;
-constexpr int kTilePitch = kD + 4;  // floats
-constexpr int kTileFloats = kTileRows * kTilePitch;
-constexpr int kTA = 8, kTB = 4;  // rows of A and B per thread
-constexpr int kTilesPerSm = 3;
-
-// The thread's rows: ty + 8 i of A, tx + 16 j of B.  A warp holds four ty
-// and eight tx; warps 2 and 3 have the other four ty, odd warps the other tx.
-__device__ __forceinline__ int tile_ty() { return ((threadIdx.x >> 3) & 3) + 4 * (threadIdx.x >> 6); }
-__device__ __forceinline__ int tile_tx() { return (threadIdx.x & 7) + 8 * ((threadIdx.x >> 5) & 1); }
-
-// Starts the copy of rows src(0) .. src(nrows - 1) (512 bytes each) into a
-// tile; the rows after them become zero.  A warp copies one row at a time.
-template <class Src>
-__device__ __forceinline__ void tile_load(float* dst, int nrows, Src src) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll 4
-  for (int r = threadIdx.x >> 5; r < kTileRows; r += kTileThreads / 32) {
-    float* d = dst + r * kTilePitch + 4 * lane;
-    if (r < nrows) {
-      const uint32_t da = static_cast<uint32_t>(__cvta_generic_to_shared(d));
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(da), "l"(src(r) + 4 * lane) : "memory");
-    } else {
-      *reinterpret_cast<float4*>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-  }
-}
-// Every copy of the CTA has landed (and every thread's use of the tiles
-// before this call is over).
-__device__ __forceinline__ void tile_ready() {
-  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-  __syncthreads();
-}
-
-// d[i][j] = A row (ty + 8 i) . B row (tx + 16 j)
-__device__ __forceinline__ void tile_dots(const float* a, const float* b, float (&d)[kTA][kTB]) {
-  const float* ap = a + tile_ty() * kTilePitch;
-  const float* bp = b + tile_tx() * kTilePitch;
-  unsigned long long acc[kTA][kTB];
-#pragma unroll
-  for (int i = 0; i < kTA; ++i)
-#pragma unroll
-    for (int j = 0; j < kTB; ++j) acc[i][j] = 0ull;
-#pragma unroll 4
-  for (int k = 0; k < kD; k += 4) {
-    ulonglong2 y[kTB];
-#pragma unroll
-    for (int j = 0; j < kTB; ++j) y[j] = *reinterpret_cast<const ulonglong2*>(bp + 16 * j * kTilePitch + k);
-#pragma unroll
-    for (int i = 0; i < kTA; ++i) {
-      const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(ap + 8 * i * kTilePitch + k);
-#pragma unroll
-      for (int j = 0; j < kTB; ++j) {
-        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][j]) : "l"(x.x), "l"(y[j].x));
-        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][j]) : "l"(x.y), "l"(y[j].y));
-      }
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < kTA; ++i)
-#pragma unroll
-    for (int j = 0; j < kTB; ++j) {
-      float lo, hi;
-      asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[i][j]));
-      d[i][j] = lo + hi;
-    }
-}
-
 // ------------------------------------------------------- row statistics
 // Window score, first pass (fp32): for every query row r of KV head h (r =
 // window row * G + group member) the maximum m and sum l of 2^(x - m), x =
@@ -542,19 +458,6 @@ constexpr int kScoreSimtSmem = 2 * kTileFloats * 4;
 __device__ __forceinline__ const float* q_row(const float* q, const Problem& p, int h, int r) {
   const int G = p.G(), wr = r / G;
   return q + ((size_t)wr * p.hq + h * G + (r - wr * G)) * kD;
-}
-
-// (m, l) <- the states (m, l) and (m2, l2) together; l = 0: an empty state.
-__device__ __forceinline__ void merge_state(float& m, float& l, float m2, float l2) {
-  if (l2 == 0.f) return;
-  if (l == 0.f) {
-    m = m2;
-    l = l2;
-    return;
-  }
-  const float mn = fmaxf(m, m2);
-  l = (m == mn ? l : l * exp2f(m - mn)) + (m2 == mn ? l2 : l2 * exp2f(m2 - mn));
-  m = mn;
 }
 
 __global__ void __launch_bounds__(kTileThreads, kTilesPerSm)
@@ -585,41 +488,16 @@ __global__ void __launch_bounds__(kTileThreads, kTilesPerSm)
     tile_dots(qs, ks, d);
 #pragma unroll
     for (int i = 0; i < kTA; ++i) {
-      float mn = m[i];
 #pragma unroll
-      for (int j = 0; j < kTB; ++j) {
-        d[i][j] = tx + 16 * j < nk ? d[i][j] * c : -CUDART_INF_F;
-        mn = fmaxf(mn, d[i][j]);
-      }
-      if (mn != -CUDART_INF_F) {  // no key yet otherwise
-        float sum = 0.f;
-#pragma unroll
-        for (int j = 0; j < kTB; ++j) sum += d[i][j] == mn ? 1.f : exp2f(d[i][j] - mn);
-        ls[i] = (m[i] == mn ? ls[i] : ls[i] * exp2f(m[i] - mn)) + sum;
-        m[i] = mn;
-      }
+      for (int j = 0; j < kTB; ++j) d[i][j] = tx + 16 * j < nk ? d[i][j] * c : -CUDART_INF_F;
+      fold_scores(m[i], ls[i], d[i]);
     }
     __syncthreads();  // the key tile is rewritten
   }
-  // a row's states: eight lanes of each of two warps
-#pragma unroll
-  for (int i = 0; i < kTA; ++i)
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
-      const float m2 = __shfl_xor_sync(0xffffffffu, m[i], o), l2 = __shfl_xor_sync(0xffffffffu, ls[i], o);
-      merge_state(m[i], ls[i], m2, l2);
-    }
-  tile_ready();  // also when the split was empty: the query rows' copies end before the CTA does
-  float2* xch = reinterpret_cast<float2*>(ks);
-  if (tx == 8)
-#pragma unroll
-    for (int i = 0; i < kTA; ++i) xch[ty + 8 * i] = make_float2(m[i], ls[i]);
-  __syncthreads();
+  merge_rows(m, ls, ks);
   if (tx == 0)
 #pragma unroll
     for (int i = 0; i < kTA; ++i) {
-      const float2 o = xch[ty + 8 * i];
-      merge_state(m[i], ls[i], o.x, o.y);
       const int row = r0 + ty + 8 * i;
       if (row < R) part[((size_t)h * nsplit + s) * R + row] = make_float2(m[i], ls[i]);
     }
@@ -690,18 +568,7 @@ __global__ void __launch_bounds__(kTileThreads, kTilesPerSm)
     }
     __syncthreads();  // the query tile is rewritten
   }
-#pragma unroll
-  for (int i = 0; i < kTA; ++i)
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
-  tile_ready();  // also for a CTA without query rows, whose key copies are still in flight
-  if (tx == 8)
-#pragma unroll
-    for (int i = 0; i < kTA; ++i) qs[ty + 8 * i] = acc[i];
-  __syncthreads();
-  if (tx == 0)
-#pragma unroll
-    for (int i = 0; i < kTA; ++i) qs[ty + 8 * i] += acc[i];
+  sum_rows(acc, qs);
   if (split > 1)
     cl.sync();
   else
