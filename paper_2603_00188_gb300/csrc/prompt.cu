@@ -31,7 +31,7 @@
 // Both passes are bound by their epilogues (0.9 and 1.1 us per 128 x 256 item,
 // the MMA alone 0.66).  8,576 positions, 28 query heads (one layer), with one
 // CTA per m-tile and per key tile, the biases in the query rows' stages and a
-// kernel that filled the bias array first: 6 + 210 + 255 us; now 196 + 241.
+// kernel that filled the bias array first: 6 + 210 + 255 us; now 187 + 241.
 #include <cooperative_groups.h>
 #include <cudaTypedefs.h>
 
@@ -127,9 +127,15 @@ __global__ void __maxnreg__(kPrMaxReg)
   uint8_t* sm = pr_align1024(smem_raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // work item i: KV head i % hkv, m-tile n_mt - 1 - i / hkv (longest rows
-  // first); CTA b takes items b, b + grid, ...  An item's rows are positions
-  // [pr0, pr0 + npos), its keys [0, p_first + pr0 + npos).
+  // first).  The CTAs take a grid's worth of items per round, in turn from the
+  // first to the last CTA and back: always in the same order, the first CTA
+  // had 16 % more keys than the last (8,576 positions: 197 us, now 187).  An
+  // item's rows are positions [pr0, pr0 + npos), its keys [0, p_first + pr0 +
+  // npos).
   const int n_items = a.n_mt * a.hkv, p_first = a.n - a.nq;
+  auto item = [&](int round) {
+    return round * (int)gridDim.x + (int)(round & 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+  };
   auto item_pr0 = [&](int i) { return (a.n_mt - 1 - i / a.hkv) * a.p1; };
   auto item_tiles = [&](int pr0) { return (p_first + pr0 + min(a.p1, a.nq - pr0) + 255) / 256; };
   const uint32_t sQ = smem_u32(sm + kP1Q), sK = smem_u32(sm + kP1K);
@@ -178,7 +184,7 @@ __global__ void __maxnreg__(kPrMaxReg)
       int ks = 0, qi = 0;  // key stage; items so far
       uint32_t kp = 0u;
       bool ok = true;
-      for (int i = blockIdx.x; ok && i < n_items; i += gridDim.x, ++qi) {
+      for (int i = item(0); ok && i < n_items; i = item(++qi)) {
         const int qs = qi & 1, h = i % a.hkv, pr0 = item_pr0(i), ntiles = item_tiles(pr0);
         if (!mbar_wait(b_qempty + 8 * qs, ((uint32_t)(qi >> 1) & 1u) ^ 1u, err, abort_flag)) break;
         mbar_arrive_expect_tx(b_qfull + 8 * qs, qbytes);
@@ -209,7 +215,7 @@ __global__ void __maxnreg__(kPrMaxReg)
       bool ok = true;
       int ks = 0, qi = 0, u = 0;  // key stage; items, key tiles so far
       uint32_t kp = 0u;
-      for (int i = blockIdx.x; ok && i < n_items; i += gridDim.x, ++qi) {
+      for (int i = item(0); ok && i < n_items; i = item(++qi)) {
         const int qs = qi & 1, ntiles = item_tiles(item_pr0(i));
         if (!mbar_wait(b_qfull + 8 * qs, (uint32_t)(qi >> 1) & 1u, err, abort_flag)) break;
         for (int it = 0; it < ntiles;
@@ -242,8 +248,8 @@ __global__ void __maxnreg__(kPrMaxReg)
     const int g = (warp - 2) >> 2, quarter = warp & 3, row = quarter * 32 + lane;
     const uint32_t lanebase = tmem + ((uint32_t)(quarter * 32) << 16) + g * 64;
     bool live = true;  // after a wait gave up every warp still meets the others at each item's end
-    int u = 0, xb = 0;
-    for (int i = blockIdx.x; i < n_items; i += gridDim.x, xb ^= 1) {
+    int u = 0, round = 0;
+    for (int i = item(0); i < n_items; i = item(++round)) {
     const int h = i % a.hkv, pr0 = item_pr0(i), ntiles = item_tiles(pr0);
     const int pa = p_first + pr0, rows = min(a.p1, a.nq - pr0) * a.G, pos = pa + row / a.G;
     float m = -CUDART_INF_F, l = 0.f;
@@ -308,7 +314,7 @@ __global__ void __maxnreg__(kPrMaxReg)
     }
     // merge the four groups' states per row in group order (two exchange
     // buffers in turn: one is rewritten after the other's barrier)
-    float2* xp = xch + xb * kPrGroups * 128;
+    float2* xp = xch + (round & 1) * kPrGroups * 128;
     xp[g * 128 + row] = make_float2(m, l);
     epilogue_sync();
     if (g == 0 && row < rows && live && !*abort_flag) {
