@@ -269,27 +269,44 @@ cudaError_t launch_css(const Problem& p, const FrameTable& ft, const LayerPtrs& 
 // the box sum separates into row sums and a sum of 2R+1 rows.  A CTA (tile,
 // frame, layer*Hkv + head) stages kBoxRows x kBoxCols output cells plus an
 // R-cell halo (out-of-grid cells as zero keys with rn = 0, so they add
-// nothing); each 16-lane half-warp owns one output column, 8 dimensions per
-// lane, walks the tile's rows once and keeps the last 2R+1 row sums in
-// registers.  rn of a cell uses the same operation sequence as the norms
-// kernel, so both agree bit for bit.
-constexpr int kBoxRows = 8, kBoxCols = 16, kBoxThreads = 256;
+// nothing); 16 or 32 lanes own a pair of adjacent output columns, walk the
+// tile's rows once and keep the last 2R+1 row sums in registers.  rn of a cell
+// uses the same operation sequence as the norms kernel, so both agree bit for
+// bit.  Bound by issue slots and shared-memory reads: a pair reads a row's
+// 2R+2 cells once where two single columns read 4R+2, and the sums use packed
+// fp32x2 operations (each half rounded as a scalar one).  5x5 over 28 layers
+// of 53,600 bf16 tokens: 1,141 -> 925 us; 9x9: 2,000 -> 1,640; fp32, 23,104
+// tokens: 61 -> 52 us.  16 lanes (8 dimensions each) for the small bf16 boxes;
+// else 32: with twice the warps and half the registers 7x7 takes 1,320 us, not
+// 1,426, and fp32, whose 127 KB tile leaves one CTA per SM, 52 us, not 71 (5x5
+// bf16: 987, not 925).
+constexpr int kBoxRows = 8, kBoxCols = 16;
+
+// two fp32 values of a packed fp32x2 operand, first in the low half
+__device__ __forceinline__ uint64_t pack_f2(float x, float y) {
+  return (uint64_t)__float_as_uint(y) << 32 | __float_as_uint(x);
+}
+__device__ __forceinline__ float2 unpack_f2(uint64_t v) {
+  return make_float2(__uint_as_float((uint32_t)v), __uint_as_float((uint32_t)(v >> 32)));
+}
 
 template <typename T, int R>
 struct BoxGeom {
   static constexpr int TH = kBoxRows + 2 * R, TW = kBoxCols + 2 * R, cells = TH * TW;
   static constexpr int stride = kD * (int)sizeof(T) + 16;  // padded key row
   static constexpr int smem = cells * stride + cells * 4;
+  static constexpr int lanes = sizeof(T) == 2 && R <= 2 ? 16 : 32;  // of a pair of columns
+  static constexpr int threads = kBoxCols / 2 * lanes;
 };
 
 template <typename T, int R>
-__global__ void __launch_bounds__(kBoxThreads) k_css_box(const __grid_constant__ LayerPtrs io,
+__global__ void __launch_bounds__(BoxGeom<T, R>::threads) k_css_box(const __grid_constant__ LayerPtrs io,
                                                          const __grid_constant__ FrameTable ft, int hkv,
                                                          Strided<float> phi_all, NormsOut norms) {
   using Gm = BoxGeom<T, R>;
   constexpr int kChunks = kD * (int)sizeof(T) / 16;
   constexpr int kPer = 16 / (int)sizeof(T);
-  constexpr int TW = Gm::TW, TH = Gm::TH, D2 = 2 * R + 1;
+  constexpr int TW = Gm::TW, TH = Gm::TH, D2 = 2 * R + 1, kLanes = Gm::lanes;
   extern __shared__ float4 box_smem[];
   uint8_t* keys = reinterpret_cast<uint8_t*>(box_smem);
   float* rn = reinterpret_cast<float*>(keys + (size_t)Gm::cells * Gm::stride);
@@ -342,60 +359,76 @@ __global__ void __launch_bounds__(kBoxThreads) k_css_box(const __grid_constant__
     rn[cell] = r;
   }
   __syncthreads();
-  // box sums: lane group (16 lanes) = output column, 8 dimensions per lane
-  const int dg = tid & 15, col = tid >> 4;
-  const int v = v0 + col;
+  // box sums: kLanes lanes = a pair of output columns
+  constexpr int kPairs = kD / kLanes / 2;  // a lane's dimensions, in pairs
+  const int dg = tid % kLanes, col = 2 * (tid / kLanes);
   float* phi = phi_all.at(l);
-  auto load8 = [&](int cell, float (&x)[8]) {
-    const uint8_t* p0 = keys + (size_t)cell * Gm::stride + dg * 8 * (int)sizeof(T);
-#pragma unroll
-    for (int c = 0; c < 8 / kPer; ++c) {
+  auto load = [&](int cell, uint64_t (&x)[kPairs]) {
+    const uint8_t* p0 = keys + (size_t)cell * Gm::stride + dg * kPairs * 2 * (int)sizeof(T);
+    if constexpr (kPairs * 2 * sizeof(T) == 8) {  // 4 bf16
+      const uint2 w = *reinterpret_cast<const uint2*>(p0);
+      x[0] = pack_f2(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u));
+      x[1] = pack_f2(__uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
+    } else {
       float y[kPer];
-      unpack16<T>(*reinterpret_cast<const uint4*>(p0 + 16 * c), y);
+      unpack16<T>(*reinterpret_cast<const uint4*>(p0), y);
 #pragma unroll
-      for (int t = 0; t < kPer; ++t) x[c * kPer + t] = y[t];
+      for (int t = 0; t < kPairs; ++t) x[t] = pack_f2(y[2 * t], y[2 * t + 1]);
     }
   };
-  float ring[D2][8];
+  uint64_t ring[D2][2][kPairs];  // the last 2R+1 row sums of the two columns
 #pragma unroll
   for (int a = 0; a < TH; ++a) {
-    float hs[8];
+    uint64_t(&hs)[2][kPairs] = ring[a % D2];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) hs[e] = 0.f;
+    for (int e = 0; e < kPairs; ++e) hs[0][e] = hs[1][e] = 0ull;
 #pragma unroll
-    for (int dv = 0; dv < D2; ++dv) {
+    for (int dv = 0; dv <= D2; ++dv) {
       const int cell = a * TW + col + dv;
       const float r = rn[cell];
-      float x[8];
-      load8(cell, x);
+      const uint64_t rr = pack_f2(r, r);
+      uint64_t x[kPairs];
+      load(cell, x);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) hs[e] = fmaf(r, x[e], hs[e]);
+      for (int e = 0; e < kPairs; ++e) {
+        if (dv < D2) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(hs[0][e]) : "l"(rr), "l"(x[e]));
+        if (dv > 0) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(hs[1][e]) : "l"(rr), "l"(x[e]));
+      }
     }
-#pragma unroll
-    for (int e = 0; e < 8; ++e) ring[a % D2][e] = hs[e];
     if (a >= 2 * R) {
       const int o = a - 2 * R;  // output row of the tile
-      const int cell = (o + R) * TW + col + R;
-      const float ri = rn[cell];
-      float x[8];
-      load8(cell, x);
-      float dot = 0.f;
+      float dot[2];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        float s = ring[0][e];
+      for (int c = 0; c < 2; ++c) {
+        const int cell = (o + R) * TW + col + c + R;
+        const float nr = -rn[cell];
+        const uint64_t rr = pack_f2(nr, nr);
+        uint64_t x[kPairs];
+        load(cell, x);
+        dot[c] = 0.f;
 #pragma unroll
-        for (int q = 1; q < D2; ++q) s += ring[q][e];
-        const float kh = ri * x[e];
-        dot = fmaf(kh, s - kh, dot);
+        for (int e = 0; e < kPairs; ++e) {
+          uint64_t s = ring[0][c][e], nk;  // nk = -khat
+#pragma unroll
+          for (int q = 1; q < D2; ++q) asm("add.rn.f32x2 %0, %0, %1;" : "+l"(s) : "l"(ring[q][c][e]));
+          asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(nk) : "l"(rr), "l"(x[e]));
+          asm("add.rn.f32x2 %0, %0, %1;" : "+l"(s) : "l"(nk));
+          const float2 sf = unpack_f2(s), kf = unpack_f2(nk);
+          dot[c] = fmaf(-kf.x, sf.x, dot[c]);
+          dot[c] = fmaf(-kf.y, sf.y, dot[c]);
+        }
       }
+      // the lower half of the lanes goes on with the first column, the upper half with the second
+      const bool up = dg & (kLanes / 2);
+      float d = (up ? dot[1] : dot[0]) + __shfl_xor_sync(0xffffffffu, up ? dot[0] : dot[1], kLanes / 2);
 #pragma unroll
-      for (int m = 8; m > 0; m >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, m);
-      const int u = u0 + o;
-      if (dg == 0 && u < gh && v < gw) {
+      for (int m = kLanes / 4; m > 0; m >>= 1) d += __shfl_xor_sync(0xffffffffu, d, m);
+      const int u = u0 + o, v = v0 + col + (up ? 1 : 0);
+      if (dg % (kLanes / 2) == 0 && u < gh && v < gw) {
         const int nu = min(u + R, gh - 1) - max(u - R, 0) + 1;
         const int nv = min(v + R, gw - 1) - max(v - R, 0) + 1;
         const int cnt = nu * nv - 1;
-        phi[(size_t)h * n + off + u * gw + v] = cnt ? 1.0f - dot / (float)cnt : 0.0f;
+        phi[(size_t)h * n + off + u * gw + v] = cnt ? 1.0f - d / (float)cnt : 0.0f;
       }
     }
   }
@@ -414,7 +447,7 @@ static cudaError_t css_box_t(const Problem& p, const FrameTable& ft, const Layer
   }
   TimingScope ts("css_box", st);
   dim3 grid((unsigned)tiles, (unsigned)(ft.n_frames > 0 ? ft.n_frames : 1), (unsigned)(p.L * p.hkv));
-  k_css_box<T, R><<<grid, kBoxThreads, Gm::smem, st>>>(io, ft, p.hkv, phi, norms);
+  k_css_box<T, R><<<grid, Gm::threads, Gm::smem, st>>>(io, ft, p.hkv, phi, norms);
   return cudaGetLastError();
 }
 
