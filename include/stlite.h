@@ -250,7 +250,7 @@ typedef struct {
 /* Algorithm 1 for n_layers layers of one sequence (one frame layout, one
  * budget), each layer compressed independently with its own window queries;
  * the result for every layer equals stlite_compress_layer's.  Each kernel
- * launch covers up to 32 layers at a time (with TSG and CSS on, eight
+ * launch covers up to 32 layers at a time (with TSG and CSS on, at most eight
  * launches per batch of up to 32 layers), so small per-layer stages (the
  * selections, the compaction) fill the GPU.  layers: HOST array
  * [n_layers].  ws: n_layers times stlite_workspace_size() bytes (layer l uses
