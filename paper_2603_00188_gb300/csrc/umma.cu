@@ -9,9 +9,8 @@
 // All three share one structure: warp 0 issues TMA loads of 128-byte-swizzled
 // key tiles, warp 1 issues tcgen05.mma into TMEM (fp32 accumulators), and
 // groups of four warps (one warp per TMEM lane quarter) drain TMEM with
-// tcgen05.ld and run the fp32 epilogue: two groups (warps 2-9) in TSG and
-// the column sums, four (warps 2-17) in the row statistics.  Every mbarrier
-// wait is bounded.
+// tcgen05.ld and run the fp32 epilogue: four groups (warps 2-17), two
+// (warps 2-9) in the saliency.  Every mbarrier wait is bounded.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -78,10 +77,20 @@ __device__ __forceinline__ void tsg_tile_next(const FrameTable& ft, int t, int& 
 // =========================================================================
 // TSG.  CTA (x, chunk, h): current-frame columns [512*chunk, 512*chunk+512)
 // of head h stay in shared memory (128 KB); historical row tiles of 128
-// tokens stream through two 32 KB stages.  TMEM holds the 128 x 512 fp32
-// product as two 256-column accumulator stages; epilogue group g owns stage g
-// and folds max_j acc_ij * rn_j over them into rho_key.  Columns past the
-// current frame carry rn = NaN, which fmaxf ignores.
+// tokens stream through three 32 KB stages.  TMEM holds the 128 x 512 fp32
+// product as two 256-column accumulator stages; two epilogue groups each drain
+// 128 columns of a stage, release it when their columns are in registers and
+// fold max_j acc_ij * rn_j into rho_key.  Columns past the current frame carry
+// rn = NaN, which fmaxf ignores.
+//
+// Bound by the tensor pipe and the exposed part of the drain; over many layers
+// by the power cap.  Against one group of four warps per stage (168 registers)
+// the drain is shorter, most of all where a frame fills part of its last
+// chunk: one layer of 20,736 historical rows and 2,304 columns 41.7 -> 39.6
+// us, three chunks of 1,296 125.7 -> 121.3, a 28-layer sequence of the small
+// backbone 152 -> 147, 28 x 50,176 rows and 1,024 columns 837 -> 819 (1,799
+// TFLOP/s) where the power cap leaves the clock alone.
+constexpr int kTsgThreads = 576, kTsgMaxReg = 96;  // TMA, MMA and four groups of four warps
 constexpr int kTsgB = 0;                  // [2][512][128 B]
 constexpr int kTsgAStages = 3;
 constexpr int kTsgA = 131072;                              // [3 stages][2][128][128 B]
@@ -94,7 +103,7 @@ constexpr int kTsgSmem = 232448;                           // the per-CTA maximu
 // |k_j|^2 (the row's own -|k_i|^2 is added by the selection kernel).  The
 // per-column term sits in rn_s (rn_j, 1, or -|k_j|^2), NaN past the frame.
 template <int METRIC>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __maxnreg__(kTsgMaxReg)
     k_tsg_umma(const __grid_constant__ KMaps maps, const __grid_constant__ FrameTable ft,
                Strided<const float> rc_all, int cur_pad, Strided<uint32_t> rho_all, int hkv, uint32_t* err) {
   extern __shared__ uint8_t smem_raw[];
@@ -130,7 +139,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(b_accfull + 8 * i, 1);
-      mbar_init(b_accempty + 8 * i, 4);
+      mbar_init(b_accempty + 8 * i, valid - i * 256 > 128 ? 8 : 4);
     }
     mbar_init(b_bfull, 1);
     mbar_init(b_done, 1);
@@ -143,7 +152,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_relinquish();
   }
   // inverse norms of this chunk's current-frame columns (NaN past the frame)
-  for (int c = (int)threadIdx.x - 64; c < 512; c += kThreads - 64) {
+  for (int c = (int)threadIdx.x - 64; c < 512; c += kTsgThreads - 64) {
     if (c >= 0) {
       float v = CUDART_NAN_F;
       if (c < valid) {
@@ -216,85 +225,52 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_wait_drain(b_done, 0);
     }
   } else {
-    const int g = (warp - 2) >> 2, quarter = warp & 3;
-    if (g < nst) {
-      const int valid_g = min(256, valid - g * 256);
-      const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + g * 256;
-      const float* rg = rn_s + g * 256;
+    // group g drains half g >> 1 (128 columns) of stage g & 1
+    const int grp = (warp - 2) >> 2, g = grp & 1, half = grp >> 1, quarter = warp & 3;
+    if (valid > g * 256 + half * 128) {
+      const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + g * 256 + half * 128;
+      const float* rg = rn_s + g * 256 + half * 128;
       int it = 0, tf = 0;
       for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++it) {
         if (!warp_wait(b_accfull + 8 * g, (uint32_t)it & 1u, err, abort_flag)) break;
         tc_fence_after();
-        float mx = -CUDART_INF_F;
-        if (valid_g > 192) {
-          // (nearly) full stage: packed products and 3-input max into eight
-          // independent running maxima (short dependency chains); a column
-          // past the frame carries rn = NaN, and the maximum ignores NaN,
-          // whatever is left in its TMEM column
-          float m[8];
+        // packed products and 3-input max into eight independent running
+        // maxima (short dependency chains); a column past the frame carries
+        // rn = NaN, and the maximum ignores NaN, whatever is left in its TMEM
+        // column (a second path for halves of few columns: within 2 %)
+        float m[8];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) m[i] = -CUDART_INF_F;
-          auto reduce = [&](const uint32_t (&v)[64], int c) {
-            const float4* r4 = reinterpret_cast<const float4*>(rg + c * 64);
+        for (int i = 0; i < 8; ++i) m[i] = -CUDART_INF_F;
+        auto reduce = [&](const uint32_t (&v)[64], int c) {
+          const float4* r4 = reinterpret_cast<const float4*>(rg + c * 64);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float4 r = r4[i];
-              const float v0 = __uint_as_float(v[4 * i]), v1 = __uint_as_float(v[4 * i + 1]);
-              const float v2 = __uint_as_float(v[4 * i + 2]), v3 = __uint_as_float(v[4 * i + 3]);
-              float p0, p1, p2, p3;
-              if (METRIC == kTsgNegL2) {
-                fma2(v0, v1, 2.f, 2.f, r.x, r.y, p0, p1);
-                fma2(v2, v3, 2.f, 2.f, r.z, r.w, p2, p3);
-              } else {
-                mul2(v0, v1, r.x, r.y, p0, p1);
-                mul2(v2, v3, r.z, r.w, p2, p3);
-              }
-              m[(2 * i) & 7] = max3(m[(2 * i) & 7], p0, p1);
-              m[(2 * i + 1) & 7] = max3(m[(2 * i + 1) & 7], p2, p3);
+          for (int i = 0; i < 16; ++i) {
+            const float4 r = r4[i];
+            const float v0 = __uint_as_float(v[4 * i]), v1 = __uint_as_float(v[4 * i + 1]);
+            const float v2 = __uint_as_float(v[4 * i + 2]), v3 = __uint_as_float(v[4 * i + 3]);
+            float p0, p1, p2, p3;
+            if (METRIC == kTsgNegL2) {
+              fma2(v0, v1, 2.f, 2.f, r.x, r.y, p0, p1);
+              fma2(v2, v3, 2.f, 2.f, r.z, r.w, p2, p3);
+            } else {
+              mul2(v0, v1, r.x, r.y, p0, p1);
+              mul2(v2, v3, r.z, r.w, p2, p3);
             }
-          };
-          // two register sets: chunk c + 1 loads while chunk c is reduced
-          uint32_t b0[64], b1[64];
-          tmem_ld64_issue(tbase, b0);
-          tmem_ld64_wait(b0);
-          tmem_ld64_issue(tbase + 64, b1);
-          reduce(b0, 0);
-          tmem_ld64_wait_after(b1, m);
-          tmem_ld64_issue(tbase + 128, b0);
-          reduce(b1, 1);
-          tmem_ld64_wait_after(b0, m);
-          tmem_ld64_issue(tbase + 192, b1);
-          reduce(b0, 2);
-          tmem_ld64_wait_after(b1, m);
-          reduce(b1, 3);
-          mx = fmaxf(fmaxf(max3(m[0], m[1], m[2]), max3(m[3], m[4], m[5])), fmaxf(m[6], m[7]));
-        } else {
-          // ragged stage: columns past the frame carry rn = NaN, ignored by fmaxf
-          for (int c = 0; c < 8; ++c) {
-            if (c * 32 >= valid_g) break;
-            float v[32];
-            tmem_ld32(tbase + c * 32, v);
-            const float4* r4 = reinterpret_cast<const float4*>(rg + c * 32);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              float4 r = r4[i];
-              if (METRIC == kTsgNegL2) {
-                mx = fmaxf(mx, fmaf(v[4 * i], 2.f, r.x));
-                mx = fmaxf(mx, fmaf(v[4 * i + 1], 2.f, r.y));
-                mx = fmaxf(mx, fmaf(v[4 * i + 2], 2.f, r.z));
-                mx = fmaxf(mx, fmaf(v[4 * i + 3], 2.f, r.w));
-              } else {
-                mx = fmaxf(mx, v[4 * i] * r.x);
-                mx = fmaxf(mx, v[4 * i + 1] * r.y);
-                mx = fmaxf(mx, v[4 * i + 2] * r.z);
-                mx = fmaxf(mx, v[4 * i + 3] * r.w);
-              }
-            }
+            m[(2 * i) & 7] = max3(m[(2 * i) & 7], p0, p1);
+            m[(2 * i + 1) & 7] = max3(m[(2 * i + 1) & 7], p2, p3);
           }
-        }
+        };
+        uint32_t v[64];
+        tmem_ld64_issue(tbase, v);
+        tmem_ld64_wait(v);
+        reduce(v, 0);
+        tmem_ld64_issue(tbase + 64, v);
+        tmem_ld64_wait_after(v, m);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(b_accempty + 8 * g);
+        reduce(v, 1);
+        const float mx = fmaxf(fmaxf(max3(m[0], m[1], m[2]), max3(m[3], m[4], m[5])), fmaxf(m[6], m[7]));
         int tok0, fend;
         tsg_tile_next(ft, t, tf, tok0, fend);
         const int tok = tok0 + quarter * 32 + lane;
@@ -1441,7 +1417,7 @@ cudaError_t launch_tsg_umma(const Problem& p, const FrameTable& ft, const LayerP
   const int gx = pick_split(groups, n_tiles, sm_count(), n_tiles, 4);
   dim3 grid(gx, nchunk, p.L * p.hkv);
   TimingScope ts("tsg_umma", st);
-  kern<<<grid, kThreads, kTsgSmem, st>>>(local, ft, rn_cur, cur_pad, rho_key, p.hkv, err);
+  kern<<<grid, kTsgThreads, kTsgSmem, st>>>(local, ft, rn_cur, cur_pad, rho_key, p.hkv, err);
   return cudaGetLastError();
 }
 
