@@ -84,12 +84,14 @@ __device__ __forceinline__ void tsg_tile_next(const FrameTable& ft, int t, int& 
 // rn = NaN, which fmaxf ignores.
 //
 // Bound by the tensor pipe and the exposed part of the drain; over many layers
-// by the power cap.  Against one group of four warps per stage (168 registers)
-// the drain is shorter, most of all where a frame fills part of its last
-// chunk: one layer of 20,736 historical rows and 2,304 columns 41.7 -> 39.6
-// us, three chunks of 1,296 125.7 -> 121.3, a 28-layer sequence of the small
-// backbone 152 -> 147, 28 x 50,176 rows and 1,024 columns 837 -> 819 (1,799
-// TFLOP/s) where the power cap leaves the clock alone.
+// by the power cap.  Two groups per stage (one of 168 registers before) shorten
+// the drain: 28 x 50,176 historical rows and 1,024 columns 837 -> 819 us, one
+// layer of 20,736 rows and 2,304 columns 41.7 -> 39.6.  The thread that issues
+// the MMAs is on the critical path of every tile: with the operands' descriptors
+// formed once and the ring stage counted, not divided out, 819 -> 785 us (1,877
+// TFLOP/s).  A last chunk of few columns alternates the stages and gets fewer
+// CTAs (TsgSplit): with both, one layer of 2,304 columns 39.8 -> 35.5 us and one
+// of 1,296 121.5 -> 113.3.
 constexpr int kTsgThreads = 576, kTsgMaxReg = 96;  // TMA, MMA and four groups of four warps
 constexpr int kTsgB = 0;                  // [2][512][128 B]
 constexpr int kTsgAStages = 3;
@@ -99,13 +101,17 @@ constexpr int kTsgBar = kTsgRn + 2048;                     // 12 mbarriers + slo
 constexpr int kTsgUsed = kTsgBar + 128;                    // bytes after 1024-alignment
 constexpr int kTsgSmem = 232448;                           // the per-CTA maximum; the rest is alignment slack
 
+struct TsgSplit {
+  int nchunk, full, last;  // column chunks; CTAs of each but the last, CTAs of the last
+};
+
 // METRIC kTsgCosine: acc_ij * rn_j; kTsgDot: acc_ij; kTsgNegL2: 2 acc_ij -
 // |k_j|^2 (the row's own -|k_i|^2 is added by the selection kernel).  The
 // per-column term sits in rn_s (rn_j, 1, or -|k_j|^2), NaN past the frame.
 template <int METRIC>
 __global__ void __maxnreg__(kTsgMaxReg)
     k_tsg_umma(const __grid_constant__ KMaps maps, const __grid_constant__ FrameTable ft,
-               Strided<const float> rc_all, int cur_pad, Strided<uint32_t> rho_all, int hkv, uint32_t* err) {
+               Strided<const float> rc_all, int cur_pad, Strided<uint32_t> rho_all, int hkv, TsgSplit sp, uint32_t* err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = align1024(smem_raw);
   if ((int)(sm - smem_raw) + kTsgUsed > kTsgSmem) {  // uniform: the layout would not fit
@@ -113,14 +119,20 @@ __global__ void __maxnreg__(kTsgMaxReg)
     return;
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int chunk = blockIdx.y, l = blockIdx.z / hkv, h = blockIdx.z % hkv, n = ft.n_tokens;
+  // CTA b of a (layer, head): `full` CTAs for each chunk but the last, then
+  // `last` CTAs for that one; CTA x of a chunk takes every step-th row tile
+  const int chunk = min((int)blockIdx.x / sp.full, sp.nchunk - 1), t0 = (int)blockIdx.x - chunk * sp.full;
+  const int step = chunk == sp.nchunk - 1 ? sp.last : sp.full;
+  const int l = blockIdx.y / hkv, h = blockIdx.y % hkv, n = ft.n_tokens;
   const CUtensorMap& kmap = maps.m[l];
   const float* rn_cur = rc_all.at(l) + (size_t)h * cur_pad;  // 16-byte aligned rows
   uint32_t* rho_key = rho_all.at(l) + (size_t)h * n;
   const int n_tiles = ft.tsg_tiles;
   const int col0 = chunk * 512;
   const int valid = min(512, ft.cur_len - col0);
-  const int nst = valid > 256 ? 2 : 1;
+  // a chunk of at most 256 columns alternates the two stages between its row
+  // tiles (`alt`): with one, the next product would wait for the whole drain
+  const bool alt = valid <= 256;
   const uint32_t sB = smem_u32(sm + kTsgB), sA = smem_u32(sm + kTsgA);
   float* rn_s = reinterpret_cast<float*>(sm + kTsgRn);
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kTsgBar);
@@ -139,7 +151,7 @@ __global__ void __maxnreg__(kTsgMaxReg)
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(b_accfull + 8 * i, 1);
-      mbar_init(b_accempty + 8 * i, valid - i * 256 > 128 ? 8 : 4);
+      mbar_init(b_accempty + 8 * i, valid - (alt ? 0 : i * 256) > 128 ? 8 : 4);
     }
     mbar_init(b_bfull, 1);
     mbar_init(b_done, 1);
@@ -174,11 +186,10 @@ __global__ void __maxnreg__(kTsgMaxReg)
         for (int rb = 0; rb < 4; ++rb)
           tma_load_3d(sB + kb * 65536 + rb * 16384, &kmap, b_bfull, kb * 64, h,
                       ft.cur_off + col0 + rb * 128);
-      int it = 0, issued[kTsgAStages] = {0, 0, 0}, tf = 0;
-      for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++it) {
-        const int s = it % kTsgAStages;
-        const uint32_t u = (uint32_t)(it / kTsgAStages);
-        if (!mbar_wait(b_aempty + 8 * s, (u & 1u) ^ 1u, err, abort_flag)) break;
+      int s = 0, issued[kTsgAStages] = {0, 0, 0}, tf = 0;
+      uint32_t pass = 0;
+      for (int t = t0; t < n_tiles; t += step, s = s + 1 == kTsgAStages ? 0 : s + 1, pass += s == 0 ? 1u : 0u) {
+        if (!mbar_wait(b_aempty + 8 * s, (pass & 1u) ^ 1u, err, abort_flag)) break;
         int tok0, fend;
         tsg_tile_next(ft, t, tf, tok0, fend);
         mbar_arrive_expect_tx(b_afull + 8 * s, 32768);
@@ -195,29 +206,30 @@ __global__ void __maxnreg__(kTsgMaxReg)
   } else if (warp == 1) {
     if (lane == 0) {
       bool ok = mbar_wait(b_bfull, 0, err, abort_flag);
-      int it = 0;
-      for (int t = blockIdx.x; ok && t < n_tiles; t += gridDim.x, ++it) {
-        const int s = it % kTsgAStages;
-        const uint32_t u = (uint32_t)(it / kTsgAStages);
-        if (!mbar_wait(b_afull + 8 * s, u & 1u, err, abort_flag)) break;
+      const uint64_t da = desc_sw128(sA), db = desc_sw128(sB);
+      const uint32_t id0 = idesc_bf16(128, (min(256, valid) + 15) & ~15);
+      const uint32_t id1 = idesc_bf16(128, (valid - 256 + 15) & ~15);
+      // stage g = the row tile in ring stage s times the columns at `b`
+      auto product = [&](int g, int s, uint64_t b, uint32_t idesc, uint32_t use) {
+        if (!mbar_wait(b_accempty + 8 * g, (use & 1u) ^ 1u, err, abort_flag)) return false;
         tc_fence_after();
-        for (int g = 0; g < nst && ok; ++g) {
-          if (!mbar_wait(b_accempty + 8 * g, ((uint32_t)it & 1u) ^ 1u, err, abort_flag)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const int ncols = (min(256, valid - g * 256) + 15) & ~15;
-          const uint32_t idesc = idesc_bf16(128, ncols);
+        const uint64_t a = da + (uint64_t)(s * (32768 >> 4));
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const uint32_t kb = k >> 2, koff = (k & 3) * 32;
-            uint64_t ad = desc_sw128(sA + s * 32768 + kb * 16384 + koff);
-            uint64_t bd = desc_sw128(sB + kb * 65536 + g * 256 * 128 + koff);
-            umma_bf16(tmem + g * 256, ad, bd, idesc, k > 0 ? 1u : 0u);
-          }
-          umma_commit(b_accfull + 8 * g);
-        }
+        for (int k = 0; k < 8; ++k)
+          umma_bf16(tmem + g * 256, a + ((k >> 2) * 16384 + (k & 3) * 32) / 16, b + ((k >> 2) * 65536 + (k & 3) * 32) / 16,
+                    idesc, k > 0 ? 1u : 0u);
+        umma_commit(b_accfull + 8 * g);
+        return true;
+      };
+      int s = 0;
+      uint32_t pass = 0, it = 0;
+      for (int t = t0; ok && t < n_tiles; t += step, ++it, s = s + 1 == kTsgAStages ? 0 : s + 1, pass += s == 0 ? 1u : 0u) {
+        if (!mbar_wait(b_afull + 8 * s, pass & 1u, err, abort_flag)) break;
+        tc_fence_after();
+        if (alt)
+          ok = product((int)(it & 1u), s, db, id0, it >> 1);
+        else
+          ok = product(0, s, db, id0, it) && product(1, s, db + 256 * 128 / 16, id1, it);
         if (!ok) break;
         umma_commit(b_aempty + 8 * s);
       }
@@ -225,13 +237,14 @@ __global__ void __maxnreg__(kTsgMaxReg)
       mbar_wait_drain(b_done, 0);
     }
   } else {
-    // group g drains half g >> 1 (128 columns) of stage g & 1
+    // group grp drains half grp >> 1 (128 columns) of stage grp & 1
     const int grp = (warp - 2) >> 2, g = grp & 1, half = grp >> 1, quarter = warp & 3;
-    if (valid > g * 256 + half * 128) {
+    const int c0 = (alt ? 0 : g * 256) + half * 128, every = alt ? 2 * step : step;
+    if (valid > c0) {
       const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + g * 256 + half * 128;
-      const float* rg = rn_s + g * 256 + half * 128;
+      const float* rg = rn_s + c0;
       int it = 0, tf = 0;
-      for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++it) {
+      for (int t = alt ? t0 + g * step : t0; t < n_tiles; t += every, ++it) {
         if (!warp_wait(b_accfull + 8 * g, (uint32_t)it & 1u, err, abort_flag)) break;
         tc_fence_after();
         // packed products and 3-input max into eight independent running
@@ -1400,6 +1413,33 @@ int score_nsplit_max(const Problem& p) {
 
 int score_nsplit(const Problem& p) { return score_nsplit_max(p); }
 
+// TSG's CTAs per column chunk.  pick_split's choice, or, where one wave holds
+// every chunk, fewer CTAs for a last chunk whose row tiles cost less (`width`
+// columns) and the SMs they leave for the others: 4 heads of 162 tiles and 5
+// chunks, the last of 256 columns, 8 CTAs per chunk and 6 instead of 7 each.  A
+// tile of up to 256 columns takes a little more than half a full one's time
+// (its drain is not hidden by a second product), one of 272 about 0.85.
+static TsgSplit tsg_split(int units, int nchunk, int width, int tiles, int slots) {
+  constexpr int kFixed = 4;
+  TsgSplit sp{nchunk, 0, 0};
+  sp.full = sp.last = pick_split(units * nchunk, tiles, slots, tiles, kFixed);
+  const double weight = width <= 256 ? 0.56 : width <= 384 ? 0.85 : 1.0;
+  if (nchunk == 1 || weight == 1.0) return sp;
+  auto cost = [&](int s) { return kFixed + (double)((tiles + s - 1) / s); };
+  const long long waves = ((long long)units * nchunk * sp.full + slots - 1) / slots;
+  double best = (double)waves * cost(sp.full);
+  for (int f = 1; f <= tiles && (long long)units * ((long long)(nchunk - 1) * f + 1) <= slots; ++f) {
+    const int l = std::min(slots / units - (nchunk - 1) * f, f);
+    const double c = std::max(cost(f), kFixed + weight * (double)((tiles + l - 1) / l));
+    if (c < best) {
+      best = c;
+      sp.full = f;
+      sp.last = l;
+    }
+  }
+  return sp;
+}
+
 cudaError_t launch_tsg_umma(const Problem& p, const FrameTable& ft, const LayerPtrs& io,
                             Strided<const float> rn_cur, int cur_pad, Strided<uint32_t> rho_key, int metric,
                             uint32_t* err, cudaStream_t st) {
@@ -1413,11 +1453,10 @@ cudaError_t launch_tsg_umma(const Problem& p, const FrameTable& ft, const LayerP
   auto kern = metric == kTsgDot ? k_tsg_umma<kTsgDot> : (metric == kTsgNegL2 ? k_tsg_umma<kTsgNegL2> : k_tsg_umma<kTsgCosine>);
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTsgSmem);
   if (e != cudaSuccess) return e;
-  const int groups = nchunk * p.L * p.hkv;
-  const int gx = pick_split(groups, n_tiles, sm_count(), n_tiles, 4);
-  dim3 grid(gx, nchunk, p.L * p.hkv);
+  const TsgSplit sp = tsg_split(p.L * p.hkv, nchunk, ft.cur_len - (nchunk - 1) * 512, n_tiles, sm_count());
+  dim3 grid((nchunk - 1) * sp.full + sp.last, p.L * p.hkv);
   TimingScope ts("tsg_umma", st);
-  kern<<<grid, kTsgThreads, kTsgSmem, st>>>(local, ft, rn_cur, cur_pad, rho_key, p.hkv, err);
+  kern<<<grid, kTsgThreads, kTsgSmem, st>>>(local, ft, rn_cur, cur_pad, rho_key, p.hkv, sp, err);
   return cudaGetLastError();
 }
 

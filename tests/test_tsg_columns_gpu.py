@@ -1,7 +1,8 @@
 """TSG's column halves (bf16): current frames whose columns end one below, at
 and one above each 64, 128, 256 and 512, so that a chunk's second stage and a
-stage's second half are absent, nearly empty, ragged or full, against the
-fp64 oracle under the parity rules."""
+stage's second half are absent, nearly empty, ragged or full; and pools of
+many row tiles, where a last chunk of few columns gets fewer CTAs than the
+others; against the fp64 oracle under the parity rules."""
 import numpy as np
 import pytest
 import torch
@@ -23,11 +24,12 @@ def st():
     return stlite
 
 
-@pytest.mark.parametrize("cols", [1, 63, 64, 65, 127, 128, 129, 191, 193, 255, 256, 257, 320, 321, 384, 385, 511, 512,
-                                  513, 641, 769, 1025])
-def test_tsg_columns(st, cols):
+@pytest.mark.parametrize("cols, hist", [(c, (11, 13)) for c in (
+    1, 63, 64, 65, 127, 128, 129, 191, 193, 255, 256, 257, 320, 321, 384, 385, 511, 512, 513, 641, 769, 1025)] +
+    [(600, (63, 67)), (800, (77, 81)), (1100, (90, 101))])
+def test_tsg_columns(st, cols, hist):
     w, hq, hkv, text = 1, 2, 2, 3
-    grids = [(11, 13), (1, 129), (1, cols)] if cols <= 256 else [(11, 13), (1, 129), (cols, 1)]
+    grids = [hist, (1, 129), (1, cols) if cols <= 256 else (cols, 1)]
     offs, at = [], 0
     for gh, gw in grids:
         offs.append(at)
