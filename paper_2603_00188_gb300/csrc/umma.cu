@@ -1416,9 +1416,10 @@ int score_nsplit(const Problem& p) { return score_nsplit_max(p); }
 // TSG's CTAs per column chunk.  pick_split's choice, or, where one wave holds
 // every chunk, fewer CTAs for a last chunk whose row tiles cost less (`width`
 // columns) and the SMs they leave for the others: 4 heads of 162 tiles and 5
-// chunks, the last of 256 columns, 8 CTAs per chunk and 6 instead of 7 each.  A
-// tile of up to 256 columns takes a little more than half a full one's time
-// (its drain is not hidden by a second product), one of 272 about 0.85.
+// chunks, the last of 256 columns, 8 CTAs per chunk and 6 instead of 7 each
+// (39.8 -> 35.5 us with the alternating stages).  The weights: a tile of up to
+// 256 columns is half a full one's product and never quite hides its drain; one
+// of up to 384 is more than half of it, and its first stage waits for a drain.
 static TsgSplit tsg_split(int units, int nchunk, int width, int tiles, int slots) {
   constexpr int kFixed = 4;
   TsgSplit sp{nchunk, 0, 0};
