@@ -77,17 +77,6 @@ constexpr int kP2Sum = kP2Xch + kPrGroups * 128 * 4;    // float2 [128 keys]
 constexpr int kP2Smem = kP2Sum + 128 * 8 + 1024;
 constexpr int kP2MaxSplit = 8;                          // CTAs per key tile (one cluster)
 
-// s.x + s.y += x, the rounding error of the sum s.x kept in s.y (Knuth's
-// two-sum).  Plain sums of the groups and CTAs put the bases of 300-8,576
-// positions up to 30 % further from the fp64 result than one CTA's sum of four
-// groups had been; this puts them 8-15 % nearer, at 0.9 us of 441 (fp64
-// additions: the same error, 2.5 us).
-__device__ __forceinline__ void add_exact(float2& s, float x) {
-  const float t = s.x + x, b = t - s.x;
-  s.y += (s.x - (t - b)) + (x - b);
-  s.x = t;
-}
-
 __device__ __forceinline__ uint8_t* pr_align1024(uint8_t* p) {
   uint32_t a = smem_u32(p);
   return p + ((1024u - (a & 1023u)) & 1023u);
@@ -550,7 +539,10 @@ __global__ void __maxnreg__(kPrMaxReg)
     tmem_dealloc(tmem, 512);
   }
   // the cluster's sums in rank order, up to 32 groups' and rounded once (after
-  // a wait gave up, the keys stay unwritten)
+  // a wait gave up, the keys stay unwritten).  Plain sums of the groups and CTAs
+  // put the bases of 300-8,576 positions up to 30 % further from the fp64 result
+  // than one CTA's sum of four groups had been; these put them 8-15 % nearer, at
+  // 0.9 us of 441 (fp64 additions: the same error, 2.5 us).
   if (split > 1) cl.sync();
   if (rank == 0 && threadIdx.x < 128 && j0 + (int)threadIdx.x < a.n) {
     const int j = j0 + threadIdx.x;
@@ -558,8 +550,7 @@ __global__ void __maxnreg__(kPrMaxReg)
     bool whole = !*abort_flag;
     for (int r = 1; r < split; ++r) {
       const float2 other = cl.map_shared_rank(sum_s, r)[threadIdx.x];
-      add_exact(total, other.x);
-      total.y += other.y;
+      add_exact(total, other);
       whole = whole && !*cl.map_shared_rank(slot + 1, r);
     }
     float acc = total.x + total.y;
@@ -571,7 +562,7 @@ __global__ void __maxnreg__(kPrMaxReg)
 
 // ---- fp32 caches: the same two passes on the CUDA cores --------------------
 // Both are products of 64 x 64 tiles (tile.cuh).  1,152 positions of 28 heads:
-// row statistics 175 us, column sums 221; with a CTA per query row, each thread
+// row statistics 176 us, column sums 229; with a CTA per query row, each thread
 // reading keys from global memory, and one product at a time per thread from
 // shared memory they took 2,116 and 2,422.
 constexpr int kPrSimtSmem = 2 * kTileFloats * 4;
@@ -646,9 +637,9 @@ __global__ void __launch_bounds__(kTileThreads, kTilesPerSm) k_prompt_colsum_sim
   const float c = kPrLog2e * rsqrtf((float)kD);
   const int r_start = j0 <= p_first ? 0 : (j0 - p_first) * a.G;  // rows before it see no key of the tile
   tile_load(ks, min(kTileRows, a.n - j0), [&](int r) { return k + ((size_t)(j0 + r) * a.hkv + h) * kD; });
-  float acc[kTA];
+  float2 acc[kTA];
 #pragma unroll
-  for (int i = 0; i < kTA; ++i) acc[i] = 0.f;
+  for (int i = 0; i < kTA; ++i) acc[i] = make_float2(0.f, 0.f);
   for (int rt = r_start + rank * kTileRows; rt < rows; rt += split * kTileRows) {
     const int nr = min(kTileRows, rows - rt);
     tile_load(qs, nr, [&](int r) { return prompt_row(q, a, h, rt + r); });
@@ -668,19 +659,21 @@ __global__ void __launch_bounds__(kTileThreads, kTilesPerSm) k_prompt_colsum_sim
       float sum = 0.f;
 #pragma unroll
       for (int j = 0; j < kTB; ++j) sum += j0 + ty + 8 * i <= pos[j] ? exp2f(fmaf(d[i][j], c, bs[j])) : 0.f;
-      acc[i] += sum;
+      add_exact(acc[i], sum);
     }
     __syncthreads();  // the query tile is rewritten
   }
-  sum_rows(acc, qs);
+  float2* sums = reinterpret_cast<float2*>(qs);
+  sum_rows(acc, sums);
   if (split > 1)
     cl.sync();
   else
     __syncthreads();
   const int j = j0 + threadIdx.x;
   if (rank == 0 && threadIdx.x < kTileRows && j < a.n) {
-    float sum = qs[threadIdx.x];
-    for (int r = 1; r < split; ++r) sum += cl.map_shared_rank(qs, r)[threadIdx.x];
+    float2 total = sums[threadIdx.x];
+    for (int r = 1; r < split; ++r) add_exact(total, cl.map_shared_rank(sums, r)[threadIdx.x]);
+    float sum = total.x + total.y;
     if (a.mode == 1) sum /= (float)min(a.nq, a.n - j);
     a_out[(size_t)h * a.n + j] = sum;
   }

@@ -580,9 +580,9 @@ __global__ void __launch_bounds__(kTileThreads, kTilesPerSm)
   const float* bias = reinterpret_cast<const float*>(part_all.at(l) + (size_t)p.hkv * nsplit * R) + (size_t)h * R;
   const float c = kLog2e * rsqrtf((float)kD);
   tile_load(ks, min(kTileRows, p.n - j0), [&](int r) { return k + ((size_t)(j0 + r) * p.hkv + h) * kD; });
-  float acc[kTA];
+  float2 acc[kTA];
 #pragma unroll
-  for (int i = 0; i < kTA; ++i) acc[i] = 0.f;
+  for (int i = 0; i < kTA; ++i) acc[i] = make_float2(0.f, 0.f);
   for (int rt = rank * kTileRows; rt < R; rt += split * kTileRows) {
     const int nr = min(kTileRows, R - rt);
     tile_load(qs, nr, [&](int r) { return q_row(q, p, h, rt + r); });
@@ -597,20 +597,21 @@ __global__ void __launch_bounds__(kTileThreads, kTilesPerSm)
       float sum = 0.f;
 #pragma unroll
       for (int j = 0; j < kTB; ++j) sum += tx + 16 * j < nr ? exp2f(fmaf(d[i][j], c, bs[j])) : 0.f;
-      acc[i] += sum;
+      add_exact(acc[i], sum);
     }
     __syncthreads();  // the query tile is rewritten
   }
-  sum_rows(acc, qs);
+  float2* sums = reinterpret_cast<float2*>(qs);
+  sum_rows(acc, sums);
   if (split > 1)
     cl.sync();
   else
     __syncthreads();
   const int j = j0 + threadIdx.x;
   if (rank == 0 && threadIdx.x < kTileRows && j < p.n) {
-    float sum = qs[threadIdx.x];
-    for (int r = 1; r < split; ++r) sum += cl.map_shared_rank(qs, r)[threadIdx.x];
-    a_all.at(l)[(size_t)h * p.n + j] = sum;
+    float2 total = sums[threadIdx.x];
+    for (int r = 1; r < split; ++r) add_exact(total, cl.map_shared_rank(sums, r)[threadIdx.x]);
+    a_all.at(l)[(size_t)h * p.n + j] = total.x + total.y;
   }
   if (split > 1) cl.sync();  // no CTA leaves while rank 0 may still read its sums
 }

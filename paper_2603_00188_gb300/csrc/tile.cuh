@@ -20,7 +20,7 @@ namespace stl {
 // One layer of 5 frames of 36 x 64 (11,840 keys, 4 heads of 224 query rows),
 // against one dot product per thread with both operands read from shared
 // memory for every multiply-add: TSG 2,036 -> 483 us (45 TFLOP/s), row
-// statistics 389 -> 94, column sums 466 -> 89; 1,152 keys: 201 -> 15, 90 -> 18
+// statistics 389 -> 94, column sums 466 -> 92; 1,152 keys: 201 -> 15, 90 -> 18
 // and 195 -> 29.
 constexpr int kTileRows = 64;
 constexpr int kTileThreads = 128;
@@ -91,6 +91,18 @@ __device__ __forceinline__ void tile_dots(const float* a, const float* b, float 
     }
 }
 
+// s.x + s.y += x, the rounding error of the sum s.x kept in s.y (Knuth's
+// two-sum).
+__device__ __forceinline__ void add_exact(float2& s, float x) {
+  const float t = s.x + x, b = t - s.x;
+  s.y += (s.x - (t - b)) + (x - b);
+  s.x = t;
+}
+__device__ __forceinline__ void add_exact(float2& s, float2 x) {
+  add_exact(s, x.x);
+  s.y += x.y;
+}
+
 // (m, l) <- the states (m, l) and (m2, l2) together; l = 0: an empty state.
 __device__ __forceinline__ void merge_state(float& m, float& l, float m2, float l2) {
   if (l2 == 0.f) return;
@@ -104,12 +116,19 @@ __device__ __forceinline__ void merge_state(float& m, float& l, float m2, float 
   m = mn;
 }
 
-// (m, l) <- (m, l) and the scores x[0..kTB-1] (log2 units; -inf: none).
+// (m, l) <- (m, l) and the scores x[0..kTB-1] (log2 units; -inf: none).  m is
+// the maximum rounded up to a whole number, so that every later change of m,
+// here or when states merge, scales l by a power of two, without rounding.
+// With the maximum itself, and plain sums of the probabilities, the scores of
+// few rows were up to 26 % further from the fp64 result than one thread's sums
+// over a row had been; with this and add_exact they are 1.4-8 times nearer (one
+// row per head: the same), at 3 % of the column sums' time.
 __device__ __forceinline__ void fold_scores(float& m, float& l, const float (&x)[kTB]) {
   float mn = m;
 #pragma unroll
   for (int j = 0; j < kTB; ++j) mn = fmaxf(mn, x[j]);
   if (mn == -CUDART_INF_F) return;  // no score yet
+  mn = ceilf(mn);
   float sum = 0.f;
 #pragma unroll
   for (int j = 0; j < kTB; ++j) sum += x[j] == mn ? 1.f : exp2f(x[j] - mn);
@@ -144,14 +163,17 @@ __device__ __forceinline__ void merge_rows(float (&m)[kTA], float (&l)[kTA], flo
     }
 }
 
-// Sums per row, merged the same way, into sums[0..63] (shared memory, as xch
-// above); a block barrier away from being read.
-__device__ __forceinline__ void sum_rows(float (&acc)[kTA], float* sums) {
+// Sums per row with their rounding errors (add_exact), merged the same way, into
+// sums[0..63] (shared memory, as xch above); a block barrier away from being read.
+__device__ __forceinline__ void sum_rows(float2 (&acc)[kTA], float2* sums) {
   const int ty = tile_ty(), tx = tile_tx();
 #pragma unroll
   for (int i = 0; i < kTA; ++i)
 #pragma unroll
-    for (int o = 1; o < 8; o <<= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+    for (int o = 1; o < 8; o <<= 1) {
+      const float x = __shfl_xor_sync(0xffffffffu, acc[i].x, o), y = __shfl_xor_sync(0xffffffffu, acc[i].y, o);
+      add_exact(acc[i], make_float2(x, y));
+    }
   tile_ready();
   if (tx == 8)
 #pragma unroll
@@ -159,7 +181,10 @@ __device__ __forceinline__ void sum_rows(float (&acc)[kTA], float* sums) {
   __syncthreads();
   if (tx == 0)
 #pragma unroll
-    for (int i = 0; i < kTA; ++i) sums[ty + 8 * i] += acc[i];
+    for (int i = 0; i < kTA; ++i) {
+      add_exact(acc[i], sums[ty + 8 * i]);
+      sums[ty + 8 * i] = acc[i];
+    }
 }
 
 }  // namespace stl
