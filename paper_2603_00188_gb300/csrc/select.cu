@@ -444,7 +444,8 @@ struct ScoreIn4 {
 
 __global__ void __launch_bounds__(kSelThreads, 4) k_select(Problem p, const __grid_constant__ FrameTable ft,
                                                         SelectArgs a) {
-  extern __shared__ uint32_t keys[];
+  extern __shared__ uint4 key_smem[];  // its type aligns it: cluster_select reads four keys at a time
+  uint32_t* const keys = reinterpret_cast<uint32_t*>(key_smem);
   __shared__ SelShared sh;
   cg::cluster_group cl = cg::this_cluster();
   const int ncta = (int)cl.num_blocks(), c = (int)cl.block_rank();
