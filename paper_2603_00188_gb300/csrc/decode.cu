@@ -23,19 +23,12 @@ constexpr int kDecThreads = 256;  // 8 warps
 constexpr float kDecLog2e = 1.4426950408889634f;
 constexpr int kDecWarps = kDecThreads / 32;
 
-// Eight consecutive elements of a row as floats (16-byte aligned).
-__device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&f)[8]) {
-  const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
-  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    f[2 * i] = __uint_as_float(w[i] << 16);
-    f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-  }
-}
+// Eight consecutive elements of a row (16-byte aligned).  A plain load, as all
+// of this file's: the kernels are launched ahead of their predecessors
+// (launch_after), which may have written q, k or v.
 __device__ __forceinline__ void load8(const float* p, float (&f)[8]) {
-  const float4 a = __ldg(reinterpret_cast<const float4*>(p));
-  const float4 b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+  const float4 a = reinterpret_cast<const float4*>(p)[0];
+  const float4 b = reinterpret_cast<const float4*>(p)[1];
   f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w;
   f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
 }
@@ -51,7 +44,7 @@ __device__ __forceinline__ float weight(float a, float m) { return a == -CUDART_
 
 // Dynamic shared memory: qs[G][128] (query rows times log2(e)/sqrt(d)), then
 // per warp o[G][128] and (m, l)[G].
-template <typename T, int GM>
+template <int GM>
 __global__ void __launch_bounds__(kDecThreads, 2) k_decode_split(const __grid_constant__ DecBatch b, int w, int n,
                                                               int hq, int hkv, int per, float* part_o_all,
                                                               float2* part_ml_all) {
@@ -59,9 +52,9 @@ __global__ void __launch_bounds__(kDecThreads, 2) k_decode_split(const __grid_co
   pdl_trigger();
   pdl_wait();
   const int split = blockIdx.x, h = blockIdx.y, r = blockIdx.z % w, layer = blockIdx.z / w, nsplit = gridDim.x;
-  const T* __restrict__ q = static_cast<const T*>(b.q[layer]);
-  const T* __restrict__ k = static_cast<const T*>(b.k[layer]);
-  const T* __restrict__ v = static_cast<const T*>(b.v[layer]);
+  const float* q = static_cast<const float*>(b.q[layer]);
+  const float* k = static_cast<const float*>(b.k[layer]);
+  const float* v = static_cast<const float*>(b.v[layer]);
   float* part_o = part_o_all + (size_t)layer * nsplit * w * hq * kD;
   float2* part_ml = part_ml_all + (size_t)layer * nsplit * w * hq;
   const int G = hq / hkv;
@@ -72,7 +65,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) k_decode_split(const __grid_co
   const float scale = kDecLog2e * rsqrtf((float)kD);
   for (int e = threadIdx.x; e < G * kD; e += kDecThreads) {
     const int g = e / kD, c = e % kD;
-    qs[e] = Elem<T>::load1(q + ((size_t)r * hq + h * G + g) * kD + c) * scale;
+    qs[e] = q[((size_t)r * hq + h * G + g) * kD + c] * scale;
   }
   __syncthreads();
 
@@ -92,7 +85,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) k_decode_split(const __grid_co
 #pragma unroll
     for (int g = 0; g < GM; ++g) s[g] = 0.f;
     if (t < j1) {
-      const T* kr = k + (size_t)t * rs + (size_t)h * kD;
+      const float* kr = k + (size_t)t * rs + (size_t)h * kD;
 #pragma unroll 8
       for (int c = 0; c < kD; c += 8) {
         float kf[8];
@@ -130,7 +123,8 @@ __global__ void __launch_bounds__(kDecThreads, 2) k_decode_split(const __grid_co
       float4 vv[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        if (t0 + u < cnt) vv[u] = Elem<T>::load4(v + (size_t)(base + t0 + u) * rs + (size_t)h * kD + 4 * lane);
+        if (t0 + u < cnt)
+          vv[u] = *reinterpret_cast<const float4*>(v + (size_t)(base + t0 + u) * rs + (size_t)h * kD + 4 * lane);
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         if (t0 + u < cnt) {
@@ -257,7 +251,7 @@ __global__ void __launch_bounds__(kDecMmaThreads, 1)
   const int split = blockIdx.x, h = blockIdx.y, r = blockIdx.z % w, layer = blockIdx.z / w;
   const CUtensorMap& kmap = maps.k[layer];
   const CUtensorMap& vmap = maps.v[layer];
-  const __nv_bfloat16* __restrict__ q = static_cast<const __nv_bfloat16*>(b.q[layer]);
+  const __nv_bfloat16* q = static_cast<const __nv_bfloat16*>(b.q[layer]);
   float* part_o = part_o_all + (size_t)layer * gridDim.x * w * hq * kD;
   float2* part_ml = part_ml_all + (size_t)layer * gridDim.x * w * hq;
   const int G = hq / hkv;
@@ -306,8 +300,8 @@ __global__ void __launch_bounds__(kDecMmaThreads, 1)
     const uint32_t* qr = reinterpret_cast<const uint32_t*>(q + ((size_t)r * hq + h * G + (head < G ? head : 0)) * kD);
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks) {
-      qb[ks][nt][0] = head < G ? __ldg(qr + 8 * ks + t4) : 0u;
-      qb[ks][nt][1] = head < G ? __ldg(qr + 8 * ks + 4 + t4) : 0u;
+      qb[ks][nt][0] = head < G ? qr[8 * ks + t4] : 0u;
+      qb[ks][nt][1] = head < G ? qr[8 * ks + 4 + t4] : 0u;
     }
   }
   const float scale = kDecLog2e * rsqrtf((float)kD);
@@ -575,9 +569,9 @@ cudaError_t launch_decode(DType dt, const DecBatch& b, int layers, int n, int hq
     const size_t smem = (size_t)G * kD * 4 + (size_t)kDecWarps * G * kD * 4 + (size_t)kDecWarps * G * 8;
     auto run = [&](auto gm) {
       constexpr int GM = decltype(gm)::value;
-      e = cudaFuncSetAttribute(k_decode_split<float, GM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      e = cudaFuncSetAttribute(k_decode_split<GM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return;
-      e = launch_after(k_decode_split<float, GM>, grid, kDecThreads, smem, st, b, w, n, hq, hkv, per, part_o, part_ml);
+      e = launch_after(k_decode_split<GM>, grid, kDecThreads, smem, st, b, w, n, hq, hkv, per, part_o, part_ml);
     };
     TimingScope ts("decode_split", st);
     if (G <= 4)

@@ -792,7 +792,9 @@ cudaError_t launch_select(const Problem& p, const FrameTable& ft, const SelectAr
 // ------------------------------------------------------------------ gather
 // k_out[l][r][h][:] = k_l[idx[l][h][r]][h][:] (and v): 16-byte chunks, four
 // rows per thread in flight, consecutive threads cover consecutive chunks of
-// one output row (coalesced stores, whole 16-byte source vectors).
+// one output row (coalesced stores, whole 16-byte source vectors).  Plain
+// loads: idx, and whatever else the kernel before it wrote, was written while
+// this one was already resident (and v may be page-locked host memory).
 // grid.y = layer.
 template <int CPR>
 __global__ void __launch_bounds__(256) k_gather(const __grid_constant__ LayerPtrs io, int n, int hkv) {
@@ -819,11 +821,11 @@ __global__ void __launch_bounds__(256) k_gather(const __grid_constant__ LayerPtr
         const int c = (int)(e % CPR);
         const long long rh = e / CPR;
         const int h = (int)(rh % hkv), r = (int)(rh / hkv);
-        const int src = __ldg(idx + (size_t)h * budget + r);
+        const int src = idx[(size_t)h * budget + r];
         if (src >= 0 && src < n) {
           const size_t s = ((size_t)src * hkv + h) * CPR + c;
-          kv[u] = __ldg(k + s);
-          vv[u] = v[s];  // plain load: v may be page-locked host memory
+          kv[u] = k[s];
+          vv[u] = v[s];
           ok[u] = true;
         }
       }

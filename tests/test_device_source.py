@@ -28,3 +28,65 @@ def test_dynamic_shared_memory_aligned_by_type(name):
     for kind, var, following in found:
         own = kind == "uint8_t" and re.search(r"align1024\(%s\)|%s \+ \(\(1024u" % (var, var), following)
         assert own or kind in ("float4", "uint4"), (name, kind, var)
+
+
+def _body(code, at):
+    """The text from the first brace at or after `at` to its match."""
+    i = j = code.index("{", at)
+    depth = 0
+    while True:
+        depth += {"{": 1, "}": -1}.get(code[j], 0)
+        j += 1
+        if depth == 0:
+            return code[i:j]
+
+
+def _functions():
+    """Bodies of every device function, by name (overloads together)."""
+    out = {}
+    for code in FILES.values():
+        for m in re.finditer(r"__(?:global|device)__[^;{}]*?\b(\w+)\((?=[^;{}]*\{)", code):
+            names = re.findall(r"(\w+)\(", code[m.start():code.index("{", m.start())])
+            for name in names:
+                out[name] = out.get(name, "") + _body(code, m.start())
+    return out
+
+
+def _launched_after():
+    """Kernels launched with launch_after, also through a local variable."""
+    out = set()
+    for code in FILES.values():
+        for m in re.finditer(r"launch_after\(([^,]*?),", code):
+            arg = m.group(1)
+            if "(*kern)" in arg:
+                continue
+            names = re.findall(r"\bk_\w+", arg)
+            for var in [] if names else re.findall(r"\b[a-z]\w*", arg):
+                for definition in re.findall(r"\b%s = ([^;]*);" % var, code):
+                    names += re.findall(r"\bk_\w+", definition)
+            assert names, arg
+            out |= set(names)
+    return sorted(out)
+
+
+@pytest.mark.parametrize("kernel", _launched_after())
+def test_kernels_launched_ahead_use_plain_loads(kernel):
+    """A kernel launched ahead of its predecessor is resident while that one
+    still writes.  Loads through the read-only path are defined only for data
+    that nobody writes during a kernel's lifetime, so it must not have any,
+    also not in the functions it calls; and it waits for its predecessor."""
+    functions = _functions()
+    todo, seen = [kernel], set()
+    while todo:
+        name = todo.pop()
+        seen.add(name)
+        for bad in ("__ldg", "__restrict__", "ld.global.nc", "__ldcs"):
+            assert bad not in functions[name], (kernel, name, bad)
+        todo += [f for f in set(re.findall(r"\b(\w+)(?:<[^;()]*>)?\(", functions[name])) if f in functions and f not in seen]
+    assert "pdl_wait()" in functions[kernel]
+    assert len(seen) > 1  # the calls were followed
+
+
+def test_kernels_launched_ahead_are_found():
+    assert {"k_gather", "k_colsum_umma", "k_row_bias", "k_decode_split", "k_decode_mma",
+            "k_decode_combine"} <= set(_launched_after())
