@@ -155,9 +155,12 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
 // Programmatic dependent launch (launch_after): a kernel launched that way may
 // start while its predecessor in the stream still runs; pdl_wait returns once
 // the predecessor has completed and its writes are visible, and pdl_trigger
-// lets a successor start.  Every thread of such a kernel waits before it
-// touches global memory, so a kernel completes after its predecessor does and
-// the order of the stream holds for whatever follows.
+// lets a successor start.  Every thread of such a kernel waits, so it completes
+// after its predecessor does and the order of the stream holds for whatever
+// follows.  Before the wait it touches no global memory, with one exception:
+// k_colsum_umma, which reads q and k (see launch_score_umma).  And since it is
+// resident while its predecessor still writes, it reads with plain or
+// asynchronous loads only, never through the read-only path.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -101,8 +101,9 @@ class TimingScope {
 };
 
 // Launches `kern` so that it may start once every CTA of its predecessor in
-// the stream has called pdl_trigger (see pdl_wait, which kern calls before it
-// touches anything the predecessor writes, reads or was ordered after).
+// the stream has called pdl_trigger.  kern calls pdl_wait before it touches
+// global memory; what it reads before that must have been written before an
+// ordinary launch earlier in the same call (see pdl_wait).
 template <typename... P, typename... A>
 cudaError_t launch_after(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};

@@ -759,7 +759,9 @@ __global__ void __maxnreg__(kScoreMaxReg)
     tmem_relinquish();
   }
   load_q_sw128(sm, NQ, q, p, h);
-  // what follows needs the row statistics; the copies above do not
+  // what follows needs the row statistics; the copies above do not, and what
+  // they read was complete before the row statistics started (an ordinary
+  // launch, see launch_score_umma)
   pdl_wait();
   // pass 1's row statistics, the splits merged: bias_r = -m_r - log2(G l_r),
   // so that 2^(x c + bias_r) is the softmax probability divided by G (padded
@@ -1485,6 +1487,9 @@ cudaError_t launch_score_umma(const Problem& p, const LayerPtrs& io, Strided<flo
     const int cph0 = pick_split(p.L * p.hkv * L1.NMH, nsplit, sm_count(), score_tiles(p), 3);
     const int cps = (nsplit + cph0 - 1) / cph0;
     const int cph = (nsplit + cps - 1) / cps;
+    // An ordinary launch, and it has to stay one: it starts when all earlier
+    // work of the stream is done, whoever wrote q and k among it.  The column
+    // sums below start after it has, and read q and k before they wait.
     rs_kernel<<<dim3(cph * L1.NMH, p.L * p.hkv), kScoreThreads, L1.total, st>>>(m1, io, p, nsplit, cps, rowpart,
                                                                                err);
   }

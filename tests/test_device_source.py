@@ -90,3 +90,15 @@ def test_kernels_launched_ahead_use_plain_loads(kernel):
 def test_kernels_launched_ahead_are_found():
     assert {"k_gather", "k_colsum_umma", "k_row_bias", "k_decode_split", "k_decode_mma",
             "k_decode_combine"} <= set(_launched_after())
+
+
+def test_order_behind_loads_before_the_wait():
+    """The column sums read q and k before they wait for the row statistics,
+    the only kernel to do so: those are launched in the ordinary way."""
+    early = []
+    for kernel in _launched_after():
+        before = _functions()[kernel].split("pdl_wait()")[0]
+        if re.search(r"tma_load|cp_async|bulk_g2s|load_q", before):
+            early.append(kernel)
+    assert early == ["k_colsum_umma"]
+    assert "k_rowstats_umma" not in _launched_after()
