@@ -14,8 +14,8 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
-#include <atomic>
 
+#include "fit_cache.h"
 #include "kernels.cuh"
 
 namespace cg = cooperative_groups;
@@ -712,17 +712,19 @@ static void select_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, co
   cfg->numAttrs = 1;
 }
 
-// Clusters of c CTAs, `occ` of them to an SM, that are resident at once on
-// device dev: what the occupancy query says, which depends on nothing else
-// here, asked once per (device, c, occ) -- a query takes the host 5 us, and a
-// launch compares up to nine cluster sizes.
-static cudaError_t clusters_fit(int dev, int c, int occ, const cudaLaunchConfig_t& cfg, int* fit) {
-  constexpr int kDevices = 64;
-  static std::atomic<int> known[kDevices][2 * kSelMaxCluster + 1][2048 / kSelThreads + 1];  // fit + 1; 0: not asked
-  std::atomic<int>* slot = dev < kDevices ? &known[dev][c][occ] : nullptr;
-  if (slot && (*fit = slot->load(std::memory_order_relaxed) - 1) >= 0) return cudaSuccess;
-  const cudaError_t e = cudaOccupancyMaxActiveClusters(fit, k_select, &cfg);
-  if (e == cudaSuccess && slot) slot->store(*fit + 1, std::memory_order_relaxed);
+// Clusters of cfg's size and shared memory that are resident at once on device
+// dev in the current context (its id; 0: not known): what the occupancy query says of the largest
+// shared memory that `occ` CTAs of an SM can have (fit_cache.h), or of cfg
+// itself where that says none.
+static cudaError_t clusters_fit(int dev, unsigned long long ctx, int c, int occ, int largest,
+                                const cudaLaunchConfig_t& cfg, int* fit) {
+  static FitCache<64, 2 * kSelMaxCluster, 2048 / kSelThreads> known;
+  if ((*fit = known.get(dev, c, occ, ctx)) >= 0) return cudaSuccess;
+  cudaLaunchConfig_t ask = cfg;
+  ask.dynamicSmemBytes = (size_t)largest;
+  cudaError_t e = cudaOccupancyMaxActiveClusters(fit, k_select, &ask);
+  if (e == cudaSuccess) known.put(dev, c, occ, ctx, *fit);
+  if (e != cudaSuccess || *fit < 1) e = cudaOccupancyMaxActiveClusters(fit, k_select, &cfg);
   return e;
 }
 
@@ -743,6 +745,8 @@ cudaError_t launch_select(const Problem& p, const FrameTable& ft, const SelectAr
   if ((e = cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&cta_smem, cudaDevAttrReservedSharedMemoryPerBlock, dev)) != cudaSuccess) return e;
   cta_smem += (int)sizeof(SelShared);
+  unsigned long long ctx = 0;
+  if (current_ctx_id(&ctx) != cudaSuccess) ctx = 0;
   // Cluster size: the CTAs of a cluster split one (layer, head)'s tokens.
   // Measured (one wave of clusters, GB300): 13 us for a lone CTA and about
   // 16.5 + 0.55 per CTA for a cluster's barriers and exchanges, plus 1.5 ns per
@@ -761,10 +765,11 @@ cudaError_t launch_select(const Problem& p, const FrameTable& ft, const SelectAr
     const int ch = select_chunk(p.n, c);
     if (ch > kSelMaxChunk) continue;
     select_config(&cfg, attr, p, c, st);
-    const int occ = std::min(2048 / kSelThreads, sm_smem / ((cta_smem + 4 * ch + 127) & ~127));
+    const int occ = ctas_per_sm(sm_smem, cta_smem, 4 * ch, 2048 / kSelThreads);
     if (occ < 1) continue;
     int fit = 0;
-    if ((e = clusters_fit(dev, c, occ, cfg, &fit)) != cudaSuccess) {
+    const int largest = largest_dynamic(sm_smem, cta_smem, occ, 4 * kSelMaxChunk);
+    if ((e = clusters_fit(dev, ctx, c, occ, largest, cfg, &fit)) != cudaSuccess) {
       if (c <= kSelMaxCluster) return e;
       break;
     }
