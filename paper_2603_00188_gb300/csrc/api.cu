@@ -123,8 +123,6 @@ WsPlan plan_workspace(const Problem& p, const FrameTable& ft) {
   WsPlan w;
   const size_t hn = (size_t)p.hkv * p.n;
   w.nsplit = score_nsplit_max(p);
-  w.nchunk = use_tensor_cores(p) && ft.n_frames >= 2 ? (ft.cur_len + 255) / 256 : 1;
-  if (w.nchunk < 1) w.nchunk = 1;
   size_t o = 0;
   auto take = [&](size_t bytes) {
     size_t at = o;
@@ -139,11 +137,11 @@ WsPlan plan_workspace(const Problem& p, const FrameTable& ft) {
   w.a_base = take(hn * 4);
   w.phi = take(hn * 4);
   w.rho = take(hn * 4);
-  w.rho_key = take((size_t)w.nchunk * hn * 4);
+  w.rho_key = take(hn * 4);
   w.tau = take((size_t)p.hkv * 4);
   w.gate = take(hn);
   w.score = take(hn * 4);
-  w.dots = take(4 * hn * 4);
+  w.dots = take(use_tensor_cores(p) ? 4 * hn * 4 : 0);
   w.total = o;
   return w;
 }

@@ -71,14 +71,13 @@ struct WsPlan {
   size_t a_base;     // float [Hkv][N]
   size_t phi;        // float [Hkv][N]
   size_t rho;        // float [Hkv][N]
-  size_t rho_key;    // uint32 [Hkv][N] TSG row maxima as float_key images (room for nchunk such arrays)
+  size_t rho_key;    // uint32 [Hkv][N] TSG row maxima as float_key images
   size_t tau;        // float [Hkv]
   size_t gate;       // uint8 [Hkv][N]
   size_t score;      // float [Hkv][N]
-  size_t dots;       // float [4][Hkv][N]: E, S, SE, SW neighbour dots (tensor-core CSS)
+  size_t dots;       // float [4][Hkv][N]: E, S, SE, SW neighbour dots (bf16: the tensor-core CSS)
   size_t total;      // bytes of one layer's region
   int nsplit;        // largest key-split count of the row-statistics pass
-  int nchunk;        // 256-column chunks of the current frame (bf16)
   int cur_pad;       // current-frame length rounded up to 4
 };
 WsPlan plan_workspace(const Problem& p, const FrameTable& ft);

@@ -95,6 +95,21 @@ def test_workspace_size_and_validation(st):
         assert e.value.status == code
 
 
+@pytest.mark.parametrize("n,hkv", [(4096, 4), (53600, 4), (11841, 2)])
+def test_workspace_holds_what_a_layer_uses(st, n, hkv):
+    """Per token and KV head: the inverse norm, A, Phi, rho, TSG's maximum and
+    S in fp32 and a gate byte, and the four neighbour dots of the tensor-core
+    CSS; per column of the current frame another inverse norm; a little for
+    the row statistics and the alignment of each array."""
+    cur = 2304
+    for dt, words in ((st.STLITE_BF16, 10), (st.STLITE_F32, 6)):
+        sh = st.Shape(n, hkv, hkv, 128, 1, dt)
+        one = st.stlite_workspace_size(sh, st.FrameSpec([0, 32], [4, 1], [4, 1]), st.make_params(0.2))
+        wide = st.stlite_workspace_size(sh, st.FrameSpec([0, 32], [4, cur // 64], [4, 64]), st.make_params(0.2))
+        assert (4 * words + 1) * n * hkv <= one <= (4 * words + 1) * n * hkv + (64 << 10)
+        assert 0 <= wide - one <= 4 * hkv * cur + 256
+
+
 def test_entry_points_reject_before_launch(st, good):
     """Malformed pointers and sizes are refused on the host (no GPU needed)."""
     lib = st._lib
