@@ -441,22 +441,30 @@ __global__ void __launch_bounds__(kDecMmaThreads, 1)
   }
 }
 
-// out[r][g][c] = merge over the splits.  grid (hq, w * layers), four slices of
+// out[r][g][c] = merge over the splits.  grid (hq, w * layers), SLICES slices of
 // 128 threads, one dimension each: the splits' weights exp2(m_s - M) and the
 // normaliser are formed in shared memory by one split (or two) per thread
-// while slice k's first eight partials (splits k, k + 4, ...) are on their way.
-// A merge is two or three memory latencies, nothing else: with one slice that
-// loaded the partials after the weights, eight at a time, it took twice as
-// long.
+// while the first partials are on their way.  The partials are summed in four
+// interleaved series (splits k, k + 4, ...) whatever SLICES is, so that it
+// changes no bit.  A merge is two or three memory latencies, nothing else: with
+// one slice that loaded the partials after the weights, eight at a time, it
+// took twice as long.  Four slices have 32 partials in flight; up to eight
+// splits one slice has them all, in a quarter of the threads: 10 us instead of
+// 22 for 256 rows of 16 heads over 60 keys (one split).
 constexpr int kDecMaxSplits = 1024;
-constexpr int kCmbSlices = 4, kCmbThreads = kCmbSlices * kD, kCmbWarps = kCmbThreads / 32;
-static_assert(kDecMaxSplits <= 2 * kCmbThreads, "two splits per thread");
-__global__ void __launch_bounds__(kCmbThreads) k_decode_combine(const __grid_constant__ DecBatch b,
-                                                                const float* part_o_all, const float2* part_ml_all,
-                                                                int nsplit, int hq, int w) {
-  __shared__ float wts[kDecMaxSplits];
-  __shared__ float red[2][kCmbWarps];
-  __shared__ float acc[kCmbSlices - 1][kD];
+constexpr int kCmbSeries = 4, kCmbOneSlice = 8;
+template <int SLICES>
+__global__ void __launch_bounds__(SLICES* kD) k_decode_combine(const __grid_constant__ DecBatch b,
+                                                               const float* part_o_all, const float2* part_ml_all,
+                                                               int nsplit, int hq, int w) {
+  constexpr int kThreads = SLICES * kD, kWarps = kThreads / 32;
+  constexpr int kOwn = kCmbSeries / SLICES;             // series of a slice: k, k + SLICES, ...
+  constexpr int kMost = SLICES == 1 ? kCmbOneSlice : kDecMaxSplits;  // splits
+  constexpr int kAtOnce = SLICES == 1 ? kMost / kCmbSeries : 8;      // partials of a series in flight
+  static_assert(kMost <= 2 * kThreads, "two splits per thread");
+  __shared__ float wts[kMost];
+  __shared__ float red[2][kWarps];
+  __shared__ float acc[kCmbSeries - 1][kD];
   const int g = blockIdx.x, r = blockIdx.y % w, layer = blockIdx.y / w;
   const int t = threadIdx.x, c = t & (kD - 1), k = t / kD, lane = t & 31, wp = t >> 5;
   const size_t rows = (size_t)w * hq;  // partial rows of one split
@@ -464,38 +472,58 @@ __global__ void __launch_bounds__(kCmbThreads) k_decode_combine(const __grid_con
   const float2* part_ml = part_ml_all + (size_t)layer * nsplit * rows + (size_t)r * hq + g;
   pdl_trigger();
   pdl_wait();
-  float x[8];
+  float x[kOwn][kAtOnce];
+  auto load = [&](int s0) {
 #pragma unroll
-  for (int u = 0; u < 8; ++u) x[u] = k + kCmbSlices * u < nsplit ? part_o[(size_t)(k + kCmbSlices * u) * rows * kD] : 0.f;
+    for (int i = 0; i < kOwn; ++i)
+#pragma unroll
+      for (int u = 0; u < kAtOnce; ++u) {
+        const int s = s0 + k + SLICES * i + kCmbSeries * u;
+        x[i][u] = s < nsplit ? part_o[(size_t)s * rows * kD] : 0.f;
+      }
+  };
+  load(0);
   const float2 none = make_float2(-CUDART_INF_F, 0.f);
   const float2 ml0 = t < nsplit ? part_ml[(size_t)t * rows] : none;
-  const float2 ml1 = t + kCmbThreads < nsplit ? part_ml[(size_t)(t + kCmbThreads) * rows] : none;
+  const float2 ml1 = t + kThreads < nsplit ? part_ml[(size_t)(t + kThreads) * rows] : none;
   const float mx = warp_max(fmaxf(ml0.x, ml1.x));
   if (lane == 0) red[0][wp] = mx;
   __syncthreads();
-  const float M = warp_max(red[0][lane % kCmbWarps]);
+  const float M = warp_max(red[0][lane % kWarps]);
   const float a0 = weight(ml0.x, M), a1 = weight(ml1.x, M);
   if (t < nsplit) wts[t] = a0;
-  if (t + kCmbThreads < nsplit) wts[t + kCmbThreads] = a1;
+  if (t + kThreads < nsplit) wts[t + kThreads] = a1;
   const float ls = warp_sum(fmaf(ml0.y, a0, ml1.y * a1));
   if (lane == 0) red[1][wp] = ls;
   __syncthreads();
-  const float L = warp_sum(lane < kCmbWarps ? red[1][lane] : 0.f);
-  float O = 0.f;
+  const float L = warp_sum(lane < kWarps ? red[1][lane] : 0.f);
+  float O[kOwn];
 #pragma unroll
-  for (int u = 0; u < 8; ++u)
-    if (k + kCmbSlices * u < nsplit) O = fmaf(x[u], wts[k + kCmbSlices * u], O);
-  for (int s0 = k + 8 * kCmbSlices; s0 < nsplit; s0 += 8 * kCmbSlices) {
+  for (int i = 0; i < kOwn; ++i) O[i] = 0.f;
+  for (int s0 = 0; s0 < nsplit; s0 += kCmbSeries * kAtOnce) {
+    if (s0 > 0) load(s0);
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-      x[u] = s0 + kCmbSlices * u < nsplit ? part_o[(size_t)(s0 + kCmbSlices * u) * rows * kD] : 0.f;
+    for (int i = 0; i < kOwn; ++i)
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (s0 + kCmbSlices * u < nsplit) O = fmaf(x[u], wts[s0 + kCmbSlices * u], O);
+      for (int u = 0; u < kAtOnce; ++u) {
+        const int s = s0 + k + SLICES * i + kCmbSeries * u;
+        if (s < nsplit) O[i] = fmaf(x[i][u], wts[s], O[i]);
+      }
   }
-  if (k > 0) acc[k - 1][c] = O;
-  __syncthreads();
-  if (k == 0) b.out[layer][((size_t)r * hq + g) * kD + c] = ((O + acc[0][c]) + (acc[1][c] + acc[2][c])) / L;
+  float o1, o2, o3;  // the other series of the thread's dimension
+  if constexpr (SLICES == 1) {
+    o1 = O[1];
+    o2 = O[2];
+    o3 = O[3];
+  } else {
+    if (k > 0) acc[k - 1][c] = O[0];
+    __syncthreads();
+    if (k > 0) return;
+    o1 = acc[0][c];
+    o2 = acc[1][c];
+    o3 = acc[2][c];
+  }
+  b.out[layer][((size_t)r * hq + g) * kD + c] = ((O[0] + o1) + (o2 + o3)) / L;
 }
 
 int decode_splits(int n, int hkv, int w, int layers) {
@@ -584,7 +612,10 @@ cudaError_t launch_decode(DType dt, const DecBatch& b, int layers, int n, int hq
   if (e != cudaSuccess) return e;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   TimingScope ts("decode_combine", st);
-  e = launch_after(k_decode_combine, dim3(hq, w * layers), kCmbThreads, 0, st, b, part_o, part_ml, nsplit, hq, w);
+  e = nsplit <= kCmbOneSlice
+          ? launch_after(k_decode_combine<1>, dim3(hq, w * layers), kD, 0, st, b, part_o, part_ml, nsplit, hq, w)
+          : launch_after(k_decode_combine<kCmbSeries>, dim3(hq, w * layers), kCmbSeries * kD, 0, st, b, part_o, part_ml,
+                         nsplit, hq, w);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -48,6 +48,29 @@ def test_decode_matches_oracle(st, w, hq, hkv, n, dtype):
     _close(out.cpu().numpy().astype(np.float64), ref, exact64(v))
 
 
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("n", [256, 257, 1025, 2048, 2049, 2304])  # 1, 2, 5, 8, 9 and 9 splits
+def test_decode_merges_any_number_of_splits(st, n, dtype):
+    """The merge takes up to eight splits in one slice of threads and more in
+    four.  Large values in the last split alone, so that a lost or doubled
+    split shows far above the tolerance."""
+    g = torch.Generator().manual_seed(n)
+    w, hq, hkv = 1, 4, 1
+    q = torch.randn((w, hq, 128), generator=g).to(dtype).cuda()
+    k = torch.randn((n, hkv, 128), generator=g).to(dtype).cuda()
+    v = torch.randn((n, hkv, 128), generator=g)
+    v[-1] *= n
+    v = v.to(dtype).cuda()
+    ws = torch.zeros(st.stlite_decode_workspace_size(st.make_shape(q, k)), dtype=torch.uint8, device="cuda")
+    out = torch.empty((w, hq, 128), dtype=torch.float32, device="cuda")
+    st.stlite_decode_attention(q, k, v, out, ws)
+    p = torch.softmax(torch.einsum("whd,nd->whn", q.double(), k[:, 0].double()) / 128 ** 0.5, -1)
+    ref = torch.einsum("whn,nd->whd", p, v[:, 0].double())
+    # fp32 scores, weights and sums: the bound is relative to the summed magnitudes
+    mag = torch.einsum("whn,nd->whd", p, v[:, 0].double().abs())
+    assert ((out.double() - ref).abs() <= 2e-5 * mag).all()
+
+
 def test_decode_workspace_reused(st):
     # one workspace serves many calls, eager and in a replayed graph, and
     # every call equals a call on a fresh workspace, bit for bit
