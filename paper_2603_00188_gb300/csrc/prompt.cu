@@ -578,14 +578,21 @@ __device__ __forceinline__ size_t prompt_bias_at(const PromptArgs& a, int h, int
   return ((size_t)h * a.n_ch + prel / a.p2) * a.crp + (size_t)(prel % a.p2) * a.G + (r - prel * a.G);
 }
 
-// Pass 1: a CTA per (64 query rows, KV head), longest rows first.
+// Pass 1: a cluster of CTAs per (64 query rows, KV head), longest rows first;
+// each takes every split-th tile of the keys, and their states are merged in
+// rank order.  With one CTA, few rows over a long cache were worked off by a CTA
+// or a few: one row of 28 heads over 50,000 keys took 4.05 ms, now 0.60.
+template <bool CLUSTER>
 __global__ void __launch_bounds__(kTileThreads, kTilesPerSm) k_prompt_rowstats_simt(const float* __restrict__ q,
                                                                                    const float* __restrict__ k,
                                                                                    PromptArgs a, float* bias) {
   extern __shared__ float4 tile_smem[];
   float* qs = reinterpret_cast<float*>(tile_smem);
   float* ks = qs + kTileFloats;
-  const int h = blockIdx.y, r0 = (int)(gridDim.x - 1 - blockIdx.x) * kTileRows, rows = a.nq * a.G;
+  cg::cluster_group cl = cg::this_cluster();
+  const int split = CLUSTER ? (int)cl.num_blocks() : 1, rank = CLUSTER ? (int)cl.block_rank() : 0;
+  const int rtile = ((int)gridDim.x - 1 - (int)blockIdx.x) / split;  // a cluster's CTAs follow one another
+  const int h = blockIdx.y, r0 = rtile * kTileRows, rows = a.nq * a.G;
   const int nr = min(kTileRows, rows - r0), p_first = a.n - a.nq, ty = tile_ty(), tx = tile_tx();
   const float c = kPrLog2e * rsqrtf((float)kD);
   tile_load(qs, nr, [&](int r) { return prompt_row(q, a, h, r0 + r); });
@@ -598,7 +605,7 @@ __global__ void __launch_bounds__(kTileThreads, kTilesPerSm) k_prompt_rowstats_s
     pos[i] = p_first + (r0 + min(ty + 8 * i, nr - 1)) / a.G;
   }
   const int kend = p_first + (r0 + nr - 1) / a.G + 1;  // keys that some row sees
-  for (int j0 = 0; j0 < kend; j0 += kTileRows) {
+  for (int j0 = rank * kTileRows; j0 < kend; j0 += split * kTileRows) {
     tile_load(ks, min(kTileRows, kend - j0), [&](int r) { return k + ((size_t)(j0 + r) * a.hkv + h) * kD; });
     tile_ready();
     float d[kTA][kTB];
@@ -612,12 +619,32 @@ __global__ void __launch_bounds__(kTileThreads, kTilesPerSm) k_prompt_rowstats_s
     __syncthreads();  // the key tile is rewritten
   }
   merge_rows(m, l, ks);
-  if (tx == 0)
+  float2* states = reinterpret_cast<float2*>(qs);  // (its copies ended in merge_rows, its reads before)
+  if (CLUSTER) {
+    if (rank > 0 && tx == 0)
+#pragma unroll
+      for (int i = 0; i < kTA; ++i) states[ty + 8 * i] = make_float2(m[i], l[i]);
+    cl.sync();
+  }
+  if (rank == 0 && tx == 0)
 #pragma unroll
     for (int i = 0; i < kTA; ++i) {
       const int r = ty + 8 * i;
+      if (CLUSTER) {  // every scaling is by a power of two (fold_scores), and the sum is rounded once
+        float mx = m[i];
+        for (int o = 1; o < split; ++o) mx = fmaxf(mx, cl.map_shared_rank(states, o)[r].x);
+        auto scaled = [&](float m2, float l2) { return l2 == 0.f || m2 == mx ? l2 : l2 * exp2f(m2 - mx); };
+        float2 total = make_float2(scaled(m[i], l[i]), 0.f);
+        for (int o = 1; o < split; ++o) {
+          const float2 s = cl.map_shared_rank(states, o)[r];
+          add_exact(total, scaled(s.x, s.y));
+        }
+        m[i] = mx;
+        l[i] = total.x + total.y;
+      }
       if (r < nr) bias[prompt_bias_at(a, h, r0 + r)] = -m[i] - log2f((float)a.G * l[i]);
     }
+  if (CLUSTER) cl.sync();  // no CTA leaves while rank 0 may still read its states
 }
 
 // Pass 2: a cluster of CTAs per (64 keys, KV head), each taking every split-th
@@ -770,34 +797,49 @@ cudaError_t launch_prompt_score(DType dt, const void* q, const void* k, int n, i
     const float* qf = static_cast<const float*>(q);
     const float* kf = static_cast<const float*>(k);
     const int rows = nq * a.G, ktiles = (n + kTileRows - 1) / kTileRows, rtiles = (rows + kTileRows - 1) / kTileRows;
-    if ((e = cudaFuncSetAttribute(k_prompt_rowstats_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, kPrSimtSmem)) !=
-            cudaSuccess ||
+    if ((e = cudaFuncSetAttribute(k_prompt_rowstats_simt<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  kPrSimtSmem)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(k_prompt_rowstats_simt<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  kPrSimtSmem)) != cudaSuccess ||
         (e = cudaFuncSetAttribute(k_prompt_colsum_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, kPrSimtSmem)) !=
             cudaSuccess)
       return e;
-    {
-      TimingScope ts("prompt_rowstats_simt", st);
-      k_prompt_rowstats_simt<<<dim3((unsigned)rtiles, hkv), kTileThreads, kPrSimtSmem, st>>>(qf, kf, a, bias);
-    }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // CTAs per key tile: while the CTAs fill the SMs less than four times (the
-    // first tiles see every row, the last ones few), at most one per row tile
-    int split = 1;
-    while (2 * split <= rtiles && 2 * split <= kP2MaxSplit &&
-           (long long)ktiles * hkv * 2 * split <= 4 * 152 * kTilesPerSm)
-      split *= 2;
+    // The largest cluster of 1, 2, 4 or 8 CTAs per tile, at most `others`, that
+    // keeps the grid within `limit` CTAs.  It fixes how the sums are grouped, so
+    // it depends on the shape alone.
+    auto clusters = [&](long long tiles, int others, int limit) {
+      int s = 1;
+      while (2 * s <= others && 2 * s <= kP2MaxSplit && tiles * hkv * 2 * s <= limit) s *= 2;
+      return s;
+    };
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
-    cfg.gridDim = dim3((unsigned)(ktiles * split), hkv);
     cfg.blockDim = dim3(kTileThreads);
     cfg.dynamicSmemBytes = kPrSimtSmem;
     cfg.stream = st;
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)split;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    auto grid = [&](int tiles, int split) {
+      cfg.gridDim = dim3((unsigned)(tiles * split), hkv);
+      attr[0].val.clusterDim.x = (unsigned)split;
+      cfg.numAttrs = split > 1 ? 1 : 0;
+    };
+    {
+      TimingScope ts("prompt_rowstats_simt", st);
+      // Clusters while they fill the SMs' places once, with three key tiles or
+      // more for each CTA: with one or two it spends what it spares on its copy
+      // of the query tile and on the merge (300 keys, 1,561 rows: 37 us, in
+      // clusters of two 40; 900 keys, one row: 86, in clusters of four 39).
+      const int split = clusters(rtiles, ktiles / 3, 152 * kTilesPerSm);
+      grid(rtiles, split);
+      e = cudaLaunchKernelEx(&cfg, split > 1 ? k_prompt_rowstats_simt<true> : k_prompt_rowstats_simt<false>, qf, kf, a,
+                             bias);
+    }
+    if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
     TimingScope ts("prompt_colsum_simt", st);
+    // until the CTAs fill the SMs four times (the first tiles see every row, the last ones few)
+    grid(ktiles, clusters(ktiles, rtiles, 4 * 152 * kTilesPerSm));
     e = cudaLaunchKernelEx(&cfg, k_prompt_colsum_simt, qf, kf, a, (const float*)bias, a_out);
     return e != cudaSuccess ? e : cudaGetLastError();
   }

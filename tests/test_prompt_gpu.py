@@ -181,3 +181,22 @@ def test_prompt_splits_and_pads(st, n, n_prompt, hq, hkv):
         for h in range(hkv):
             assert_within(a[h].cpu().numpy(), ora[h], a_bound(ora[h]), "head %d" % h)
         assert st.stlite_device_status(ws) == st.STLITE_OK
+
+
+@pytest.mark.parametrize("n,n_prompt,hq,hkv", [(64, 1, 7, 1), (320, 1, 7, 1), (321, 1, 7, 1), (3001, 1, 28, 4),
+                                               (600, 600, 7, 1), (2000, 40, 12, 2)])
+def test_prompt_fp32_key_splits(st, n, n_prompt, hq, hkv):
+    """fp32, one to eight CTAs per tile of query rows, each with its share of
+    the keys (some rows' keys all in the first CTA's).  Against fp64: a score of
+    128 fp32 products of values around one is within about 1e-6, and so is, relatively,
+    every probability; the sums add less."""
+    gen = torch.Generator().manual_seed(n + hq)
+    q = torch.randn((n_prompt, hq, 128), generator=gen).cuda()
+    k = torch.randn((n, hkv, 128), generator=gen).cuda()
+    a, ws = st.prompt_score(q, k, st.STLITE_PROMPT_FULL)
+    G = hq // hkv
+    x = torch.einsum("pgd,ngd->gpn", q.double(), k.double().repeat_interleave(G, 1)) / 128 ** 0.5
+    seen = torch.arange(n, device="cuda") <= torch.arange(n - n_prompt, n, device="cuda")[:, None]
+    ref = torch.softmax(x.masked_fill(~seen, -np.inf), -1).sum(1).view(hkv, G, n).mean(1)
+    assert ((a.double() - ref).abs() <= 1e-5 * ref).all()
+    assert st.stlite_device_status(ws) == st.STLITE_OK
