@@ -342,6 +342,11 @@ __global__ void __maxnreg__(kPrMaxReg)
   }
 }
 
+// CLUSTER: a cluster of CTAs per key tile; otherwise one, in code without any
+// cluster operations: compiled in, even where a CTA skips them all, they cost
+// 0.4 us of a one-chunk CTA's 5 (one row over 50,000 keys, 1,564 such CTAs: the
+// column sums 52.9 us, without them 48.8).
+template <bool CLUSTER>
 __global__ void __maxnreg__(kPrMaxReg)
     k_prompt_colsum(const __grid_constant__ PromptMaps maps, PromptArgs a, const float* bias, float* a_out,
                     uint32_t* err) {
@@ -351,7 +356,7 @@ __global__ void __maxnreg__(kPrMaxReg)
   // a cluster of `split` CTAs per key tile: rank r takes every split-th chunk
   // (keys seen by the most rows first)
   cg::cluster_group cl = cg::this_cluster();
-  const int split = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int split = CLUSTER ? (int)cl.num_blocks() : 1, rank = CLUSTER ? (int)cl.block_rank() : 0;
   const int unit = blockIdx.x / split, h = unit % a.hkv, kt = unit / a.hkv;
   const int j0 = kt * 128;
   const int p_first = a.n - a.nq;
@@ -543,21 +548,23 @@ __global__ void __maxnreg__(kPrMaxReg)
   // put the bases of 300-8,576 positions up to 30 % further from the fp64 result
   // than one CTA's sum of four groups had been; these put them 8-15 % nearer, at
   // 0.9 us of 441 (fp64 additions: the same error, 2.5 us).
-  if (split > 1) cl.sync();
+  if (CLUSTER) cl.sync();
   if (rank == 0 && threadIdx.x < 128 && j0 + (int)threadIdx.x < a.n) {
     const int j = j0 + threadIdx.x;
     float2 total = sum_s[threadIdx.x];
     bool whole = !*abort_flag;
-    for (int r = 1; r < split; ++r) {
-      const float2 other = cl.map_shared_rank(sum_s, r)[threadIdx.x];
-      add_exact(total, other);
-      whole = whole && !*cl.map_shared_rank(slot + 1, r);
+    if (CLUSTER) {
+      for (int r = 1; r < split; ++r) {
+        const float2 other = cl.map_shared_rank(sum_s, r)[threadIdx.x];
+        add_exact(total, other);
+        whole = whole && !*cl.map_shared_rank(slot + 1, r);
+      }
     }
     float acc = total.x + total.y;
     if (a.mode == 1) acc /= (float)min(a.nq, a.n - j);
     if (whole) a_out[(size_t)h * a.n + j] = acc;
   }
-  if (split > 1) cl.sync();  // no CTA leaves while rank 0 may still read its sums
+  if (CLUSTER) cl.sync();  // no CTA leaves while rank 0 may still read its sums
 }
 
 // ---- fp32 caches: the same two passes on the CUDA cores --------------------
@@ -852,8 +859,9 @@ cudaError_t launch_prompt_score(DType dt, const void* q, const void* k, int n, i
   if ((e = cudaFuncSetAttribute(k_prompt_rowstats, cudaFuncAttributeMaxDynamicSharedMemorySize, kP1Smem)) !=
       cudaSuccess)
     return e;
-  if ((e = cudaFuncSetAttribute(k_prompt_colsum, cudaFuncAttributeMaxDynamicSharedMemorySize, kP2Smem)) !=
-      cudaSuccess)
+  const int split = prompt_split(a);
+  auto cs_kernel = split > 1 ? k_prompt_colsum<true> : k_prompt_colsum<false>;
+  if ((e = cudaFuncSetAttribute(cs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kP2Smem)) != cudaSuccess)
     return e;
   int nsm = 0, dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -865,7 +873,6 @@ cudaError_t launch_prompt_score(DType dt, const void* q, const void* k, int n, i
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
-  const int split = prompt_split(a);
   cfg.gridDim = dim3((unsigned)((n + 127) / 128 * hkv * split));
   cfg.blockDim = dim3(kPrThreads);
   cfg.dynamicSmemBytes = kP2Smem;
@@ -874,9 +881,9 @@ cudaError_t launch_prompt_score(DType dt, const void* q, const void* k, int n, i
   attr[0].val.clusterDim.x = (unsigned)split;
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = split > 1 ? 1 : 0;
   TimingScope ts("prompt_colsum", st);
-  if ((e = cudaLaunchKernelEx(&cfg, k_prompt_colsum, maps, a, (const float*)bias, a_out, err)) != cudaSuccess) return e;
+  if ((e = cudaLaunchKernelEx(&cfg, cs_kernel, maps, a, (const float*)bias, a_out, err)) != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
