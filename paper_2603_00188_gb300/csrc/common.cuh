@@ -59,32 +59,6 @@ __device__ __forceinline__ int find_frame(const FrameTable& ft, int j) {
   return -1;
 }
 
-template <typename T>
-struct Elem;
-template <>
-struct Elem<float> {
-  // 4 consecutive elements starting at p (16-byte aligned)
-  static __device__ __forceinline__ float4 load4(const float* p) {
-    return __ldg(reinterpret_cast<const float4*>(p));
-  }
-  static __device__ __forceinline__ float load1(const float* p) { return __ldg(p); }
-};
-template <>
-struct Elem<__nv_bfloat16> {
-  static __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
-    uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
-    float4 r;
-    r.x = __uint_as_float(u.x << 16);
-    r.y = __uint_as_float(u.x & 0xffff0000u);
-    r.z = __uint_as_float(u.y << 16);
-    r.w = __uint_as_float(u.y & 0xffff0000u);
-    return r;
-  }
-  static __device__ __forceinline__ float load1(const __nv_bfloat16* p) {
-    return __bfloat162float(p[0]);
-  }
-};
-
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -128,10 +102,6 @@ __device__ __forceinline__ float row_bias4(const float2* pp, int R, int nsplit, 
     fold_partial(m, l, m2, l2);
   }
   return -m - log2f(G * l);
-}
-
-__device__ __forceinline__ float dot4(float4 a, float4 b) {
-  return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, a.w * b.w)));
 }
 
 // Order-preserving map float -> uint32 (ascending keys = ascending floats).

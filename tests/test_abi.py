@@ -95,6 +95,25 @@ def test_workspace_size_and_validation(st):
         assert e.value.status == code
 
 
+class _At:
+    def __init__(self, address):
+        self.address = address
+
+    def data_ptr(self):
+        return self.address
+
+
+def test_layer_tables_have_the_structs_layout(st):
+    """The binding passes layer tables as plain arrays of addresses."""
+    for fields, struct, table in ((6, st.LayerIO, st._layer_table), (4, st.DecodeIO, st._decode_table)):
+        rows = [[(1 << 40) + 4096 * (fields * l + f) for f in range(fields)] for l in range(3)]
+        got = table([tuple(_At(a) for a in row) for row in rows])
+        assert got.tobytes() == bytes((struct * 3)(*[struct(*row) for row in rows]))
+        for wrong in (fields - 1, fields + 1):
+            with pytest.raises(ValueError):
+                table([tuple(_At(64) for _ in range(wrong))])
+
+
 @pytest.mark.parametrize("n,hkv", [(4096, 4), (53600, 4), (11841, 2)])
 def test_workspace_holds_what_a_layer_uses(st, n, hkv):
     """Per token and KV head: the inverse norm, A, Phi, rho, TSG's maximum and
