@@ -382,8 +382,8 @@ KERNEL_UNITS = {
     "css_umma": ("umma.cu",),
     "css_phi": ("umma.cu",),
     "row_bias": ("simt.cu", "umma.cu"),
-    "select_gate_topk": ("select.cu",),
-    "gather": ("select.cu",),
+    "select_gate_topk": ("select.cu", "fit_cache.h"),
+    "gather": ("select.cu", "fit_cache.h"),
 }
 SHARED_UNITS = ("api.cu", "common.cuh", "kernels.cuh", "ptx.cuh")
 

@@ -1,6 +1,6 @@
 // Selection kernel.  One cluster of CL CTAs per (layer, KV head); CTA c of a
 // cluster owns the contiguous token range [c*chunk, (c+1)*chunk) and keeps
-// its radix keys in shared memory for every pass.
+// its keys in shared memory for every pass.
 //   kSelGate: rho_i = |k_i|^-1 * TSG's row maximum (Eq. 6), tau =
 //             the min(B, |pool|)-th smallest rho (Eq. 7), gate = rho <= tau
 //             (Eq. 8).
@@ -22,7 +22,7 @@ namespace cg = cooperative_groups;
 
 namespace stl {
 
-constexpr int kSelThreads = 512;  // two per histogram bin in the radix passes
+constexpr int kSelThreads = 512;  // two bins of a histogram pass each
 constexpr int kSelMaxCluster = 8;
 constexpr int kSelMaxChunk = 49152;  // keys per CTA held in shared memory (192 KB)
 

@@ -21,7 +21,7 @@ namespace stl {
 // against one dot product per thread with both operands read from shared
 // memory for every multiply-add: TSG 2,036 -> 483 us (45 TFLOP/s), row
 // statistics 389 -> 94, column sums 466 -> 92; 1,152 keys: 201 -> 15, 90 -> 18
-// and 195 -> 29.
+// and 195 -> 29 (17 with a cluster per key tile, simt.cu).
 constexpr int kTileRows = 64;
 constexpr int kTileThreads = 128;
 constexpr int kTilePitch = kD + 4;  // floats

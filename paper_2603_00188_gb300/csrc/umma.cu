@@ -75,8 +75,8 @@ __device__ __forceinline__ void tsg_tile_next(const FrameTable& ft, int t, int& 
 }
 
 // =========================================================================
-// TSG.  CTA (x, chunk, h): current-frame columns [512*chunk, 512*chunk+512)
-// of head h stay in shared memory (128 KB); historical row tiles of 128
+// TSG.  CTA (b, layer*Hkv + h): current-frame columns [512*chunk, 512*chunk+512)
+// of head h, chunk and first row tile from b (TsgSplit), stay in shared memory (128 KB); historical row tiles of 128
 // tokens stream through three 32 KB stages.  TMEM holds the 128 x 512 fp32
 // product as two 256-column accumulator stages; two epilogue groups each drain
 // 128 columns of a stage, release it when their columns are in registers and

@@ -1,13 +1,13 @@
 """The exact Top-B of the selection kernel on score distributions aimed at
-each branch of its radix select, through stlite_select_topk.
+each way its select ends, through stlite_select_topk.
 
 With no frames, TSG and CSS off, every token is text and S = A_base (Eq. 9
 with alpha = 0), so the kept set must equal the Top-B of the given scores by
 (S descending, index ascending), index for index.  The distributions are
 chosen so that the select ends in each of its ways: a bin that holds exactly
-the keys still needed after two or three 8-bit passes (the early stop),
-bins whose keys tie at the threshold (all four passes and the tie count),
-scores one unit in the last place apart, every score equal, and signed
+the keys still needed (the early stop), bins whose keys tie at the threshold
+(resolved to single values, and the tie count), scores one unit in the last
+place apart, every score equal, and signed
 zeros next to negative and positive scores (-0.0 and +0.0 compare equal).
 Sizes cover one CTA per problem, clusters, a ragged N and budgets of one,
 about a third of N and all of N.
@@ -47,8 +47,8 @@ def scores(kind, h, n, seed):
         elif kind == "ulps":
             x = _ulps(0.3 + 0.01 * i, n, rng)
         elif kind == "few_ulps_with_ties":
-            # values within 16 ulps of each other: every key shares its top
-            # 24 bits, so the last pass decides among large tie groups
+            # values within 16 ulps of each other: a range of 16 keys, a bin
+            # each, decided among large tie groups
             b = np.array([0.7], dtype=np.float32).view(np.uint32)[0]
             x = (b + rng.integers(0, 16, n).astype(np.uint32)).view(np.float32)
         elif kind == "four_values":
