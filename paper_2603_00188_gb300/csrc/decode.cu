@@ -500,8 +500,7 @@ __global__ void __launch_bounds__(SLICES* kD) k_decode_combine(const __grid_cons
   float O[kOwn];
 #pragma unroll
   for (int i = 0; i < kOwn; ++i) O[i] = 0.f;
-  for (int s0 = 0; s0 < nsplit; s0 += kCmbSeries * kAtOnce) {
-    if (s0 > 0) load(s0);
+  auto add = [&](int s0) {
 #pragma unroll
     for (int i = 0; i < kOwn; ++i)
 #pragma unroll
@@ -509,6 +508,11 @@ __global__ void __launch_bounds__(SLICES* kD) k_decode_combine(const __grid_cons
         const int s = s0 + k + SLICES * i + kCmbSeries * u;
         if (s < nsplit) O[i] = fmaf(x[i][u], wts[s], O[i]);
       }
+  };
+  add(0);
+  for (int s0 = kCmbSeries * kAtOnce; s0 < nsplit; s0 += kCmbSeries * kAtOnce) {
+    load(s0);
+    add(s0);
   }
   float o1, o2, o3;  // the other series of the thread's dimension
   if constexpr (SLICES == 1) {
