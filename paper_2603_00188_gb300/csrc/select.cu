@@ -199,18 +199,27 @@ __device__ __noinline__ Selected cluster_select(int ncta, const uint32_t* keys, 
       hist[tid] = 0u;
       __syncthreads();
     }
-    auto count = [&](uint32_t key) {
-      const uint32_t b = (key - lo) >> shift;
-      if (key - lo <= span) atomicAdd(&hist[b >> 1], b & 1u ? 0x10000u : 1u);
+    auto count = [&](uint32_t r, uint32_t n) {  // n keys of r's bin, r = key - lo
+      const uint32_t b = r >> shift;
+      if (r <= span) atomicAdd(&hist[b >> 1], b & 1u ? n << 16 : n);
     };
+    // Four neighbouring keys of one bin are added at once: where most keys
+    // crowd into a bin, their additions wait for one another (one layer with
+    // near-duplicate frames, 4 x 53,600 tokens: 36 -> 35 us; 112 x 53,600 scores,
+    // most within 0.1 % of one another and a few far off: 69 -> 58).
     for (int i = tid; i < len >> 2; i += kSelThreads) {
       const uint4 x = reinterpret_cast<const uint4*>(keys)[i];
-      count(x.x);
-      count(x.y);
-      count(x.z);
-      count(x.w);
+      const uint32_t r0 = x.x - lo, r1 = x.y - lo, r2 = x.z - lo, r3 = x.w - lo;
+      if (max(max(r0, r1), max(r2, r3)) <= span && ((r0 ^ r1) | (r0 ^ r2) | (r0 ^ r3)) >> shift == 0u) {
+        count(r0, 4u);
+      } else {
+        count(r0, 1u);
+        count(r1, 1u);
+        count(r2, 1u);
+        count(r3, 1u);
+      }
     }
-    if (tid < (len & 3)) count(keys[(len & ~3) + tid]);
+    if (tid < (len & 3)) count(keys[(len & ~3) + tid] - lo, 1u);
     cluster_barrier(cl, ncta);
     uint32_t c0 = 0, c1 = 0, b0 = 0, b1 = 0;  // counts of the thread's bins; of the CTAs before this one
     for (int r0 = 0; r0 < ncta; r0 += 8) {    // eight remote reads in flight
@@ -753,9 +762,14 @@ cudaError_t launch_select(const Problem& p, const FrameTable& ft, const SelectAr
   // token of a CTA or, where CTAs share SMs, 1.2 ns per token of an SM.  The
   // least sum over the waves wins, the smallest cluster among equals: 28 x 4
   // heads of 53,600 tokens take clusters of 5, which are all resident at once
-  // (74 us; 8 need two waves, 108), 28 x 4 of 2,144 single CTAs (17 us; 2: 21,
-  // 4: 27), 28 x 2 of 20,000 clusters of 4 (29; 3: 32, 8: 39), 4 of 23,680
-  // clusters of 8 (24; 16: 29, 4: 30), 4 of 132,800 clusters of 16 (44; 8: 56).
+  // (74 us; 8 need two waves, 98), 28 x 4 of 2,144 single CTAs (20 us; 4: 27),
+  // 28 x 2 of 20,000 clusters of 4 (29; 3: 32, 8: 43), 4 of 23,680 clusters of 8
+  // (26; 16: 31, 4: 29), 4 of 132,800 clusters of 16 (47; 8: 51).
+  // Clusters of 16 only where those of 8 have more than 7,500 tokens a CTA (4
+  // heads of 53,600: 35 us, in 16 37; of 90,000: 42 and 39), or more than
+  // 28,000 if 16 CTAs would have to share SMs, which they do from the eighth
+  // cluster on (8 heads of 53,600: 35 us, in 16 43; of 132,800: 51 and 55; of
+  // 260,000: 78 and 76).
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
   int cl = 0;
@@ -774,6 +788,12 @@ cudaError_t launch_select(const Problem& p, const FrameTable& ft, const SelectAr
       break;
     }
     if (fit < 1) continue;
+    if (c > kSelMaxCluster && cl != 0) {
+      int alone = 0;  // clusters whose CTAs have an SM each
+      const int own = largest_dynamic(sm_smem, cta_smem, 1, 4 * kSelMaxChunk);
+      if ((e = clusters_fit(dev, ctx, c, 1, own, cfg, &alone)) != cudaSuccess) break;
+      if (select_chunk(p.n, kSelMaxCluster) <= (units <= alone ? 7500 : 28000)) break;
+    }
     const double fixed = c == 1 ? 13.0 : 16.5 + 0.55 * c;
     double cost = 0.0;
     for (long long left = units; left > 0; left -= fit) {
